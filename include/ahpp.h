@@ -92,8 +92,9 @@ typedef struct {
     uint32_t batch_groups;     /* tiles processed concurrently, 1..8; 0: 1 (ahpp_autotune picks 1, 2 or 4) */
     uint32_t batch_chunk;      /* entries per chunk of a long row in the batched kernel: 128, 256 or
                                   512; 0: 256 (ahpp_autotune picks one) */
-    uint32_t single_vec_width; /* single-query kernel: at most this many lanes walk one short row
-                                  (1, 2, 4, 8, 16 or 32); 0: 2 (ahpp_autotune picks one) */
+    uint32_t single_vec_width; /* single-query kernel: at least this many lanes walk one row
+                                  (1, 2, 4, 8, 16 or 32); 0: 1, 2, 8 or 32 by the graph's size
+                                  (ahpp_autotune picks one of those) */
 } ahpp_config;
 
 /* Per-query statistics. */
@@ -126,10 +127,10 @@ typedef struct {
     uint32_t batch_chunk;                /* batched: entries per chunk of a long row */
     /* single-query kernel (the plain path): pull rounds once the frontier's
      * degree sum exceeds 1/single_dense_div of |E| + |E_A|; the attribute hop
-     * of pull rounds pushed from phase 2 through shared memory (1) or pulled
-     * over A->U (0); rows of up to 64 entries walked by at most
-     * single_vec_width lanes each (1 = one row per lane); single_smem_bytes
-     * of shared memory per block. */
+     * U->A of pull rounds added up in shared memory (single_attr_push, always
+     * 1); the shortest rows walked by single_vec_width lanes each (1 = one row
+     * per lane), longer ones by more; single_smem_bytes of shared memory per
+     * block. */
     uint32_t single_dense_div, single_attr_push, single_vec_width, single_smem_bytes;
 } ahpp_graph_info;
 
@@ -265,8 +266,9 @@ int ahpp_query_device(ahpp_graph *g, uint32_t q, double eps, uint32_t k,
  * replicated to fill four tiles of 32: queries per tile (32, 16), entries per
  * chunk of a long row (128, 256, 512), then tiles processed concurrently
  * (1, 2, 4).  Single-query kernel, on
- * up to four sample queries: lanes per short row (32, 8, 2, 1: at most that
- * many lanes walk one row), then the frontier fraction 1/dense_div (8, 16,
+ * up to four sample queries: lanes per short row (32, 8, 2, 1: at least that
+ * many lanes walk one row; the kernel's layout of the graph is built anew for
+ * each), then the frontier fraction 1/dense_div (8, 16,
  * 32, 64, 128) past which rounds run as pull sweeps.  Every candidate gives the same results
  * within FP32 rounding (only the order of sums changes).  The choice is
  * stored in the graph and reported by ahpp_get_graph_info; the measured

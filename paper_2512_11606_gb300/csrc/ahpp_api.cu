@@ -90,6 +90,15 @@ double eps_f_of(const ahpp_graph* g, double eps) {
   return g->cfg.algo == AHPP_ASRP ? eps / g->lambda : eps / (double)(g->n_e + g->n_ea);
 }
 
+// The FP32 forms of a query's tests, from its FP64 parameters.
+void set_tests(Q1Params& p) {
+  p.th_async = threshold_up(p.eps_f);
+  p.th_sync = threshold_up(0.0);
+  p.eps_f32 = (float)p.eps_f;
+  p.switch_unit = (float)(2.0 * (double)p.e_tot / p.log_inv);
+  p.switch_log = (float)(p.switch_rule == 1 ? -std::log(p.lambda) : std::log(p.eps_f));
+}
+
 Q1Params q1_params(const ahpp_graph* g, uint32_t q_new, double eps) {
   Q1Params p;
   p.q = q_new;
@@ -100,14 +109,11 @@ Q1Params q1_params(const ahpp_graph* g, uint32_t q_new, double eps) {
   p.lambda = g->lambda;
   p.log_inv = std::log(1.0 / (1.0 - g->cfg.alpha));
   p.e_tot = (uint32_t)(g->n_e + g->n_ea);
+  set_tests(p);
   p.max_rounds = g->cfg.max_rounds ? g->cfg.max_rounds : auto_rounds(p.eps_f, g->cfg.alpha);
   p.dense_div = g->q1_dense_div;
   p.n_split = g->n_split1;
-  p.trace_cap = 4096;
   p.smem_bytes = g->q1_smem;
-  p.attr_push = g->q1_attr_push;
-  p.ta_smem = g->q1_ta_smem;
-  p.vw_max = g->q1_vw_max;
   return p;
 }
 
@@ -134,8 +140,8 @@ Q1Params noalloc_params(const ahpp_graph* g, uint32_t q_new, double eps) {
 int reset_barrier(ahpp_graph* g, GridBarrier* bar, cudaStream_t stream, bool keep_trap) {
   AHPP_CUDA(cudaMemsetAsync(bar, 0, sizeof(GridBarrier), stream));
   if (g && g->wait_trap.load()) {
-    // 0x40404040 arrivals: the block count is never reached
-    AHPP_CUDA(cudaMemsetAsync(&bar->count, 0x40, sizeof(bar->count), stream));
+    // 0xc0c0c0c0 arrivals, a billion below the first barrier's block count
+    AHPP_CUDA(cudaMemsetAsync(&bar->count, 0xc0, sizeof(bar->count), stream));
     if (!keep_trap) g->wait_trap.store(0);
   }
   return AHPP_OK;
@@ -167,9 +173,9 @@ int run_lambda(ahpp_graph* g) {
   p.lambda_mode = 1;
   p.algo = kAlgoASRP;
   p.eps_f = 0.0;
+  set_tests(p);
   p.kahan = 1;
   p.max_rounds = T;
-  p.trace_cap = 0;
   if (int rc = reset_barrier(nullptr, g->q1.bar, g->stream)) return rc;
   int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, g->stream);
   if (e) return cuda_fail((cudaError_t)e, "lambda launch");
@@ -425,7 +431,6 @@ int ahpp_load_graph(const ahpp_graph_desc* desc, const ahpp_config* cfg, ahpp_gr
   g->device = c.device;
   g->batch_tile = c.batch_tile ? c.batch_tile : (uint32_t)ahpp::kTile;
   g->batch_groups = c.batch_groups ? c.batch_groups : 1;
-  g->q1_vw_max = c.single_vec_width ? c.single_vec_width : ahpp::kQ1VecWidthDefault;
   int rc = AHPP_OK;
   if (cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
       cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess) {
@@ -451,6 +456,7 @@ void ahpp_free_graph(ahpp_graph* g) {
   if (!g) return;
   cudaSetDevice(g->device);
   if (g->stream) cudaStreamSynchronize(g->stream);
+  for (void* p : g->q1_layout_bufs) cudaFree(p);
   g->release_all();
   if (g->stream) cudaStreamDestroy(g->stream);
   io_drop(g);
@@ -472,7 +478,7 @@ int ahpp_get_graph_info(const ahpp_graph* g, ahpp_graph_info* info) {
   info->batch_groups = g->batch_groups;
   info->batch_chunk = kChunkSizes[g->dg.b_chunk];
   info->single_dense_div = g->q1_dense_div;
-  info->single_attr_push = (uint32_t)g->q1_attr_push;
+  info->single_attr_push = 1;
   info->single_vec_width = g->q1_vw_max;
   info->single_smem_bytes = g->q1_smem;
   return AHPP_OK;
@@ -536,8 +542,8 @@ int ahpp_power_iteration(ahpp_graph* g, uint32_t q, uint32_t T, float* out_pi, a
   p.pi_mode = 1;
   p.algo = kAlgoASRP;
   p.eps_f = 0.0;
+  set_tests(p);
   p.max_rounds = T;
-  p.trace_cap = 0;
   if (int rc = reset_barrier(g, g->q1.bar, g->stream)) return rc;
   int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, g->stream);
   if (e) return cuda_fail((cudaError_t)e, "power iteration launch");
@@ -808,22 +814,21 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     float best = -1.f;
     uint32_t best_v = values[0];
     for (uint32_t v : values) {
-      set(v);
+      if (int r = set(v)) return r;
       float t = 0.f;
       if (int r = time_single(g, q1, eps, &t)) return r;
       note(knob, v, t / (float)q1.size());
       if (best < 0.f || t < best) { best = t; best_v = v; }
     }
-    set(best_v);
-    return AHPP_OK;
+    return set(best_v);
   };
   const uint32_t saved_div = g->q1_dense_div, saved_vw = g->q1_vw_max;
-  rc = tune_single("single_vec_width", [&](uint32_t v) { g->q1_vw_max = v; }, {32u, 8u, 2u, 1u});
+  rc = tune_single("single_vec_width", [&](uint32_t v) { return build_q1_layout(g, v); }, {32u, 8u, 2u, 1u});
   if (rc == AHPP_OK)
-    rc = tune_single("single_dense_div", [&](uint32_t v) { g->q1_dense_div = v; }, {32u, 8u, 16u, 64u, 128u});
+    rc = tune_single("single_dense_div", [&](uint32_t v) { g->q1_dense_div = v; return AHPP_OK; }, {32u, 8u, 16u, 64u, 128u});
   if (rc != AHPP_OK) {
     g->q1_dense_div = saved_div;
-    g->q1_vw_max = saved_vw;
+    build_q1_layout(g, saved_vw);
     return rc;
   }
   g->tune_log = log + "}";

@@ -80,14 +80,6 @@ constexpr int kGL = kTile / kQL;       // lanes per row group (one 128- or 64-by
 constexpr int kGPW = 32 / kGL;         // row groups per warp
 static_assert(kTile == 16 || kTile == 32, "tile of 16 or 32 queries");
 
-// Smallest float f with (r > th) <=> (r >= f) for every float r: the mark
-// test r > th of Algorithm 4 taken exactly against the FP64 threshold.
-__device__ __forceinline__ float threshold_up(double th) {
-  float f = (float)th;
-  if ((double)f <= th) f = nextafterf(f, INFINITY);
-  return f;
-}
-
 // Graph arrays, reserves and compensations are read once per round:
 // streamed with the evict-first policy so that they do not push the
 // gathered state rows out of L2.
@@ -559,6 +551,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
   const uint32_t n_split = g.b_v.n_split + g.b_a.n_split + g.b_u.n_split;
   const size_t nu32 = (size_t)g.n_u * kTile;
   const uint32_t kmax = p.kmax;
+  unsigned int epoch = 0;                               // of the group's barrier
 
   for (uint32_t w = grp; w < n_work; w += groups) {
     const uint32_t tile = SERVE ? sv.live[w] : w;
@@ -624,7 +617,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         for (int r = 0; r < 5; ++r) tb.racc[r * kTile + lane] = RAcc{};
       }
     }
-    if (!grid_sync(tb.bar, nbg)) return;
+    if (!grid_sync(tb.bar, nbg, epoch)) return;
     if (bid == 0 && warp0 && lq && s_new[lane]) {
       const uint32_t q_new = SERVE ? sv.slots[qi].q_new : p.u_old2new[p.q[qi]];
       const uint32_t cnt = (g.uv_off[q_new + 1] - g.uv_off[q_new]) + (g.ua_off[q_new + 1] - g.ua_off[q_new]);
@@ -643,7 +636,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         tb.r_u[(size_t)q_new * kTile + lane] = 1.f;
       }
     }
-    if (!grid_sync(tb.bar, nbg)) return;
+    if (!grid_sync(tb.bar, nbg, epoch)) return;
 
     // ---- rounds (Algorithm 3 / 4) for the active lanes
     Partials part;
@@ -673,11 +666,11 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
       float* ta_cur = (tround & 1) ? tb.t_a2 : tb.t_a;     // t_A of this round
       float* ta_next = (tround & 1) ? tb.t_a : tb.t_a2;    // t_A of the next round
       gphase1<WA>(c, A, true, false, nullptr, ta_cur, ta_next, true);
-      if (!grid_sync(tb.bar, nbg)) { wait_fail = true; break; }
+      if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
       if (p.algo == kAlgoASRP) gphase2<WA, false, false>(c, s_ctl, A, ta_cur, ta_next);
       else if (p.algo == kAlgoAPP) gphase2<WA, true, false>(c, s_ctl, A, ta_cur, ta_next);
       else gphase2<WA, true, true>(c, s_ctl, A, ta_cur, ta_next);
-      if (!grid_sync(tb.bar, nbg)) { wait_fail = true; break; }
+      if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
       ++tround;
 
       if (warp0) {
@@ -733,11 +726,11 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
           }
         }
         flush_lane_partials(part, A);
-        if (!grid_sync(tb.bar, nbg)) { wait_fail = true; break; }
+        if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
         // the new marks also push into the next round's t_A: recompute it by
         // the pull form from the complete marks (once per switch)
         gphase1<WA>(c, A, false, true, (tround & 1) ? tb.t_a2 : tb.t_a, nullptr, nullptr, false);
-        if (!grid_sync(tb.bar, nbg)) { wait_fail = true; break; }
+        if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
       }
     }
     if (wait_fail && warp0 && lq && s_ctl[lane].valid) {
@@ -770,7 +763,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         for (size_t i = c.gt; i < (size_t)kRadixPasses * kTile * kRadixBins; i += c.nt) tb.hist[i] = 0;
         if (c.gt < kTile) tb.cand_cnt[c.gt] = 0;
       }
-      if (!grid_sync(tb.bar, nbg)) return;
+      if (!grid_sync(tb.bar, nbg, epoch)) return;
 
       if (bid == 0 && fin) {
         const LaneCtl L = s_ctl[lane];
@@ -820,7 +813,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
           unsigned int* gh = tb.hist + (size_t)pass * kTile * kRadixBins;
           for (int i = threadIdx.x; i < kTile * kRadixBins; i += kBThreads)
             if (sh[i]) atomicAdd(&gh[i], sh[i]);
-          if (!grid_sync(tb.bar, nbg)) return;
+          if (!grid_sync(tb.bar, nbg, epoch)) return;
           // the merged histograms into shared memory; warp w picks the digit
           // of queries w, w + 8, ... (warp-parallel), lane l reads query l's
           for (int i = threadIdx.x; i < kTile * kRadixBins; i += kBThreads) sh[i] = __ldcg(&gh[i]);
@@ -855,7 +848,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
             }
           }
         }
-        if (!grid_sync(tb.bar, nbg)) return;
+        if (!grid_sync(tb.bar, nbg, epoch)) return;
         // sort each lane's keys descending (bitonic in shared memory), one block per lane
         unsigned long long* sk = reinterpret_cast<unsigned long long*>(smem);
         for (uint32_t l = bid; l < kTile; l += nbg) {
@@ -912,7 +905,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
       }
       if (lane == 0) sv.tile_round[tile] = tround;
     }
-    if (!grid_sync(tb.bar, nbg)) return;
+    if (!grid_sync(tb.bar, nbg, epoch)) return;
   }
 }
 

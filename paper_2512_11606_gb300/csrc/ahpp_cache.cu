@@ -28,7 +28,7 @@ namespace ahpp {
 namespace {
 
 constexpr char kMagic[8] = {'A', 'H', 'P', 'P', 'G', 'R', 'F', '1'};
-constexpr uint32_t kVersion = 5;
+constexpr uint32_t kVersion = 6;
 
 struct CacheHeader {
   char magic[8];
@@ -50,7 +50,7 @@ void visit_graph_ptrs(ahpp_graph* g, F f) {
   f((const void**)&G.au_off); f((const void**)&G.au_idx); f((const void**)&G.au_w); f((const void**)&G.au_c);
   f((const void**)&G.ua_pc);
   f((const void**)&G.rnorm_u); f((const void**)&G.cnorm_a);
-  ItemList* lists[] = {&G.s1_v, &G.s1_a, &G.s1_u, &G.b_v, &G.b_a, &G.b_u};
+  ItemList* lists[] = {&G.s1_v, &G.s1_a, &G.b_v, &G.b_a, &G.b_u};
   for (ItemList* L : lists) {
     f((const void**)&L->items);
     f((const void**)&L->split_nchunks);
@@ -208,7 +208,6 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
   g->device = c.device;
   g->batch_tile = c.batch_tile ? c.batch_tile : (uint32_t)kTile;
   g->batch_groups = c.batch_groups ? c.batch_groups : 1;
-  g->q1_vw_max = c.single_vec_width ? c.single_vec_width : ahpp::kQ1VecWidthDefault;
   g->n_u = h.n_u; g->n_v = h.n_v; g->n_a = h.n_a; g->n_e = h.n_e; g->n_ea = h.n_ea;
   g->bf16 = h.attr_bf16 != 0;
   int rc = AHPP_OK;

@@ -338,7 +338,7 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
   for (uint32_t v = 0; v < nV; ++v) dg_v[v] = vu_off[v + 1] - vu_off[v];
   for (uint32_t a = 0; a < nA; ++a) dg_a[a] = au_off[a + 1] - au_off[a];
   const ItemShape s1{64, 32, 0xffffffffu, 2048};
-  HostItems i1v = build_items(dg_v, s1), i1a = build_items(dg_a, s1), i1u = build_items(dg_u, s1);
+  HostItems i1v = build_items(dg_v, s1), i1a = build_items(dg_a, s1);
   std::vector<HostItems> ib;
   for (int c = 0; c < kChunkChoices; ++c) {
     ib.push_back(build_units(dg_v, kChunkSizes[c]));
@@ -391,7 +391,7 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
     L.split_nchunks = (const uint32_t*)up(h.split_nchunks.data(), h.split_nchunks.size() * 4);
     L.n_long = h.n_long;
   };
-  up_items(i1v, G.s1_v); up_items(i1a, G.s1_a); up_items(i1u, G.s1_u);
+  up_items(i1v, G.s1_v); up_items(i1a, G.s1_a);
   G.b_split_max = 0;
   for (int c = 0; c < kChunkChoices; ++c) {
     for (int d = 0; d < 3; ++d) up_items(ib[3 * c + d], G.b_alt[c][d]);
@@ -414,26 +414,17 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
   return alloc_query_state(g);
 }
 
-// Shared-memory plan of the single-query kernel's pull rounds: phase 2
-// holds t_A and, with the attribute push, its accumulator over A when both
-// fit in kQ1AttrSmem.  Shared memory not planned here stays L1.
-void plan_query1_smem(ahpp_graph* g) {
-  constexpr uint64_t kQ1AttrSmem = 96 * 1024;
-  const DevGraph& G = g->dg;
-  const uint32_t smax = query1_max_smem(g->device);
-  const uint64_t na4 = 4ull * G.n_a;
-  g->q1_attr_push = 2 * na4 <= std::min<uint64_t>(kQ1AttrSmem, smax);
-  g->q1_ta_smem = g->q1_attr_push;
-  g->q1_smem = g->q1_attr_push ? (uint32_t)((2 * na4 + 15) / 16 * 16) : 0u;
-}
-
 // Single-query state of a loaded graph (working vectors, lists, accumulators,
 // barrier, trace) and the launch grid of the single-query kernel.
 int alloc_query_state(ahpp_graph* g) {
   const ahpp_config& cfg = g->cfg;
   const DevGraph& G = g->dg;
   const uint32_t nU = G.n_u, nV = G.n_v, nA = G.n_a;
-  g->n_split1 = G.s1_v.n_split + G.s1_a.n_split + G.s1_u.n_split;
+  const int max_blocks = query1_max_grid(g->sm_count, kQ1SmemMax);
+  if (max_blocks <= 0) { set_error("ahpp_load_graph: occupancy query failed"); return AHPP_ECUDA; }
+  g->q1_max_blocks = (uint32_t)max_blocks;
+  if (int rc = build_q1_layout(g, cfg.single_vec_width)) return rc;
+  g->n_split1 = 2 * G.q1.v.n_split + G.q1.u.n_split;
   const size_t before = g->bufs.size();
   Q1State& s = g->q1;
   s.r_u = (float*)g->alloc(4ull * nU);
@@ -449,9 +440,6 @@ int alloc_query_state(ahpp_graph* g) {
   s.racc = (RAcc*)g->alloc(3 * sizeof(RAcc));
   s.bar = (GridBarrier*)g->alloc(sizeof(GridBarrier));
   s.final_maxr_bits = (unsigned int*)g->alloc(2 * sizeof(unsigned int));
-  const uint32_t trace_cap = 4096;
-  s.trace_frontier = (uint32_t*)g->alloc(4ull * trace_cap);
-  s.trace_maxr = (float*)g->alloc(4ull * trace_cap);
   g->q1_bytes = 0;
   for (size_t i = before; i < g->bufs.size(); ++i) {
     if (!g->bufs[i].p) { set_error("ahpp_load_graph: device allocation failed"); return AHPP_ENOMEM; }
@@ -460,9 +448,6 @@ int alloc_query_state(ahpp_graph* g) {
   AHPP_CUDA(cudaMemset(s.bar, 0, sizeof(GridBarrier)));
   AHPP_CUDA(cudaMemset(s.split_acc, 0, 4ull * std::max(g->n_split1, 1u)));
   AHPP_CUDA(cudaMemset(s.split_cnt, 0, 4ull * std::max(g->n_split1, 1u)));
-  plan_query1_smem(g);
-  g->q1_grid = query1_max_grid(g->bf16, g->sm_count, g->q1_smem);
-  if (g->q1_grid <= 0) { set_error("ahpp_load_graph: occupancy query failed"); return AHPP_ECUDA; }
   BatchParams plan;
   if (int rc = batch_plan(g, plan)) return rc;
   if (cfg.hbm_budget_bytes && g->graph_bytes + g->q1_bytes > cfg.hbm_budget_bytes) {

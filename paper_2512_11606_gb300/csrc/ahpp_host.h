@@ -94,11 +94,12 @@ struct ahpp_graph {
   // single-query state
   ahpp::Q1State q1{};
   int q1_grid = 0;
-  // single-query kernel's shared-memory plan (see Q1Params)
-  uint32_t q1_smem = 0;
-  int q1_attr_push = 0, q1_ta_smem = 0;
+  // single-query pull layout (dg.q1): its buffers, the most blocks the device
+  // keeps resident, shared memory per block, lanes of the shortest rows
+  std::vector<void*> q1_layout_bufs;
+  uint64_t q1_layout_bytes = 0;
+  uint32_t q1_max_blocks = 0, q1_smem = 0, q1_vw_max = 0;
   uint32_t q1_dense_div = 32;     // pull rounds once the frontier covers > 1/dense_div of the edges
-  uint32_t q1_vw_max = ahpp::kQ1VecWidthDefault;   // lanes per short row in the pull phases (at most)
   std::string tune_log;           // the last autotune's measurements (JSON object)
   uint32_t n_split1 = 0;
   uint64_t q1_bytes = 0;
@@ -134,9 +135,9 @@ int barrier_status(GridBarrier* bar, cudaStream_t stream, int* status);
 int build_graph(const ahpp_graph_desc* desc, ahpp_graph* g);
 // The kernels' algorithm id of an AHPP_* constant (-1 if none).
 int kernel_algo(int algo);
-// Shared-memory plan of the single-query kernel (the grid does not depend on
-// it: one block per SM).
-void plan_query1_smem(ahpp_graph* g);
+// Sliced layout of the single-query pull rounds with at least vec_width lanes
+// per row (0: by the graph's size); replaces the one the graph has.
+int build_q1_layout(ahpp_graph* g, uint32_t vec_width);
 // Index into kChunkSizes of a configured chunk size (0: the default), -1 if
 // it is not one of them.
 int chunk_choice(uint32_t chunk);

@@ -23,6 +23,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace ahpp {
@@ -49,6 +50,55 @@ struct ItemList {
   uint32_t n_long = 0;                  // batched lists: rows [0, n_long) are chunked
 };
 
+// Sliced rows of the single-query pull phases (built by ahpp_q1layout.cu).
+// A step is 128 entries, four per lane of a warp; it is stored as units of
+// 512 bytes, 16 per lane: an index unit (uint32) and a coefficient unit (FP32),
+// or one compact unit of four uint16 indices and four bfloat16 weights per lane
+// (attribute steps whose indices fit and whose weights are bfloat16).  An item
+// is a slice of 32 / vw rows of similar length (rows are sorted by degree)
+// with vw lanes on each row: entry k of a row sits in step k / (4 vw), lane
+// (k / 4) % vw of the row, place k % 4; places past a row's end hold index 0
+// and coefficient 0.  An item's V steps come before its attribute steps.  Rows
+// too long for one warp are cut into chunk items (vw = 32, one row):
+//   {first row, rows | lg vw << 8 | chunk << 31, V steps, attribute steps}
+// Every warp of the grid owns one range of items, its chunks first, cut so that
+// the warps' costs are about equal, and their units, which lie in the order in
+// which it uses them: ranges[w] = {item begin, end, unit begin, end}.
+struct Q1Rows {
+  const uint4* items = nullptr;
+  const uint4* ranges = nullptr;
+  const uint4* units = nullptr;         // [units][32]
+  const uint32_t* chunks_of = nullptr;  // chunks of each split row (rows [0, n_split))
+  uint32_t n_split = 0;
+};
+
+// The attribute hop U -> A, cut by blocks of U rows: block b of rows (vb[b] =
+// {first row, rows}) adds up its rows' share of every attribute it touches
+// from a copy of their residues in shared memory, then one reduction per
+// (block, attribute).  Items over (block, attribute) segments:
+//   {first segment, segments | lg vw << 8, first unit, steps}
+// with row indices local to the block; ranges[w] = {item begin, end, unit
+// begin, end} of warp w % kQ1Warps of block w / kQ1Warps; meta[s] = {attribute,
+// bits of the float scale of the sum} of segment s.
+struct Q1Segs {
+  const uint4* items = nullptr;
+  const uint4* ranges = nullptr;
+  const uint2* vb = nullptr;
+  const uint2* meta = nullptr;
+  const uint4* units = nullptr;
+  uint32_t n_vb = 0, own_cap = 0;       // blocks of rows, and the most rows of one
+};
+
+struct Q1Layout {
+  Q1Rows v, u;
+  Q1Segs s;
+  const uint32_t *deg_u = nullptr, *deg_v = nullptr, *deg_a = nullptr;
+  uint32_t n_warps = 0;                 // ranges per row space
+  uint32_t compact_a = 0, compact_s = 0;   // attribute steps of u / s in compact units
+  // leading entries of p, t_A and t_V that the pull phases hold in shared memory
+  uint32_t hub_u = 0, hub_a = 0, hub_v = 0;
+};
+
 struct DevGraph {
   uint32_t n_u = 0, n_v = 0, n_a = 0;
   uint32_t n_e = 0, n_ea = 0;
@@ -66,8 +116,9 @@ struct DevGraph {
   const float* cnorm_a = nullptr;
   float alpha = 0.f;
   float k_attr = 0.f;                   // (1 - alpha) * beta
-  // single-query (one row per lane / warp-cooperative) work items
-  ItemList s1_v, s1_a, s1_u;
+  // single-query push rounds: work items of the V and attribute flush
+  ItemList s1_v, s1_a;
+  Q1Layout q1;                          // single-query pull rounds
   // batched row-group units (the active chunk size) and those of every chunk
   // choice (kChunkSizes); b_split_max = the most split slots of any choice
   ItemList b_v, b_a, b_u;
@@ -133,55 +184,57 @@ struct RAcc {
   uint32_t above;
 };
 
-// Software grid barrier for persistent cooperative launches.  Every spin is
-// bounded; on expiry the barrier records an error and returns false, and the
-// kernel unwinds instead of hanging.
-struct GridBarrier {
+// Software grid barrier for persistent cooperative launches: blocks count up
+// one word, which the host clears before the launch, and wait until it has
+// reached the arrivals of all blocks at all barriers so far (`epoch`, kept by
+// the caller).  One word instead of a counter and a generation saves the last
+// block's two extra round trips to L2 on the path that every block waits for.
+// Every spin is bounded; on expiry the barrier records an error and returns
+// false, and the kernel unwinds instead of hanging.
+struct alignas(16) GridBarrier {
   unsigned int count;
-  unsigned int gen;
   unsigned int err;
-  unsigned int pad;
+  unsigned int pad[2];
 };
 
-constexpr unsigned int kSpinLimit = 1u << 22;   // x ~256 ns sleep, about one second
+constexpr unsigned int kSpinLimit = 1u << 20;   // polls of about a microsecond: about one second
+constexpr unsigned int kSpinEager = 64;         // polls before the wait backs off
 
-__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+// Arrivals (low word) and error flag (high word) in one acquiring load.
+__device__ __forceinline__ unsigned long long ld_barrier(const GridBarrier* b) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(b) : "memory");
   return v;
 }
 
-// Barrier over the blocks [0, nblocks) that share `b`.
-__device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned int nblocks) {
+// Barrier over the blocks [0, nblocks) that share `b`; epoch starts at 0 with
+// b->count cleared and is the same in every block.  then() runs in thread 0 of
+// every block once all have arrived, before the block's other threads go on.
+template <typename Then>
+__device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned int nblocks, unsigned int& epoch, Then then) {
   __shared__ unsigned int s_ok;
-  // data written with ordinary stores before the barrier may be read by TMA
-  // (the async proxy) after it
-  asm volatile("fence.proxy.async.global;" ::: "memory");
+  epoch += nblocks;
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned int ok = 1;
-    unsigned int g = ld_acquire_u32(&b->gen);
-    __threadfence();
-    unsigned int arrived = atomicAdd(&b->count, 1u);
-    if (arrived == nblocks - 1) {
-      atomicExch(&b->count, 0u);
-      __threadfence();
-      atomicAdd(&b->gen, 1u);
-    } else {
-      unsigned int spins = 0;
-      while (ld_acquire_u32(&b->gen) == g) {
-        if (++spins > kSpinLimit) { atomicOr(&b->err, 1u); ok = 0; break; }
-        if ((spins & 255u) == 0 && ld_acquire_u32(&b->err)) { ok = 0; break; }
-        __nanosleep(256);
-      }
+    // the release covers the block's writes (ordered before it by the block
+    // barrier), the acquire its later reads; a fence on either side instead
+    // would add about 500 cycles each to the 2,500 that this takes
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
+    unsigned int spins = 0;
+    unsigned long long w = ld_barrier(b);
+    while ((w >> 32) == 0 && (int)((unsigned int)w - epoch) < 0) {
+      if (++spins > kSpinLimit) { atomicOr(&b->err, 1u); w = 1ull << 32; break; }
+      if (spins > kSpinEager) __nanosleep(40);
+      w = ld_barrier(b);
     }
-    __threadfence();
-    if (ld_acquire_u32(&b->err)) ok = 0;
-    s_ok = ok;
+    s_ok = (w >> 32) == 0;
+    if (s_ok) then();
   }
   __syncthreads();
-  asm volatile("fence.proxy.async.global;" ::: "memory");
   return s_ok != 0;
+}
+__device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned int nblocks, unsigned int& epoch) {
+  return grid_sync(b, nblocks, epoch, [] {});
 }
 
 // ------------------------------------------------------------ reductions
@@ -257,48 +310,54 @@ struct Partials {
   unsigned long long marked_deg = 0;
   unsigned long long np_flush = 0;
   double sum_r = 0.0;
-  float max_rel = 0.f;       // APP(S) statistics (see RAcc)
-  uint32_t above = 0;
 };
 
-// Block reduction of Partials into acc (one atomic per field per block);
-// NW = warps per block; APPS: also APP(S)'s max_rel and above.
-template <int NW, bool APPS = false>
-__device__ __forceinline__ void flush_partials(Partials& p, RAcc* acc) {
-  __shared__ float s_max[NW];
-  __shared__ uint32_t s_marked[NW];
-  __shared__ unsigned long long s_deg[NW], s_np[NW];
-  __shared__ double s_sum[NW];
-  __shared__ float s_rel[NW];
-  __shared__ uint32_t s_above[NW];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float m = warp_max(p.max_r);
-  uint32_t mk = warp_sum_u32(p.marked);
-  unsigned long long dg = warp_sum_u64(p.marked_deg);
-  unsigned long long np = warp_sum_u64(p.np_flush);
-  double sm = warp_sum_d(p.sum_r);
-  float rel = APPS ? warp_max(p.max_rel) : 0.f;
-  uint32_t ab = APPS ? warp_sum_u32(p.above) : 0u;
-  if (lane == 0) {
-    s_max[warp] = m; s_marked[warp] = mk; s_deg[warp] = dg; s_np[warp] = np; s_sum[warp] = sm;
-    s_rel[warp] = rel; s_above[warp] = ab;
+// FP64 runs at two lanes a cycle on an SM of this chip: one FP64 instruction
+// of a full block of 1,024 threads takes a quarter of a microsecond, an FP64
+// log in every thread 25.  So the per-round tests of the kernels are taken in
+// FP32 where that decides them for certain, and in FP64 only in the band where
+// rounding could; the outcome is the FP64 test's in every case.
+
+// Smallest float f with (r > th) <=> (r >= f) for every float r: the mark
+// test r > th of Algorithm 4 taken exactly against the FP64 threshold.
+__host__ __device__ inline float threshold_up(double th) {
+  float f = (float)th;
+  if ((double)f <= th) f = nextafterf(f, INFINITY);
+  return f;
+}
+
+// r > th * cnt (APP's per-node threshold), th_f = (float)th.
+__device__ __forceinline__ bool above_node_threshold(float r, double th, float th_f, uint32_t cnt) {
+  const float t = th_f * (float)cnt;                 // relative error below 3 * 2^-24
+  if (t > 1e-30f) {
+    if (r > t * 1.000001f) return true;
+    if (r < t * 0.999999f) return false;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < NW; ++w) {
-      m = fmaxf(m, s_max[w]); mk += s_marked[w]; dg += s_deg[w]; np += s_np[w]; sm += s_sum[w];
-      if (APPS) { rel = fmaxf(rel, s_rel[w]); ab += s_above[w]; }
-    }
-    if (APPS && rel > 0.f) atomicMax(&acc->max_rel_bits, __float_as_uint(rel));
-    if (APPS && ab) atomicAdd(&acc->above, ab);
-    if (m > 0.f) atomicMax(&acc->max_r_bits, __float_as_uint(m));
-    if (mk) atomicAdd(&acc->marked, mk);
-    if (dg) atomicAdd(&acc->marked_deg, dg);
-    if (np) atomicAdd(&acc->np_flush, np);
-    if (sm != 0.0) atomicAdd(&acc->sum_r, sm);
-  }
-  __syncthreads();
-  p = Partials();
+  return (double)r > th * (double)cnt;
+}
+
+// The switch test of Algorithm 4, n_p >= 2 (|E| + |E_A|) max(0, log(M / eps_f)) / log_inv
+// (rule 0), or with log(1 / (lambda M)) in the place of the log (rule 1, as
+// printed); never for rule 2.
+static __device__ __noinline__ bool switch_due_fp64(uint32_t e_tot, int rule, double eps_f, double lambda,
+                                                    double log_inv, unsigned long long n_p, float m) {
+  const double EE = (double)e_tot, M = (double)m;
+  const double budget = rule == 1 ? 2.0 * EE * (log(1.0 / (lambda * M)) / log_inv)
+                                  : 2.0 * EE * fmax(0.0, log(M / eps_f) / log_inv);
+  return (double)n_p >= budget;
+}
+
+// log_ref: (float)log(eps_f) (rule 0) or (float)log(1 / lambda) (rule 1);
+// unit: (float)(2 (|E| + |E_A|) / log_inv).  Both logs are off by less than
+// 1e-5 for every float M and normal eps_f, so a margin of 1e-4 decides.
+__device__ __forceinline__ bool switch_due(uint32_t e_tot, int rule, double eps_f, double lambda, double log_inv,
+                                           float unit, float log_ref, unsigned long long n_p, float m) {
+  if (rule == 2) return false;
+  const float l = logf(m), d = rule == 1 ? log_ref - l : fmaxf(0.f, l - log_ref);
+  const float have = (float)n_p;
+  if (have > unit * (d + 1e-4f) * 1.00001f) return true;
+  if (have < unit * (d - 1e-4f) * 0.99999f) return false;
+  return switch_due_fp64(e_tot, rule, eps_f, lambda, log_inv, n_p, m);
 }
 
 // Kahan-compensated accumulation s += v with compensation c (FP32).

@@ -68,8 +68,6 @@ size_t carve(const ahpp_graph* g, char* base, Q1State* s) {
   s->racc = (RAcc*)take(3 * sizeof(RAcc));
   s->bar = (GridBarrier*)take(sizeof(GridBarrier));
   s->final_maxr_bits = (unsigned int*)take(2 * sizeof(unsigned int));
-  s->trace_frontier = nullptr;
-  s->trace_maxr = nullptr;
   return off;
 }
 
@@ -110,7 +108,6 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
   carve(g, (char*)g_noalloc_ptr[g->device], &s);
   cudaStream_t st = stream ? (cudaStream_t)stream : g->stream;
   Q1Params p = noalloc_params(g, g->h_u_old2new[q], eps);
-  p.trace_cap = 0;
   if (int rc = reset_barrier(g, s.bar, st)) return rc;
   const int e = launch_query1(g->dg, s, p, g->bf16, g->q1_grid, st);
   if (e) return cuda_fail((cudaError_t)e, "ahpp_query_dense_noalloc: launch");

@@ -4,30 +4,33 @@
 
 namespace ahpp {
 
-// Device state of one query (all arrays indexed by internal ids).
-// Block size of the single-query kernel: kQ1Blocks blocks of kQ1Threads per
-// SM (64 registers a thread).  Measured on the medium graph: one block of
-// 1024 a little faster (34.5 ms a query) than two of 512 (36.1 ms).
+// Block size of the single-query kernel: one block of kQ1Threads per SM (64
+// registers a thread).  On the medium graph 1,024 threads with rings of four
+// units took 24.0 ms a query, 768 threads 24.5, 512 with rings of eight 31.3.
 constexpr int kQ1Threads = 1024;
 constexpr int kQ1Warps = kQ1Threads / 32;
 constexpr int kQ1Blocks = 1;
-// Default lanes per short row (the fastest on the medium graph: 33.7 ms a
-// query against 39.7 / 40.0 / 70.4 for 1 / 8 / 32 lanes, autotuner timings).
-constexpr uint32_t kQ1VecWidthDefault = 2;
+// The most dynamic shared memory of a block.  What is left of the 256 KB is L1,
+// whose lines hold the lookups in flight: 21.4 ms a query on the medium graph
+// at 188 KB, 22.0 at 160, 21.8 at 128 (less of the tables copied), 36.5 at 204.
+constexpr uint32_t kQ1SmemMax = 188 * 1024;
+// Units (512 bytes) of each warp's ring in shared memory: its stream of graph
+// entries is copied that far ahead of its use.
+constexpr uint32_t kQ1Ring = 4;
+constexpr uint32_t kQ1RingBytes = kQ1Warps * kQ1Ring * 512;
 
+// Device state of one query (all arrays indexed by internal ids).
 struct Q1State {
   float *r_u = nullptr, *pi = nullptr, *pic = nullptr;   // residues (sign = marked), reserves, Kahan
   float *t_v = nullptr, *t_a = nullptr;                  // r(v)/d(v), r(a)/W_col(a)
-  float* t_a2 = nullptr;                                 // the other t_A buffer (attribute push)
+  float* t_a2 = nullptr;                                 // the other t_A buffer (pull rounds alternate)
   uint32_t* list_u = nullptr;                            // push rounds: the marked list
-  float* split_acc = nullptr;                            // partial sums of split rows
-  uint32_t* split_cnt = nullptr;                         // finished chunks of split rows
+  float* split_acc = nullptr;                            // sums of split rows (see SplitAcc)
+  uint32_t* split_cnt = nullptr;                         // finished chunks of split U rows
   QCtl* ctl = nullptr;
   RAcc* racc = nullptr;                                  // [3]
   GridBarrier* bar = nullptr;
   unsigned int* final_maxr_bits = nullptr;               // [2]: max |r_U|, max pi
-  uint32_t* trace_frontier = nullptr;                    // [trace_cap] frontier size per round
-  float* trace_maxr = nullptr;                           // [trace_cap] max r_U after each round
 };
 
 struct Q1Params {
@@ -39,21 +42,14 @@ struct Q1Params {
   double lambda = 1.0;
   double log_inv = 0.0;        // ln(1 / (1 - alpha))
   uint32_t e_tot = 0;          // |E| + |E_A|
+  // FP32 forms of the tests above (see switch_due, above_node_threshold):
+  // smallest floats above eps_f and 0, eps_f, 2 e_tot / log_inv, and the log of
+  // the switch test's reference
+  float th_async = 0.f, th_sync = 0.f, eps_f32 = 0.f, switch_unit = 0.f, switch_log = 0.f;
   uint32_t max_rounds = 0;
   uint32_t dense_div = 32;     // pull rounds once the frontier covers > 1/dense_div of the edges
-  uint32_t n_split = 0;        // split-row slots (phase 1 V + A, phase 2 U)
-  uint32_t trace_cap = 0;
-  // Pull rounds and shared memory (dynamic, smem_bytes per block):
-  //   attr_push: the attribute hop of round t+1 is pushed during round t's
-  //     phase 2 into a block-local accumulator over A (shared memory), then
-  //     added to the next t_A; otherwise it is pulled in phase 1 over A->U;
-  //   ta_smem: phase 2 reads t_A from a shared-memory copy.
-  uint32_t smem_bytes = 0;
-  int attr_push = 0;
-  int ta_smem = 0;
-  // short rows of the pull phases: at most vw_max lanes per row (a power of
-  // two, 1..32; 1 = one row per lane)
-  uint32_t vw_max = 32;
+  uint32_t n_split = 0;        // entries of split_acc
+  uint32_t smem_bytes = 0;     // dynamic shared memory of a block (Q1Layout's tables)
   // Theorem 3 mode: start from r = 1 on every U node, run exactly max_rounds
   // synchronous rounds; the reserves are then pi_T and final_maxr_bits[1]
   // holds max_u pi_T(u).
@@ -68,8 +64,6 @@ int launch_query1(const DevGraph& g, const Q1State& s, const Q1Params& p, bool b
                   cudaStream_t stream);
 // Persistent grid of the single-query kernel with smem_bytes of dynamic
 // shared memory per block (-1 if it cannot be made resident).
-int query1_max_grid(bool bf16, int sm_count, uint32_t smem_bytes);
-// Largest dynamic shared memory a block of the single-query kernel may use.
-uint32_t query1_max_smem(int device);
+int query1_max_grid(int sm_count, uint32_t smem_bytes);
 
 }  // namespace ahpp

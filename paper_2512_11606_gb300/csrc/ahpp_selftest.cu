@@ -13,7 +13,8 @@ namespace ahpp {
 namespace {
 
 __global__ void k_wait_selftest(GridBarrier* bar, unsigned int participants, unsigned int* gave_up) {
-  const bool ok = grid_sync(bar, participants);
+  unsigned int epoch = 0;
+  const bool ok = grid_sync(bar, participants, epoch);
   if (threadIdx.x == 0 && !ok) atomicAdd(gave_up, 1u);
 }
 

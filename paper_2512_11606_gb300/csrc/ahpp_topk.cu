@@ -20,11 +20,12 @@ __device__ __forceinline__ unsigned long long key_of(const float* score, const u
          (unsigned long long)(0xffffffffu - n2o[u]);
 }
 
+// hist, cand_cnt and bar start at zero (cleared by the host before a launch).
 struct TopkScratch {
   unsigned int* hist;          // [kPasses][kBinsMax]
-  unsigned long long* cand;    // [AHPP_MAX_K]
   uint32_t* cand_cnt;
   GridBarrier* bar;
+  unsigned long long* cand;    // [AHPP_MAX_K]
 };
 
 __global__ void __launch_bounds__(kThreads)
@@ -34,9 +35,7 @@ k_topk1(const float* __restrict__ score, const uint32_t* __restrict__ n2o, uint3
   __shared__ unsigned long long sk[AHPP_MAX_K];
   const uint32_t gt = blockIdx.x * kThreads + threadIdx.x, nt = gridDim.x * kThreads;
   const unsigned int nb = gridDim.x;
-  for (uint32_t i = gt; i < kPasses * kBinsMax; i += nt) sc.hist[i] = 0;
-  if (gt == 0) *sc.cand_cnt = 0;
-  if (!grid_sync(sc.bar, nb)) return;
+  unsigned int epoch = 0;
   unsigned long long prefix = 0;
   unsigned long long thresh = 0;   // smallest winning key, once known
   uint32_t krem = k;
@@ -59,7 +58,7 @@ k_topk1(const float* __restrict__ score, const uint32_t* __restrict__ n2o, uint3
     unsigned int* gh = sc.hist + pass * kBinsMax;
     for (int i = threadIdx.x; i < bins; i += kThreads)
       if (sh[i]) atomicAdd(&gh[i], sh[i]);
-    if (!grid_sync(sc.bar, nb)) return;
+    if (!grid_sync(sc.bar, nb, epoch)) return;
     // the merged histogram into shared memory, then a warp-parallel pick
     for (int i = threadIdx.x; i < bins; i += kThreads) sh[i] = __ldcg(&gh[i]);
     __syncthreads();
@@ -83,7 +82,7 @@ k_topk1(const float* __restrict__ score, const uint32_t* __restrict__ n2o, uint3
       if (pos < AHPP_MAX_K) sc.cand[pos] = key;
     }
   }
-  if (!grid_sync(sc.bar, nb)) return;
+  if (!grid_sync(sc.bar, nb, epoch)) return;
   if (blockIdx.x != 0) return;
   uint32_t m = 1;
   while (m < k) m <<= 1;
@@ -116,19 +115,20 @@ int topk_single(ahpp_graph* g, const float* d_score, uint32_t k, uint32_t* d_nod
   const uint32_t n = (uint32_t)g->n_u;
   if (k > n) k = n;
   if (k == 0) return cudaMemsetAsync(d_n, 0, 4, stream) == cudaSuccess ? AHPP_OK : AHPP_ECUDA;
-  const size_t need = kPasses * kBinsMax * 4 + AHPP_MAX_K * 8 + 16 + sizeof(GridBarrier);
+  const size_t hist_bytes = kPasses * kBinsMax * 4, clear = hist_bytes + 16 + sizeof(GridBarrier);
+  const size_t need = clear + AHPP_MAX_K * 8;
   if (!g->topk_scratch) {
     g->topk_scratch = g->alloc(need);
     if (!g->topk_scratch) { set_error("top-k scratch allocation failed"); return AHPP_ENOMEM; }
     g->topk_scratch_bytes = need;
-    AHPP_CUDA(cudaMemset(g->topk_scratch, 0, need));
   }
   char* base = (char*)g->topk_scratch;
   TopkScratch sc;
   sc.hist = (unsigned int*)base;
-  sc.cand = (unsigned long long*)(base + kPasses * kBinsMax * 4);
-  sc.cand_cnt = (uint32_t*)(base + kPasses * kBinsMax * 4 + AHPP_MAX_K * 8);
-  sc.bar = (GridBarrier*)(base + kPasses * kBinsMax * 4 + AHPP_MAX_K * 8 + 16);
+  sc.cand_cnt = (uint32_t*)(base + hist_bytes);
+  sc.bar = (GridBarrier*)(base + hist_bytes + 16);
+  sc.cand = (unsigned long long*)(base + clear);
+  AHPP_CUDA(cudaMemsetAsync(base, 0, clear, stream));
   static int per_sm = 0;
   if (per_sm == 0) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_topk1, kThreads, 0) !=

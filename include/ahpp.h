@@ -89,9 +89,12 @@ typedef struct {
     uint32_t max_rounds;       /* round cap per query; 0: automatic */
     uint32_t batch_tile;       /* queries per batched tile: 16 or 32; 0: 32 (ahpp_autotune picks one);
                                   serving always uses tiles of 32 */
-    uint32_t batch_groups;     /* tiles processed concurrently, 1..8; 0: 1 (ahpp_autotune picks 1, 2 or 4) */
-    uint32_t batch_chunk;      /* entries per chunk of a long row in the batched kernel: 128, 256 or
-                                  512; 0: 256 (ahpp_autotune picks one) */
+    uint32_t batch_groups;     /* tiles processed concurrently, 1..8; 0: as many as share the GPU well,
+                                  by the graph's size and the batch's (ahpp_autotune keeps that or
+                                  picks 1, 2 or 4) */
+    uint32_t batch_chunk;      /* entries per chunk of a long row in the batched kernel, at most: 128,
+                                  256 or 512 (less on graphs too small for it); 0: 256
+                                  (ahpp_autotune picks one) */
     uint32_t single_vec_width; /* single-query kernel: at least this many lanes walk one row
                                   (1, 2, 4, 8, 16 or 32); 0: 1, 2, 8 or 32 by the graph's size
                                   (ahpp_autotune picks one of those) */
@@ -123,7 +126,8 @@ typedef struct {
     uint64_t tile_state_bytes;           /* device bytes per batched tile */
     int device;
     int sm_count;
-    uint32_t batch_tile, batch_groups;   /* batched launch shape in use */
+    uint32_t batch_tile, batch_groups;   /* batched launch shape in use (groups: 1 where the
+                                            configuration leaves them to the library) */
     uint32_t batch_chunk;                /* batched: entries per chunk of a long row */
     /* single-query kernel (the plain path): pull rounds once the frontier's
      * degree sum exceeds 1/single_dense_div of |E| + |E_A|; the attribute hop
@@ -265,7 +269,7 @@ int ahpp_query_device(ahpp_graph *g, uint32_t q, double eps, uint32_t k,
  * knob at a time with the others fixed.  Batched kernel, on the sample
  * replicated to fill four tiles of 32: queries per tile (32, 16), entries per
  * chunk of a long row (128, 256, 512), then tiles processed concurrently
- * (1, 2, 4).  Single-query kernel, on
+ * (by the library's rule, 1, 2, 4; a later value has to be 2 % faster).  Single-query kernel, on
  * up to four sample queries: lanes per short row (32, 8, 2, 1: at least that
  * many lanes walk one row; the kernel's layout of the graph is built anew for
  * each), then the frontier fraction 1/dense_div (8, 16,

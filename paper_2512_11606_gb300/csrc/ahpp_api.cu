@@ -50,14 +50,10 @@ __global__ void k_ctl_to_stats(const QCtl* ctl, const unsigned int* maxr, const 
   *st = S;
 }
 
-struct WaitBars {
-  const GridBarrier* bar[kMaxGroups];
-  uint32_t n_bars;
-};
-
-__global__ void k_batch_wait_status(const WaitBars wb, uint32_t n, ahpp_stats* st, uint32_t* out_n) {
+__global__ void k_batch_wait_status(const GridBarrier* bars, uint32_t n_bars, uint32_t n, ahpp_stats* st,
+                                    uint32_t* out_n) {
   unsigned int err = 0;
-  for (uint32_t i = 0; i < wb.n_bars; ++i) err |= wb.bar[i]->err;
+  for (uint32_t i = 0; i < n_bars; ++i) err |= bars[i].err;
   if (!err) return;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (st) st[i].status = kStatusWait;
@@ -137,27 +133,28 @@ Q1Params noalloc_params(const ahpp_graph* g, uint32_t q_new, double eps) {
   return q1_params(g, q_new, eps);
 }
 
-int reset_barrier(ahpp_graph* g, GridBarrier* bar, cudaStream_t stream, bool keep_trap) {
-  AHPP_CUDA(cudaMemsetAsync(bar, 0, sizeof(GridBarrier), stream));
-  if (g && g->wait_trap.load()) {
+int reset_barriers(ahpp_graph* g, GridBarrier* bars, uint32_t n, cudaStream_t stream) {
+  AHPP_CUDA(cudaMemsetAsync(bars, 0, n * sizeof(GridBarrier), stream));
+  if (g && g->wait_trap.exchange(0)) {
     // 0xc0c0c0c0 arrivals, a billion below the first barrier's block count
-    AHPP_CUDA(cudaMemsetAsync(&bar->count, 0xc0, sizeof(bar->count), stream));
-    if (!keep_trap) g->wait_trap.store(0);
+    AHPP_CUDA(cudaMemset2DAsync(&bars->count, sizeof(GridBarrier), 0xc0, sizeof(bars->count), n, stream));
   }
   return AHPP_OK;
 }
 
-int barrier_status(GridBarrier* bar, cudaStream_t stream, int* status) {
-  unsigned int err = 0;
-  AHPP_CUDA(cudaMemcpyAsync(&err, &bar->err, sizeof(err), cudaMemcpyDeviceToHost, stream));
+int barrier_status(const GridBarrier* bars, uint32_t n, cudaStream_t stream, int* status) {
+  GridBarrier h[kMaxGroups];
+  AHPP_CUDA(cudaMemcpyAsync(h, bars, n * sizeof(GridBarrier), cudaMemcpyDeviceToHost, stream));
   AHPP_CUDA(cudaStreamSynchronize(stream));
-  *status = err ? kStatusWait : kStatusOk;
+  *status = kStatusOk;
+  for (uint32_t i = 0; i < n; ++i)
+    if (h[i].err) *status = kStatusWait;
   return AHPP_OK;
 }
 
 int run_query1_launch(ahpp_graph* g, uint32_t q_new, double eps, cudaStream_t stream) {
   Q1Params p = q1_params(g, q_new, eps);
-  if (int rc = reset_barrier(g, g->q1.bar, stream)) return rc;
+  if (int rc = reset_barriers(g, g->q1.bar, 1, stream)) return rc;
   int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, stream);
   if (e) return cuda_fail((cudaError_t)e, "k_query1 launch");
   return AHPP_OK;
@@ -176,7 +173,7 @@ int run_lambda(ahpp_graph* g) {
   set_tests(p);
   p.kahan = 1;
   p.max_rounds = T;
-  if (int rc = reset_barrier(nullptr, g->q1.bar, g->stream)) return rc;
+  if (int rc = reset_barriers(nullptr, g->q1.bar, 1, g->stream)) return rc;
   int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, g->stream);
   if (e) return cuda_fail((cudaError_t)e, "lambda launch");
   unsigned int bits[2] = {0, 0};
@@ -184,7 +181,7 @@ int run_lambda(ahpp_graph* g) {
   AHPP_CUDA(cudaMemcpyAsync(bits, g->q1.final_maxr_bits, sizeof(bits), cudaMemcpyDeviceToHost, g->stream));
   AHPP_CUDA(cudaMemcpyAsync(&ctl, g->q1.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, g->stream));
   int bst = kStatusOk;
-  if (int rc = barrier_status(g->q1.bar, g->stream, &bst)) return rc;
+  if (int rc = barrier_status(g->q1.bar, 1, g->stream, &bst)) return rc;
   if (ctl.status == kStatusWait || bst == kStatusWait) {
     set_error("lambda estimate: device wait gave up");
     return AHPP_ETIMEOUT;
@@ -197,12 +194,11 @@ int run_lambda(ahpp_graph* g) {
   return AHPP_OK;
 }
 
-int batch_plan(ahpp_graph* g, BatchParams& p) {
+int batch_plan(ahpp_graph* g) {
   if (g->bt_grid <= 0) {
-    g->bt_grid = batch_max_grid(g->bf16, g->sm_count);
+    g->bt_grid = batch_max_grid(g->sm_count);
     if (g->bt_grid <= 0) { set_error("batched occupancy query failed"); return AHPP_ECUDA; }
   }
-  (void)p;
   return AHPP_OK;
 }
 
@@ -211,55 +207,72 @@ int ensure_batch(ahpp_graph* g, uint32_t groups, uint32_t kmax) {
   kmax = std::max<uint32_t>(kmax, 1);
   if (s.n_groups >= groups && s.kmax_cap >= kmax) return AHPP_OK;
   const DevGraph& G = g->dg;
-  const size_t n_split = G.b_split_max;        // any chunk choice fits
+  const size_t n_split = std::max(G.tl.split_u_max, 1u);        // any chunk choice fits
   const uint32_t kcap = std::max(kmax, s.kmax_cap);
   const uint32_t ng = std::max(groups, s.n_groups);
   uint64_t bytes = 0;
-  for (uint32_t i = 0; i < ng; ++i) {
+  bool ok = true;
+  auto A = [&](size_t b) {
+    bytes += b;
+    void* p = g->alloc(b);
+    ok = ok && p;
+    return p;
+  };
+  if (!s.bars) {
+    s.bars = (GridBarrier*)A(kMaxGroups * sizeof(GridBarrier));
+    s.d_tb = (TileBuf*)A(kMaxGroups * sizeof(TileBuf));
+    if (ok) AHPP_CUDA(cudaMemset(s.bars, 0, kMaxGroups * sizeof(GridBarrier)));
+    bytes = 0;
+  }
+  for (uint32_t i = 0; i < ng && ok; ++i) {
     TileBuf& t = s.tb[i];
     const bool fresh = i >= s.n_groups;
-    auto A = [&](size_t b) { bytes += b; return g->alloc(b); };
     if (fresh) {
       t.r_u = (float*)A((size_t)G.n_u * kTile * 4);
       t.pi = (float*)A((size_t)G.n_u * kTile * 4);
       t.pic = (float*)A((size_t)G.n_u * kTile * 4);
-      t.t_v = (float*)A((size_t)std::max(G.n_v, 1u) * kTile * 4);
-      t.t_a = (float*)A((size_t)std::max(G.n_a, 1u) * kTile * 4);
-      t.t_a2 = (float*)A((size_t)std::max(G.n_a, 1u) * kTile * 4);
-      t.split_acc = (float*)A(std::max<size_t>(n_split, 1) * kTile * 4);
-      t.split_cnt = (uint32_t*)A(std::max<size_t>(n_split, 1) * 4);
-      t.racc = (RAcc*)A(5 * kTile * sizeof(RAcc));
-      t.bar = (GridBarrier*)A(sizeof(GridBarrier));
+      t.t = (float*)A(((size_t)G.n_v + 2 * (size_t)G.tl.acc_max + 1) * kTile * 4);
+      t.split_acc = (float*)A(n_split * kTile * 4);
+      t.split_cnt = (uint32_t*)A(n_split * 4);
+      t.tacc = (TAcc*)A(kTAccs * sizeof(TAcc));
+      t.racc = (RAcc*)A(2 * kTile * sizeof(RAcc));
       t.hist = (unsigned int*)A((size_t)kRadixPasses * kTile * kRadixBins * 4);
       t.cand_cnt = (uint32_t*)A(kTile * 4);
-      if (!t.r_u || !t.pi || !t.pic || !t.t_v || !t.t_a || !t.t_a2 || !t.split_acc || !t.split_cnt ||
-          !t.racc || !t.bar || !t.hist || !t.cand_cnt) {
-        set_error("batched state allocation failed");
-        return AHPP_ENOMEM;
-      }
-      AHPP_CUDA(cudaMemset(t.bar, 0, sizeof(GridBarrier)));
     }
-    if (fresh || kcap > s.kmax_cap) {
-      t.cand = (unsigned long long*)A((size_t)kTile * kcap * 8);
-      if (!t.cand) { set_error("batched state allocation failed"); return AHPP_ENOMEM; }
-    }
+    if (fresh || kcap > s.kmax_cap) t.cand = (unsigned long long*)A((size_t)kTile * kcap * 8);
   }
+  if (!ok) { set_error("batched state allocation failed"); return AHPP_ENOMEM; }
+  AHPP_CUDA(cudaMemcpy(s.d_tb, s.tb, ng * sizeof(TileBuf), cudaMemcpyHostToDevice));
   if (s.n_groups == 0) g->tile_bytes = bytes / ng;
   s.n_groups = ng;
   s.kmax_cap = kcap;
   return AHPP_OK;
 }
 
+// Parameters that a batch and a serving step share.
+void set_batch_params(const ahpp_graph* g, BatchParams& p) {
+  p.u_old2new = g->d_u_old2new;
+  p.u_new2old = g->d_u_new2old;
+  p.algo = kernel_algo(g->cfg.algo);
+  p.kahan = g->cfg.kahan;
+  p.switch_rule = g->cfg.switch_rule;
+  p.lambda = g->lambda;
+  p.log_inv = std::log(1.0 / (1.0 - g->cfg.alpha));
+  p.e_tot = (uint32_t)(g->n_e + g->n_ea);
+  p.switch_unit = (float)(2.0 * (double)p.e_tot / p.log_inv);
+  p.switch_log = (float)-std::log(p.lambda);
+}
+
 int run_batch_launch(ahpp_graph* g, uint32_t n, const uint32_t* d_q, const double* d_eps,
                      const uint32_t* d_k, uint32_t kmax, uint32_t* d_nodes, float* d_scores,
                      uint32_t* d_n, ahpp_stats* d_stats, float* d_dense, cudaStream_t stream) {
-  const uint32_t groups = std::max<uint32_t>(1, std::min<uint32_t>(g->batch_groups, kMaxGroups));
-  int rc = ensure_batch(g, groups, kmax);
+  int rc = batch_plan(g);
   if (rc) return rc;
+  const uint32_t groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile);
+  if ((rc = ensure_batch(g, groups, kmax))) return rc;
   BatchParams p;
-  if ((rc = batch_plan(g, p))) return rc;
-  const int grid = g->bt_grid / (int)groups * (int)groups;
-  if (grid < (int)groups) { set_error("grid too small for the group count"); return AHPP_EINVAL; }
+  const uint32_t per_group = (uint32_t)g->bt_grid / groups;
+  if ((rc = tile_ranges(g, per_group * kBWarps, &p.ranges_t, &p.ranges_u))) return rc;
   p.n = n;
   p.q = d_q;
   p.eps = d_eps;
@@ -270,30 +283,21 @@ int run_batch_launch(ahpp_graph* g, uint32_t n, const uint32_t* d_q, const doubl
   p.out_n = d_n;
   p.out_stats = d_stats;
   p.out_dense = d_dense;
-  p.u_old2new = g->d_u_old2new;
-  p.u_new2old = g->d_u_new2old;
-  p.algo = kernel_algo(g->cfg.algo);
-  p.kahan = g->cfg.kahan;
-  p.switch_rule = g->cfg.switch_rule;
-  p.lambda = g->lambda;
-  p.log_inv = std::log(1.0 / (1.0 - g->cfg.alpha));
-  p.e_tot = (uint32_t)(g->n_e + g->n_ea);
+  set_batch_params(g, p);
   // one cap for the whole launch: generous enough for eps down to 1e-14 / lambda
   p.max_rounds = g->cfg.max_rounds ? g->cfg.max_rounds
                                    : auto_rounds(1e-14 / std::max(g->lambda, 1.0), g->cfg.alpha);
   p.groups = groups;
+  p.tbufs = g->bt.d_tb;
+  p.bars = g->bt.bars;
   p.tile = g->batch_tile;
-  for (uint32_t i = 0; i < groups; ++i)
-    if (int rc = reset_barrier(g, g->bt.tb[i].bar, stream, i + 1 < groups)) return rc;
-  int e = launch_batch(g->dg, g->bt, p, g->bf16, grid, stream);
+  if ((rc = reset_barriers(g, g->bt.bars, groups, stream))) return rc;
+  int e = launch_batch(g->dg, p, (int)(per_group * groups), stream);
   if (e) return cuda_fail((cudaError_t)e, "k_batch launch");
   // a group whose barrier gave up may have left some of its tiles without
   // results: report every query of the launch as a device wait that gave up
-  WaitBars wb{};
-  for (uint32_t i = 0; i < groups; ++i) wb.bar[i] = g->bt.tb[i].bar;
-  wb.n_bars = groups;
   k_batch_wait_status<<<std::max<uint32_t>(1, std::min<uint32_t>((n + 255) / 256, 1024)), 256, 0, stream>>>(
-      wb, n, d_stats, d_n);
+      g->bt.bars, groups, n, d_stats, d_n);
   AHPP_CUDA(cudaGetLastError());
   return AHPP_OK;
 }
@@ -406,7 +410,7 @@ int ahpp_load_graph(const ahpp_graph_desc* desc, const ahpp_config* cfg, ahpp_gr
     set_error("ahpp_load_graph: batch_tile must be 0, 16 or 32");
     return AHPP_EINVAL;
   }
-  if (c.batch_groups > (uint32_t)kMaxGroups) {
+  if (c.batch_groups > kMaxBatchGroups) {
     set_error("ahpp_load_graph: batch_groups must be at most 8");
     return AHPP_EINVAL;
   }
@@ -430,14 +434,13 @@ int ahpp_load_graph(const ahpp_graph_desc* desc, const ahpp_config* cfg, ahpp_gr
   g->cfg = c;
   g->device = c.device;
   g->batch_tile = c.batch_tile ? c.batch_tile : (uint32_t)ahpp::kTile;
-  g->batch_groups = c.batch_groups ? c.batch_groups : 1;
+  g->batch_groups = c.batch_groups;
   int rc = AHPP_OK;
   if (cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
       cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess) {
     rc = cuda_fail(cudaGetLastError(), "ahpp_load_graph: device setup");
   }
   if (rc == AHPP_OK) rc = build_graph(desc, g);
-  if (rc == AHPP_OK) select_chunk(g->dg, (uint32_t)chunk_choice(c.batch_chunk));
   if (rc == AHPP_OK) {
     if (c.algo == AHPP_ASRP && !(c.lambda > 0.0)) rc = run_lambda(g);
     else g->lambda = c.lambda > 0.0 ? c.lambda : 1.0;
@@ -457,6 +460,7 @@ void ahpp_free_graph(ahpp_graph* g) {
   cudaSetDevice(g->device);
   if (g->stream) cudaStreamSynchronize(g->stream);
   for (void* p : g->q1_layout_bufs) cudaFree(p);
+  for (void* p : g->tile_layout_bufs) cudaFree(p);
   g->release_all();
   if (g->stream) cudaStreamDestroy(g->stream);
   io_drop(g);
@@ -475,8 +479,8 @@ int ahpp_get_graph_info(const ahpp_graph* g, ahpp_graph_info* info) {
   info->device = g->device;
   info->sm_count = g->sm_count;
   info->batch_tile = g->batch_tile;
-  info->batch_groups = g->batch_groups;
-  info->batch_chunk = kChunkSizes[g->dg.b_chunk];
+  info->batch_groups = std::max(1u, g->batch_groups);
+  info->batch_chunk = kChunkSizes[g->dg.tl.chunk];
   info->single_dense_div = g->q1_dense_div;
   info->single_attr_push = 1;
   info->single_vec_width = g->q1_vw_max;
@@ -505,7 +509,7 @@ static int finish_single(ahpp_graph* g, double eps, ahpp_stats* st) {
   AHPP_CUDA(cudaMemcpyAsync(&ctl, g->q1.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, g->stream));
   AHPP_CUDA(cudaMemcpyAsync(bits, g->q1.final_maxr_bits, sizeof(bits), cudaMemcpyDeviceToHost, g->stream));
   int bst = kStatusOk;
-  if (int rc = barrier_status(g->q1.bar, g->stream, &bst)) return rc;
+  if (int rc = barrier_status(g->q1.bar, 1, g->stream, &bst)) return rc;
   if (bst == kStatusWait) ctl.status = kStatusWait;
   if (st) {
     st->rounds = ctl.rounds;
@@ -544,7 +548,7 @@ int ahpp_power_iteration(ahpp_graph* g, uint32_t q, uint32_t T, float* out_pi, a
   p.eps_f = 0.0;
   set_tests(p);
   p.max_rounds = T;
-  if (int rc = reset_barrier(g, g->q1.bar, g->stream)) return rc;
+  if (int rc = reset_barriers(g, g->q1.bar, 1, g->stream)) return rc;
   int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, g->stream);
   if (e) return cuda_fail((cudaError_t)e, "power iteration launch");
   int rc;
@@ -766,8 +770,8 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     if (log.size() > 1) log += ", ";
     log += "\"" + std::string(knob) + "=" + std::to_string(v) + "\": " + std::to_string(t);
   };
-  // ---- batched launch shape, one knob at a time (hub rows in shared memory,
-  // entries per chunk of a long row, concurrent tile groups), every candidate
+  // ---- batched launch shape, one knob at a time (tile width, entries per chunk
+  // of a long row, concurrent tile groups), every candidate
   // on the same queries: the sample replicated to fill four tiles; one
   // warm-up launch first
   const uint32_t n = std::max<uint32_t>(n_sample, 4 * (uint32_t)kTile);
@@ -786,23 +790,23 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     float best = -1.f;
     uint32_t best_v = values[0];
     for (uint32_t v : values) {
-      set(v);
+      if (int r = set(v)) return r;
       float t = 0.f;
       if (int r = time_batch(g, io, n, &t)) return r;
       note(knob, v, t / (float)n);
-      if (best < 0.f || t < best) { best = t; best_v = v; }
+      // a later value has to be faster by more than runs differ
+      if (best < 0.f || t < 0.98f * best) { best = t; best_v = v; }
     }
-    set(best_v);
-    return AHPP_OK;
+    return set(best_v);
   };
-  const uint32_t saved_groups = g->batch_groups, saved_chunk = g->dg.b_chunk, saved_tile = g->batch_tile;
-  rc = tune_batch("batch_tile", [&](uint32_t v) { g->batch_tile = v; }, {(uint32_t)kTile, (uint32_t)kTileNarrow});
+  const uint32_t saved_groups = g->batch_groups, saved_chunk = g->dg.tl.chunk, saved_tile = g->batch_tile;
+  rc = tune_batch("batch_tile", [&](uint32_t v) { g->batch_tile = v; return AHPP_OK; }, {(uint32_t)kTile, (uint32_t)kTileNarrow});
   if (rc == AHPP_OK)
-    rc = tune_batch("batch_chunk_choice", [&](uint32_t v) { select_chunk(g->dg, v); }, {1u, 0u, 2u});
-  if (rc == AHPP_OK) rc = tune_batch("batch_groups", [&](uint32_t v) { g->batch_groups = v; }, {1u, 2u, 4u});
+    rc = tune_batch("batch_chunk_choice", [&](uint32_t v) { return build_tile_layout(g, v); }, {1u, 0u, 2u});
+  if (rc == AHPP_OK) rc = tune_batch("batch_groups", [&](uint32_t v) { g->batch_groups = v; return AHPP_OK; }, {0u, 1u, 2u, 4u});
   if (rc != AHPP_OK) {
     g->batch_groups = saved_groups;
-    select_chunk(g->dg, saved_chunk);
+    build_tile_layout(g, saved_chunk);
     g->batch_tile = saved_tile;
     return rc;
   }

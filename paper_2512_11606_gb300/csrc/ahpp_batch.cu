@@ -18,19 +18,16 @@
 
 namespace ahpp {
 
-int launch_batch(const DevGraph& g, const BatchState& s, const BatchParams& p, bool bf16, int grid,
-                 cudaStream_t stream) {
-  return p.tile == 16 ? tw16::launch_batch(g, s, p, bf16, grid, stream)
-                      : tw32::launch_batch(g, s, p, bf16, grid, stream);
+int launch_batch(const DevGraph& g, const BatchParams& p, int grid, cudaStream_t stream) {
+  return p.tile == 16 ? tw16::launch_batch(g, p, grid, stream) : tw32::launch_batch(g, p, grid, stream);
 }
 
-int launch_serve_step(const DevGraph& g, const BatchParams& p, const ServeParams& sv, bool bf16, int grid,
-                      cudaStream_t stream) {
-  return tw32::launch_serve_step(g, p, sv, bf16, grid, stream);
+int launch_serve_step(const DevGraph& g, const BatchParams& p, const ServeParams& sv, int grid, cudaStream_t stream) {
+  return tw32::launch_serve_step(g, p, sv, grid, stream);
 }
 
-int batch_max_grid(bool bf16, int sm_count) {
-  const int a = tw32::batch_max_grid(bf16, sm_count), b = tw16::batch_max_grid(bf16, sm_count);
+int batch_max_grid(int sm_count) {
+  const int a = tw32::batch_max_grid(sm_count), b = tw16::batch_max_grid(sm_count);
   return (a <= 0 || b <= 0) ? -1 : std::min(a, b);
 }
 

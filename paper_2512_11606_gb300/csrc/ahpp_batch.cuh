@@ -7,7 +7,10 @@
 // instance of a launch's width indexes them with its own width.
 // The graph is streamed once per round per tile, shared by all its queries.
 // `groups` tiles run concurrently, each on its own slice of the persistent
-// grid with its own barrier; a group walks its tiles one after another.
+// grid with its own barrier; a group walks its tiles one after another.  A
+// tile's round on a small graph is a few latencies and two barriers long
+// whatever its share of the chip: 2,000 nodes, 50 us a tile and round with one
+// group, 7 with eight.
 #pragma once
 #include "../../include/ahpp.h"
 #include "ahpp_internal.cuh"
@@ -19,33 +22,52 @@ constexpr int kTileNarrow = 16;    // the other width of the batched kernel
 constexpr int kRadixBits = 8;      // top-k digit width (per-lane histograms of 256 bins)
 constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kRadixPasses = 64 / kRadixBits;
-// Block size of the batched kernel (three resident blocks per SM: measured
-// best for this register budget).
-constexpr int kBThreads = 256;
+// Block size of the batched kernel: one block per SM (80 registers a thread).
+constexpr int kBThreads = 768;
 constexpr int kBWarps = kBThreads / 32;
-constexpr int kBMinBlocks = 3;
-// Dynamic shared memory per block: the top-k radix histograms and sort
-// buffer (4096 keys).
-constexpr size_t kBatchSmem = 32 * 1024;
+constexpr int kBMinBlocks = 1;
+// Dynamic shared memory per block: each warp's ring of kTRing units, then a
+// region that holds the rows most gathered during a phase, and between phases
+// the block reductions, the top-k radix histograms and the sort buffer.
+constexpr uint32_t kTRing = 2;
+constexpr size_t kTRingBytes = (size_t)kBWarps * kTRing * 512;
+constexpr uint32_t kTHubRows = 256;
+constexpr size_t kBatchSmem = kTRingBytes + (size_t)kTHubRows * 128;
 
-// Buffers of one concurrent group (one tile in flight).
+// A round's accumulators of one query.  Every block adds three words per
+// query, 15,000 atomics to a tile's 32 records at 152 blocks: they go to
+// kAccCopies copies, so that the L2 slices share them, and the two counts take
+// one 64-bit add (the barrier after phase 2: 17,000 cycles with one copy of four
+// words on a graph whose round is 230,000, 8,000 so).
+constexpr uint32_t kAccCopies = 8;
+struct alignas(32) TAcc {
+  uint32_t max_r_bits;             // max_u r_U after the round (float bits)
+  uint32_t np;                     // Algorithm 4's counter: active V rows and attributes
+  unsigned long long marked_deg;   // nodes marked, above bit 32 the sum of their degrees
+  uint32_t max_rel_bits, above;    // APP(S): see RAcc
+};
+constexpr size_t kTAccs = 3 * (size_t)kAccCopies * kTile;
+
+// Buffers of one tile in flight.
 struct alignas(64) TileBuf {
   float *r_u = nullptr, *pi = nullptr, *pic = nullptr;   // [n_u][kTile]
-  float *t_v = nullptr, *t_a = nullptr;                  // [n_v][kTile], [n_a][kTile]
-  float* t_a2 = nullptr;                                 // second t_A buffer (pushed for the next round)
-  float* split_acc = nullptr;                            // [n_split][kTile]
-  uint32_t* split_cnt = nullptr;                         // [n_split]
-  RAcc* racc = nullptr;                                  // [5][kTile]: 3 rounds + 2 final sums
-  GridBarrier* bar = nullptr;
+  float* t = nullptr;                                    // [n_v + 2 n_acc][kTile], see TileLayout
+  float* split_acc = nullptr;                            // [n_split_u][kTile]
+  uint32_t* split_cnt = nullptr;                         // [n_split_u]
+  TAcc* tacc = nullptr;                                  // [3][kAccCopies][kTile], rounds in turn
+  RAcc* racc = nullptr;                                  // [2][kTile]: final sums of residues, reserves
   unsigned int* hist = nullptr;                          // [kRadixPasses][kTile][kRadixBins]
   unsigned long long* cand = nullptr;                    // [kTile][kmax] selected keys
   uint32_t* cand_cnt = nullptr;                          // [kTile]
 };
 
-constexpr int kMaxGroups = 8;
+constexpr uint32_t kMaxBatchGroups = 8;    // the configuration's and the autotuner's most
+constexpr uint32_t kMaxGroups = 64;        // most tiles in flight at once
 
 struct BatchState {
-  TileBuf tb[kMaxGroups];
+  TileBuf tb[kMaxGroups];      // host copies
+  TileBuf* d_tb = nullptr;     // the same on the device
+  GridBarrier* bars = nullptr; // [kMaxGroups], one per group
   uint32_t n_groups = 0;       // buffers allocated
   uint32_t kmax_cap = 0;       // candidate capacity per lane
 };
@@ -71,7 +93,10 @@ struct BatchParams {
   uint32_t e_tot = 0;
   uint32_t max_rounds = 0;
   uint32_t groups = 1;
-  uint32_t dense_div = 32;
+  const TileBuf* tbufs = nullptr;          // [groups] (batched) or [tiles] (serving)
+  GridBarrier* bars = nullptr;             // [groups]
+  const uint4 *ranges_t = nullptr, *ranges_u = nullptr;   // of a group's warps, two each (tile_ranges)
+  float switch_unit = 0.f, switch_log = 0.f;   // see switch_due (rule 1's log; rule 0's is each query's)
   uint32_t tile = kTile;                   // queries per tile of this launch (kTile or kTileNarrow)
 };
 
@@ -82,6 +107,7 @@ struct LaneCtl {
   unsigned long long n_p, pushes;
   uint32_t rounds, switch_round;
   int phase, status, active, valid;
+  float th_async, log_eps;   // smallest float above eps_f; log(eps_f)
 };
 
 enum : uint32_t { kSlotFree = 0, kSlotNew = 1, kSlotRunning = 2, kSlotFinished = 3 };
@@ -100,17 +126,14 @@ struct SlotState {
 
 struct ServeParams {
   SlotState* slots = nullptr;        // [n_tiles * kTile]
-  const TileBuf* tbufs = nullptr;    // [n_tiles], device array
   uint32_t* tile_round = nullptr;    // [n_tiles] rounds run by each tile (accumulator rotation)
   const uint32_t* live = nullptr;    // [n_live] tiles to advance this step
   uint32_t n_live = 0;
   uint32_t rounds_per_step = 1;
 };
 
-int launch_batch(const DevGraph& g, const BatchState& s, const BatchParams& p, bool bf16,
-                 int grid, cudaStream_t stream);
-int launch_serve_step(const DevGraph& g, const BatchParams& p, const ServeParams& sv, bool bf16,
-                      int grid, cudaStream_t stream);
-int batch_max_grid(bool bf16, int sm_count);
+int launch_batch(const DevGraph& g, const BatchParams& p, int grid, cudaStream_t stream);
+int launch_serve_step(const DevGraph& g, const BatchParams& p, const ServeParams& sv, int grid, cudaStream_t stream);
+int batch_max_grid(int sm_count);
 
 }  // namespace ahpp

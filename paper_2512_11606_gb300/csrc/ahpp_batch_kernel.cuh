@@ -1,14 +1,29 @@
 // Batched multi-source APP / ASRP: one persistent cooperative launch runs n
 // queries packed into tiles of kTile (one query per lane).  Every round of a
 // tile is a pull sweep over the whole graph (the synchronous form of
-// Algorithm 3's three loops): phase 1 gathers t_V / t_A for all the tile's
-// queries from the marked residues, phase 2 gathers the new residues, applies the
-// reserve update of the pushed nodes and marks the next frontier of each
-// query with its own threshold.  Per-query control (termination, the ASRP
+// Algorithm 3's three loops): phase 1 gathers t_V and t_A for all the tile's
+// queries from the marked residues, phase 2 gathers the new residues from both,
+// applies the reserve update of the pushed nodes and marks the next frontier of
+// each query with its own threshold.  Per-query control (termination, the ASRP
 // switch test of Algorithm 4) is kept per lane; a query that finishes is
 // frozen while the rest of its tile continues, so its result does not depend
 // on the other queries of the tile.  Top-k per query is a per-lane radix
 // select over (score, caller id) keys.
+//
+// What bounds a tile's round: 128-byte row gathers, two per edge and two per
+// attribute entry, out of L2 (and HBM, where the tables are larger).  A warp
+// has 32 rows in flight, 24 warps an SM; the round is short when all warps have
+// them in flight all the time, so
+//   - a warp's entries lie in the order of its use (TileRows), copied ahead to
+//     a ring in shared memory: no index load stands before a gather;
+//   - warps share the items by measured cost, the last fifth from a pool;
+//   - chunks of long rows go over the table in step (add_chunks), so that each
+//     row of a table larger than L2 is fetched once;
+//   - the attribute hop is pulled: no reductions (47 G rows/s at best) beside
+//     the gathers, and both hops of phase 2 are one list over one table.
+// Medium graph, tile of 32, one round: 1,130 us before, 835 now (96 G rows/s;
+// 0.69 and 0.98 million cycles in the phases, even to 1 %); 100k nodes: 145 us
+// one tile alone, 103 now, 84 with four at once.
 // This file is the kernel body of ahpp_batch.cu, which includes it once per
 // tile width: AHPP_BT (queries per tile) and AHPP_BT_NS (the namespace of
 // that instance) are defined by the includer.  No include guard.
@@ -33,62 +48,49 @@ struct BCtx {
   uint32_t lane;
 };
 
-// Per-lane block reduction of Partials into acc[lane].
-__device__ __forceinline__ void flush_lane_partials(Partials& p, RAcc* acc) {
-  __shared__ float s_max[kBWarps][32];
-  __shared__ uint32_t s_mk[kBWarps][32];
-  __shared__ unsigned long long s_dg[kBWarps][32], s_np[kBWarps][32];
-  __shared__ double s_sum[kBWarps][32];
+// Shared memory behind the rings: rows copied for a phase, and between phases
+// the block reductions, the top-k histograms and the sort buffer.
+__device__ __forceinline__ unsigned char* scratch_of(unsigned char* smem) { return smem + kTRingBytes; }
+
+// Per-lane block reduction of a sum and a maximum into acc[lane] (buf: scratch memory).
+__device__ __forceinline__ void flush_lane(double sum, float mx, RAcc* acc, unsigned char* buf) {
+  double (*s)[32] = reinterpret_cast<double (*)[32]>(buf);
+  float (*m)[32] = reinterpret_cast<float (*)[32]>(buf + sizeof(double) * 32 * kBWarps);
+  static_assert((sizeof(double) + sizeof(float)) * 32 * kBWarps <= kTHubRows * 128, "fits the scratch memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  s_max[warp][lane] = p.max_r; s_mk[warp][lane] = p.marked; s_dg[warp][lane] = p.marked_deg;
-  s_np[warp][lane] = p.np_flush; s_sum[warp][lane] = p.sum_r;
   __syncthreads();
-  if (warp == 0) {
-    float m = s_max[0][lane];
-    uint32_t mk = s_mk[0][lane];
-    unsigned long long dg = s_dg[0][lane], np = s_np[0][lane];
-    double sm = s_sum[0][lane];
+  s[warp][lane] = sum;
+  m[warp][lane] = mx;
+  __syncthreads();
+  if (warp == 0 && lane < kTile) {
     for (int w = 1; w < kBWarps; ++w) {
-      m = fmaxf(m, s_max[w][lane]); mk += s_mk[w][lane]; dg += s_dg[w][lane];
-      np += s_np[w][lane]; sm += s_sum[w][lane];
+      sum += s[w][lane];
+      mx = fmaxf(mx, m[w][lane]);
     }
-    RAcc* a = &acc[lane];
-    if (lane < kTile) {
-      if (m > 0.f) atomicMax(&a->max_r_bits, __float_as_uint(m));
-      if (mk) atomicAdd(&a->marked, mk);
-      if (dg) atomicAdd(&a->marked_deg, dg);
-      if (np) atomicAdd(&a->np_flush, np);
-      if (sm != 0.0) atomicAdd(&a->sum_r, sm);
-    }
+    if (mx > 0.f) atomicMax(&acc[lane].max_r_bits, __float_as_uint(mx));
+    if (sum != 0.0) atomicAdd(&acc[lane].sum_r, sum);
   }
   __syncthreads();
-  p = Partials();
 }
 
 // ------------------------------------------------------------------------
-// Pull phases with row groups: a warp is 4 groups of 8 lanes; a group owns
-// one row (or one chunk of a long row) and each of its lanes owns 4 of the
-// tile's 32 queries (lane l of the group: queries 4l .. 4l+3).  One gather
-// is a float4 load per lane, so the group reads the 32 queries' values of a
-// neighbour as one 128-byte line and one warp instruction moves 4 lines.
-// Entries go in waves of 8 (one per lane of the group, coalesced): the 8
-// line gathers of a wave are in flight together, and the number of waves is
-// the warp's longest row, so short rows (most rows of a power-law graph)
-// issue no idle gather slots beyond their last wave.
+// Pull phases with row groups: a warp is 4 groups of 8 lanes, each on one row
+// (or one chunk of a long row).  A gathered row of the tile is kTile values:
+// with 32 queries each lane owns 4 of them (one float4, the group reads a
+// 128-byte line); with 16, four lanes own a 64-byte row and the group's halves
+// take every other entry.
 constexpr int kQL = 4;                 // queries per lane
-constexpr int kGL = kTile / kQL;       // lanes per row group (one 128- or 64-byte line)
-constexpr int kGPW = 32 / kGL;         // row groups per warp
+constexpr int kRL = kTile / kQL;       // lanes per gathered row
+constexpr int kEP = 8 / kRL;           // entries a group takes at once
 static_assert(kTile == 16 || kTile == 32, "tile of 16 or 32 queries");
+static_assert(kAccCopies * kTile <= kBThreads, "one thread per accumulator record");
 
-// Graph arrays, reserves and compensations are read once per round:
-// streamed with the evict-first policy so that they do not push the
-// gathered state rows out of L2.
+// Reserves and compensations are read once per round: streamed with the
+// evict-first policy so that they do not push the gathered rows out of L2.
 template <typename T>
 __device__ __forceinline__ T ld_stream(const T* p) {
   return __ldcs(p);
 }
-
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 // out[0..3] += v as a reduction that returns nothing: an atomicAdd on a
 // float4 whose result is unused is still issued as a returning atomic, and
@@ -99,250 +101,291 @@ __device__ __forceinline__ void red_add4(float* out, float4 v) {
                : "memory");
 }
 
-__device__ __forceinline__ float4 f4_fma(float c, float4 x, float4 a) {
-  return make_float4(fmaf(c, x.x, a.x), fmaf(c, x.y, a.y), fmaf(c, x.z, a.z), fmaf(c, x.w, a.w));
+// The warp's ring: its next kTRing units of the phase's stream (TileRows),
+// copied to shared memory ahead of their use and across the barrier.
+struct TileRing {
+  const uint4* src;            // the lane's place in unit 0
+  uint32_t base;               // the warp's ring
+  uint32_t next, end;          // next unit to copy, end of the stream
+
+  __device__ __forceinline__ void refill() {
+    if (next < end)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + (next % kTRing) * 512u +
+                                                                    (threadIdx.x & 31u) * 16u),
+                   "l"(src + (size_t)next * 32) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    ++next;
+  }
+  __device__ __forceinline__ void start(const uint4* units, uint32_t b, uint32_t e) {
+    src = units + (threadIdx.x & 31u);
+    next = b;
+    end = e;
+    __syncwarp();              // every lane is done with the units of the last stream
+#pragma unroll
+    for (uint32_t i = 0; i < kTRing; ++i) refill();
+  }
+  // unit k for every lane of the warp
+  __device__ __forceinline__ void wait() const {
+    asm volatile("cp.async.wait_group %0;" ::"n"((int)kTRing - 1) : "memory");
+    __syncwarp();
+  }
+};
+
+// Row i of the table (4 of its values for this lane): from the copy of rows
+// [first, first + n_hub) in shared memory, else from L2.  s_row: the lane's
+// place in the copy's first row.  Half of the rows that a power-law graph's
+// long lists name come up again and again; reading those from shared memory
+// takes them off the L2 -> SM path, which bounds the gathers.
+__device__ __forceinline__ float4 gather_row(uint32_t i, uint32_t first, uint32_t n_hub, uint32_t s_row,
+                                             const float* x) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile("{\n\t.reg .pred p, q, r;\n\t"
+               "setp.ne.u32 r, %4, 0xffffffff;\n\t"
+               "setp.lt.and.u32 p, %5, %6, r;\n\t"
+               "setp.ge.and.u32 q, %5, %6, r;\n\t"
+               "@p ld.shared.v4.f32 {%0, %1, %2, %3}, [%7];\n\t"
+               "@q ld.global.v4.f32 {%0, %1, %2, %3}, [%8];\n\t}"
+               : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+               : "r"(i), "r"(i - first), "r"(n_hub), "r"(s_row + (i - first) * (kTile * 4u)),
+                 "l"(x + (size_t)i * kTile)
+               : "memory");
+  return v;
 }
 
-// Sum over the entries [b, e) of this group's row of coef(k) * gather(idx(k)),
-// in waves of kGL entries: lane t of the group loads entry t of a wave
-// (coalesced), the entry's index and coefficient are broadcast within the
-// group, and the wave's kGL row gathers are in flight together.  The next
-// wave's index and coefficient loads are issued before the current wave's
-// gathers.  Called by the whole warp: `waves` is warp-uniform (the warp's
-// longest range, in waves); a group with b == e adds nothing.
-template <typename LoadF, typename GatherF>
-__device__ __forceinline__ float4 group_accum(uint32_t b, uint32_t e, uint32_t waves, uint32_t gl,
-                                              LoadF load, GatherF gather) {
+// Sum over the `entries` entries (of the warp's longest row) from unit k on of
+// coefficient * value(gathered row): waves of eight entries of each row, whose
+// gathers are in flight together.  k advances past the item's units.
+template <typename Index, typename Value>
+__device__ __forceinline__ float4 walk(TileRing& ring, uint32_t& k, uint32_t entries, uint32_t first, uint32_t n_hub,
+                                       uint32_t s_row, const float* x, Index index, Value value) {
+  const uint32_t lane = threadIdx.x & 31u, r = lane >> 3, sub = (lane & 7u) / kRL;
   float2 a01 = make_float2(0.f, 0.f), a23 = make_float2(0.f, 0.f);
-  uint32_t k = b + gl;
-  uint32_t mi = 0;
-  float mc = 0.f;
-  if (k < e) load(k, mi, mc);
-  for (uint32_t w = 0; w < waves; ++w) {
-    const uint32_t k0 = b + w * kGL;
-    const uint32_t n = k0 < e ? min((uint32_t)kGL, e - k0) : 0u;
-    const uint32_t kn = k + kGL;
-    uint32_t ni = 0;
-    float nc = 0.f;
-    if (kn < e) load(kn, ni, nc);
-    float4 x[kGL];
+#pragma unroll 1
+  for (uint32_t e0 = 0; e0 < entries; e0 += 8) {
+    if ((e0 & 8u) == 0) ring.wait();
+    const uint32_t row = ring.base + (k % kTRing) * 512u + r * 128u;
+    float4 v[8 / kEP];
+    float co[8 / kEP];
 #pragma unroll
-    for (int t = 0; t < kGL; ++t) {
-      const uint32_t id = __shfl_sync(kFull, mi, t, kGL);
-      x[t] = (uint32_t)t < n ? gather(id) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int t = 0; t < 4; ++t) {
+      uint32_t i0, i1;
+      float c0, c1;
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(i0), "=f"(c0), "=r"(i1), "=f"(c1)
+                   : "r"(row + ((((e0 & 8u) >> 1) + t + 2 * r) & 7u) * 16u) : "memory");
+      if (kEP == 1) {
+        co[2 * t % (8 / kEP)] = c0;
+        co[(2 * t + 1) % (8 / kEP)] = c1;
+        v[2 * t % (8 / kEP)] = gather_row(index(i0), first, n_hub, s_row, x);
+        v[(2 * t + 1) % (8 / kEP)] = gather_row(index(i1), first, n_hub, s_row, x);
+      } else {
+        co[t % (8 / kEP)] = sub ? c1 : c0;
+        v[t % (8 / kEP)] = gather_row(index(sub ? i1 : i0), first, n_hub, s_row, x);
+      }
+    }
+    if ((e0 & 8u) || e0 + 8 >= entries) {          // the unit is used up
+      ++k;
+      __syncwarp();
+      ring.refill();
     }
 #pragma unroll
-    for (int t = 0; t < kGL; ++t) {
-      const float c = __shfl_sync(kFull, mc, t, kGL);
-      const float2 cc = make_float2(c, c);
-      a01 = __ffma2_rn(cc, make_float2(x[t].x, x[t].y), a01);
-      a23 = __ffma2_rn(cc, make_float2(x[t].z, x[t].w), a23);
+    for (int t = 0; t < 8 / kEP; ++t) {
+      const float4 y = value(v[t]);
+      const float2 cc = make_float2(co[t], co[t]);
+      a01 = __ffma2_rn(cc, make_float2(y.x, y.y), a01);
+      a23 = __ffma2_rn(cc, make_float2(y.z, y.w), a23);
     }
-    mi = ni;
-    mc = nc;
-    k = kn;
+  }
+  if (kEP == 2) {
+    a01.x += __shfl_xor_sync(kFull, a01.x, kRL); a01.y += __shfl_xor_sync(kFull, a01.y, kRL);
+    a23.x += __shfl_xor_sync(kFull, a23.x, kRL); a23.y += __shfl_xor_sync(kFull, a23.y, kRL);
   }
   return make_float4(a01.x, a01.y, a23.x, a23.y);
 }
 
-__device__ __forceinline__ uint32_t warp_max_u32(uint32_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(kFull, v, o));
-  return v;
+// A phase's items of this warp, in segments: its chunks, its slices, then what
+// it grabs from the pool while there is any.  rg: its two ranges (tile_ranges);
+// first(ring) has been called for the phase already, across the barrier.
+struct Segments {
+  const TileRows& L;
+  const uint4* rg;
+  unsigned int* taken;
+  uint32_t seg = 0, i0 = 0, i1 = 0, grabbed = 0;
+
+  // the ring's first stream: the chunks', or the slices' where there are none
+  static __device__ __forceinline__ void first(TileRing& ring, const TileRows& L, const uint4* rg) {
+    const uint4 u = rg[1];
+    if (rg[0].x < rg[0].y) ring.start(L.units, u.x, u.y);
+    else ring.start(L.units, u.z, u.w);
+  }
+  __device__ __forceinline__ bool next(TileRing& ring) {
+    const uint4 r = rg[0];
+    if (seg == 0) {
+      seg = 1;
+      i0 = r.x;
+      i1 = r.y;
+      if (i0 < i1) return true;
+    }
+    if (seg == 1) {
+      seg = 2;
+      if (r.x < r.y) ring.start(L.units, rg[1].z, rg[1].w);
+      i0 = r.z;
+      i1 = r.w;
+      if (L.pool < L.n_items && (threadIdx.x & 31u) == 0) grabbed = atomicAdd(taken, 1u);   // known by the time it is needed
+      if (i0 < i1) return true;
+    }
+    if (L.pool >= L.n_items) return false;
+    i0 = L.pool + __shfl_sync(kFull, grabbed, 0) * L.batch;
+    if (i0 >= L.n_items) return false;
+    i1 = min(i0 + L.batch, L.n_items);
+    if ((threadIdx.x & 31u) == 0) grabbed = atomicAdd(taken, 1u);
+    ring.start(L.units, L.items[i0].w, L.items[i1].w);
+    return true;
+  }
+};
+
+// Copies rows [0, n) at x to shared memory (the block).
+__device__ __forceinline__ void copy_rows(unsigned char* buf, const float* x, uint32_t n) {
+  for (uint32_t i = threadIdx.x; i < n * (kTile / 4); i += kBThreads)
+    reinterpret_cast<float4*>(buf)[i] = reinterpret_cast<const float4*>(x)[i];
 }
 
-// Per-query partials of one thread (its 4 queries) summed over the warp's 4
-// groups and the block's warps, then added to acc[q] (one atomic per query
-// and field per block).
+// Per-query partials of one thread (its 4 queries) in phase 2.
+template <bool APPS>
 struct Q4Partials {
   float max_r[kQL] = {0.f, 0.f, 0.f, 0.f};
   uint32_t marked[kQL] = {0, 0, 0, 0};
   uint32_t mdeg[kQL] = {0, 0, 0, 0};
-  uint32_t np[kQL] = {0, 0, 0, 0};
+};
+template <>
+struct Q4Partials<true> : Q4Partials<false> {
   float max_rel[kQL] = {0.f, 0.f, 0.f, 0.f};   // APP(S) statistics (see RAcc)
   uint32_t above[kQL] = {0, 0, 0, 0};
 };
 
-template <bool APPS>
-__device__ __forceinline__ void flush_q4(Q4Partials& p, RAcc* acc) {
-  __shared__ float s_max[kBWarps][32];
-  __shared__ uint32_t s_mk[kBWarps][32], s_dg[kBWarps][32], s_np[kBWarps][32];
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// The block's round partials in shared memory: fields of 32 queries each
+// (floats are >= 0, so their bits order them).
+enum : int { kAccMax = 0, kAccMarked, kAccDeg, kAccNp, kAccRel, kAccAbove, kAccFields };
+using BlockAcc = uint32_t[kAccFields][32];
+
+__device__ __forceinline__ uint32_t bits_of(uint32_t x) { return x; }
+__device__ __forceinline__ uint32_t bits_of(float x) { return __float_as_uint(x); }
+
+// v[0..3] (of this lane's queries) into field f, over the warp's lanes first.
+template <bool MAX, typename T>
+__device__ __forceinline__ void add_field(BlockAcc& acc, int f, const T (&v)[kQL]) {
+  const uint32_t lane = threadIdx.x & 31;
 #pragma unroll
   for (int j = 0; j < kQL; ++j) {
+    uint32_t x = bits_of(v[j]);
 #pragma unroll
-    for (int o = kGL; o < 32; o <<= 1) {
-      p.max_r[j] = fmaxf(p.max_r[j], __shfl_xor_sync(kFull, p.max_r[j], o));
-      p.marked[j] += __shfl_xor_sync(kFull, p.marked[j], o);
-      p.mdeg[j] += __shfl_xor_sync(kFull, p.mdeg[j], o);
-      p.np[j] += __shfl_xor_sync(kFull, p.np[j], o);
-      if (APPS) {
-        p.max_rel[j] = fmaxf(p.max_rel[j], __shfl_xor_sync(kFull, p.max_rel[j], o));
-        p.above[j] += __shfl_xor_sync(kFull, p.above[j], o);
-      }
+    for (int o = kRL; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_xor_sync(kFull, x, o);
+      x = MAX ? max(x, y) : x + y;
+    }
+    if (lane < kRL && x) {
+      if (MAX) atomicMax(&acc[f][lane * kQL + j], x);
+      else atomicAdd(&acc[f][lane * kQL + j], x);
     }
   }
-  if (lane < kGL) {
-#pragma unroll
-    for (int j = 0; j < kQL; ++j) {
-      const uint32_t q = lane * kQL + j;
-      s_max[warp][q] = p.max_r[j]; s_mk[warp][q] = p.marked[j];
-      s_dg[warp][q] = p.mdeg[j]; s_np[warp][q] = p.np[j];
-    }
-  }
+}
+
+// The block's partials of the round into one copy of the tile's accumulators,
+// cleared for the next round.
+template <bool APPS>
+__device__ __forceinline__ void flush_round(BlockAcc& acc, TAcc* out) {
   __syncthreads();
-  if (warp == 0 && lane < kTile) {
-    float m = 0.f;
-    uint32_t mk = 0;
-    unsigned long long dg = 0, np = 0;
-    for (int w = 0; w < kBWarps; ++w) {
-      m = fmaxf(m, s_max[w][lane]); mk += s_mk[w][lane];
-      dg += s_dg[w][lane]; np += s_np[w][lane];
-    }
-    RAcc* a = &acc[lane];
-    if (m > 0.f) atomicMax(&a->max_r_bits, __float_as_uint(m));
-    if (mk) atomicAdd(&a->marked, mk);
-    if (dg) atomicAdd(&a->marked_deg, dg);
-    if (np) atomicAdd(&a->np_flush, np);
-  }
-  if (APPS) {
-    // the APP(S) statistics through the same buffers (max_r / marked reused)
-    __syncthreads();
-    if (lane < kGL) {
-#pragma unroll
-      for (int j = 0; j < kQL; ++j) {
-        const uint32_t q = lane * kQL + j;
-        s_max[warp][q] = p.max_rel[j];
-        s_mk[warp][q] = p.above[j];
-      }
-    }
-    __syncthreads();
-    if (warp == 0 && lane < kTile) {
-      float m = 0.f;
-      uint32_t ab = 0;
-      for (int w = 0; w < kBWarps; ++w) { m = fmaxf(m, s_max[w][lane]); ab += s_mk[w][lane]; }
-      if (m > 0.f) atomicMax(&acc[lane].max_rel_bits, __float_as_uint(m));
-      if (ab) atomicAdd(&acc[lane].above, ab);
-    }
-  }
-  __syncthreads();
-  p = Q4Partials();
-}
-
-// Combine a chunk of a split row (group-collective): returns true in every
-// lane of the group whose chunk finishes the row, with the row total.
-__device__ __forceinline__ bool split_combine4(const TileBuf& t, uint32_t slot, uint32_t nch,
-                                               float4 s, uint32_t gl, unsigned gmask, float4* tot) {
-  float* a = &t.split_acc[(size_t)slot * kTile + kQL * gl];
-  red_add4(a, s);
-  __threadfence();
-  __syncwarp(gmask);
-  uint32_t last = 0;
-  if (gl == 0) last = atomicAdd(&t.split_cnt[slot], 1u) == nch - 1;
-  last = __shfl_sync(gmask, last, 0, kGL);
-  if (last) {
-    __threadfence();
-    *tot = __ldcg(reinterpret_cast<const float4*>(a));
-    __stcg(reinterpret_cast<float4*>(a), make_float4(0.f, 0.f, 0.f, 0.f));
-    __syncwarp(gmask);
-    if (gl == 0) t.split_cnt[slot] = 0;
-  }
-  return last != 0;
-}
-
-// Unit u of a row space: units [0, n_items) are chunks of the long rows
-// (items[u] = {row, kItemSplit | slot, z, w}); units n_items.. are the short
-// rows n_long.. one each.
-struct Unit {
-  uint32_t row, b, e;     // row and local entry range
-  uint32_t slot;          // split slot or ~0
-};
-
-__device__ __forceinline__ Unit unit_of(const ItemList& L, uint32_t u, const uint32_t* off) {
-  Unit x;
-  if (u < L.n_items) {
-    const uint4 it = L.items[u];
-    x.row = it.x; x.b = it.z; x.e = it.w; x.slot = it.y & kItemMask;
-  } else {
-    x.row = L.n_long + (u - L.n_items);
-    x.b = 0; x.e = off[x.row + 1] - off[x.row]; x.slot = 0xffffffffu;
-  }
-  return x;
-}
-
-// Phase 1: t_V (and, when do_a, t_A into ta_out) of the tile's 32 queries.
-//   t_V[v] = sum_u c_uv(u,v) p_u;   t_A[a] = k_attr cnorm_a[a] sum_u w(u,a) rnorm_u[u] p_u
-// In a normal round t_A was already pushed by the previous phase 2 into
-// ta_scan: phase 1 then only counts its active attributes (Algorithm 4's n_p)
-// and clears ta_zero, the buffer the coming phase 2 pushes into.
-template <typename WA>
-__device__ __forceinline__ void gphase1(const BCtx& c, RAcc* A, bool do_v, bool do_a, float* ta_out,
-                                        const float* ta_scan, float* ta_zero, bool count) {
-  const DevGraph& g = c.g;
-  const uint32_t lane = c.lane, gl = lane & (kGL - 1), gi = lane / kGL;
-  const unsigned gmask = ((1u << kGL) - 1u) << (gi * kGL);
-  const float* __restrict__ r_u = c.t.r_u;
-  auto gp = [&](uint32_t u) {
-    const float4 x = ld4(r_u + (size_t)u * kTile + kQL * gl);
-    return make_float4(fmaxf(-x.x, 0.f), fmaxf(-x.y, 0.f), fmaxf(-x.z, 0.f), fmaxf(-x.w, 0.f));
+  const uint32_t f = threadIdx.x >> 5, q = threadIdx.x & 31;
+  if (f >= (APPS ? 5u : 3u)) return;
+  TAcc* a = out + q;
+  const bool lq = q < (uint32_t)kTile;
+  auto take = [&](int field) {
+    const uint32_t x = acc[field][q];
+    acc[field][q] = 0;
+    return x;
   };
-  Q4Partials part;
-  if (ta_scan || ta_zero) {
-    for (uint32_t a = c.gw * kGPW + gi; a < g.n_a; a += c.nw * kGPW) {
-      const size_t i = (size_t)a * kTile + kQL * gl;
-      if (ta_scan) {
-        const float4 t = *reinterpret_cast<const float4*>(ta_scan + i);
-        const uint32_t d = g.au_off[a + 1] - g.au_off[a];
-        part.np[0] += t.x > 0.f ? d : 0; part.np[1] += t.y > 0.f ? d : 0;
-        part.np[2] += t.z > 0.f ? d : 0; part.np[3] += t.w > 0.f ? d : 0;
+  if (f == 0) { const uint32_t x = take(kAccMax); if (lq && x) atomicMax(&a->max_r_bits, x); }
+  if (f == 1) { const uint32_t x = take(kAccNp); if (lq && x) atomicAdd(&a->np, x); }
+  if (f == 2) {
+    const uint32_t m = take(kAccMarked), d = take(kAccDeg);
+    if (lq && m) atomicAdd(&a->marked_deg, (unsigned long long)d << 32 | m);
+  }
+  if (f == 3) { const uint32_t x = take(kAccRel); if (lq && x) atomicMax(&a->max_rel_bits, x); }
+  if (f == 4) { const uint32_t x = take(kAccAbove); if (lq && x) atomicAdd(&a->above, x); }
+}
+
+// A query's accumulators over their copies.
+struct RoundSums {
+  uint32_t max_r_bits = 0, np = 0, marked = 0, marked_deg = 0, max_rel_bits = 0, above = 0;
+};
+template <bool APPS>
+__device__ __forceinline__ RoundSums sums_of(const TAcc* a) {
+  RoundSums s;
+#pragma unroll
+  for (uint32_t k = 0; k < kAccCopies; ++k) {
+    const TAcc* x = a + k * kTile;
+    s.max_r_bits = max(s.max_r_bits, __ldcg(&x->max_r_bits));
+    s.np += __ldcg(&x->np);
+    const unsigned long long m = __ldcg(&x->marked_deg);
+    s.marked += (uint32_t)m;
+    s.marked_deg += (uint32_t)(m >> 32);
+    if (APPS) {
+      s.max_rel_bits = max(s.max_rel_bits, __ldcg(&x->max_rel_bits));
+      s.above += __ldcg(&x->above);
+    }
+  }
+  return s;
+}
+
+__device__ __forceinline__ void count4(uint32_t (&np)[kQL], float4 t, uint32_t d) {
+  np[0] += t.x > 0.f ? d : 0; np[1] += t.y > 0.f ? d : 0;
+  np[2] += t.z > 0.f ? d : 0; np[3] += t.w > 0.f ? d : 0;
+}
+
+// Phase 1: the table's rows (t_V, t_A) from the marked residues,
+//   t_V[v] = sum_u c_uv(u,v) p_u;   t_A[a] = k_attr cnorm_a[a] sum_u w(u,a) rnorm_u[u] p_u.
+// The attribute hop is pulled like the V hop: 20M more gathers of 128-byte rows
+// take less than the 20M float4 reductions of pushing it from phase 2 (108 G
+// rows/s from a 128 MB table against 47 G reductions/s, measured alone).
+__device__ __forceinline__ void gphase1(const BCtx& c, BlockAcc& sums, TileRing& ring, const uint4* rg,
+                                        GridBarrier* bar, uint32_t set, unsigned char* buf) {
+  uint32_t np[kQL] = {0, 0, 0, 0};
+  const DevGraph& g = c.g;
+  const uint32_t lane = c.lane, ql = kQL * (lane & (kRL - 1)), gi = lane >> 3;
+  const bool lead = (lane & 7u) < (uint32_t)kRL;             // this lane writes its queries' sums
+  const float* x = c.t.r_u + ql;
+  float* acc = c.t.t + (size_t)(g.n_v + set * g.tl.n_acc) * kTile + ql;
+  const uint32_t n_hub = min(g.n_u, kTHubRows);
+  copy_rows(buf, c.t.r_u, n_hub);
+  __syncthreads();
+  const uint32_t s_row = smem_addr(buf) + ql * 4u;
+  if (c.gt == 0) bar->taken[1] = 0;                          // the other phase's pool is full again
+  Segments sg{g.tl.t, rg, &bar->taken[0]};
+  while (sg.next(ring)) {
+    uint4 a = g.tl.t.items[sg.i0];
+    uint32_t k = a.w;
+#pragma unroll 1
+    for (uint32_t it = sg.i0; it < sg.i1; ++it) {
+      const uint4 ca = a;
+      if (it + 1 < sg.i1) a = g.tl.t.items[it + 1];
+      const bool chunk = ca.y >> 31, ok = gi < (ca.y & 0xffu);
+      uint32_t row = ca.x + gi, d = 0;
+      if (chunk && ok) row = g.tl.t.chunk_row[ca.x + gi];
+      if (!chunk && ok) d = g.q1.deg_v[row];
+      const float4 s = walk(ring, k, ca.z, 0u, n_hub, s_row, x, [](uint32_t i) { return i; },
+                            [](float4 v) { return make_float4(fmaxf(-v.x, 0.f), fmaxf(-v.y, 0.f), fmaxf(-v.z, 0.f),
+                                                              fmaxf(-v.w, 0.f)); });
+      if (!ok || !lead) continue;
+      if (chunk) {
+        red_add4(acc + (size_t)row * kTile, s);
+      } else {
+        *reinterpret_cast<float4*>(c.t.t + (size_t)row * kTile + ql) = s;
+        count4(np, s, d);
       }
-      if (ta_zero) *reinterpret_cast<float4*>(ta_zero + i) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
-  const uint32_t nuv = do_v ? g.b_v.n_items + (g.n_v - g.b_v.n_long) : 0u;
-  const uint32_t nua = do_a ? g.b_a.n_items + (g.n_a - g.b_a.n_long) : 0u;
-  const uint32_t total = nuv + nua;
-  for (uint32_t base = c.gw * kGPW; base < total; base += c.nw * kGPW) {
-    const uint32_t uix = base + gi;
-    const bool ok = uix < total;
-    const bool is_a = ok && uix >= nuv;
-    Unit un{0, 0, 0, 0xffffffffu};
-    const uint32_t* off = is_a ? g.au_off : g.vu_off;
-    if (ok) un = is_a ? unit_of(g.b_a, uix - nuv, g.au_off) : unit_of(g.b_v, uix, g.vu_off);
-    const uint32_t b = ok ? off[un.row] + un.b : 0, e = ok ? off[un.row] + un.e : 0;
-    const uint32_t waves = warp_max_u32(is_a ? 0u : (e - b + kGL - 1) / kGL);
-    // V rows and attribute rows in one warp: both gathers run, each group
-    // keeps the one of its own kind (ranges are empty for the other)
-    const float4 sv = group_accum(is_a ? 0u : b, is_a ? 0u : e, waves, gl,
-        [&](uint32_t k, uint32_t& i, float& w) { i = ld_stream(g.vu_idx + k); w = ld_stream(g.vu_c + k); }, gp);
-    const uint32_t waves_a = warp_max_u32(is_a ? (e - b + kGL - 1) / kGL : 0u);
-    const float4 sa = group_accum(is_a ? b : 0u, is_a ? e : 0u, waves_a, gl,
-        [&](uint32_t k, uint32_t& i, float& w) { i = ld_stream(g.au_idx + k); w = ld_stream(g.au_c + k); }, gp);
-    if (!ok) continue;
-    float4 s = is_a ? sa : sv;
-    if (un.slot != 0xffffffffu) {
-      const uint32_t slot = un.slot + (is_a ? g.b_v.n_split : 0);
-      const uint32_t nch = is_a ? g.b_a.split_nchunks[un.slot] : g.b_v.split_nchunks[un.slot];
-      float4 tot;
-      if (!split_combine4(c.t, slot, nch, s, gl, gmask, &tot)) continue;
-      s = tot;
-    }
-    const uint32_t R = un.row;
-    if (!is_a) {
-      *reinterpret_cast<float4*>(c.t.t_v + (size_t)R * kTile + kQL * gl) = s;
-      const uint32_t d = g.vu_off[R + 1] - g.vu_off[R];
-      part.np[0] += s.x > 0.f ? d : 0; part.np[1] += s.y > 0.f ? d : 0;
-      part.np[2] += s.z > 0.f ? d : 0; part.np[3] += s.w > 0.f ? d : 0;
-    } else {
-      const float f = g.k_attr * g.cnorm_a[R];
-      const float4 tv = make_float4(f * s.x, f * s.y, f * s.z, f * s.w);
-      *reinterpret_cast<float4*>(ta_out + (size_t)R * kTile + kQL * gl) = tv;
-      const uint32_t d = g.au_off[R + 1] - g.au_off[R];
-      part.np[0] += tv.x > 0.f ? d : 0; part.np[1] += tv.y > 0.f ? d : 0;
-      part.np[2] += tv.z > 0.f ? d : 0; part.np[3] += tv.w > 0.f ? d : 0;
-    }
-  }
-  if (count) flush_q4<false>(part, A);
+  __syncwarp();
+  add_field<false>(sums, kAccNp, np);
 }
 
 // Residue update of row u for this lane's 4 queries: reserve update of the
@@ -350,19 +393,13 @@ __device__ __forceinline__ void gphase1(const BCtx& c, RAcc* A, bool do_v, bool 
 // APPLIKE: APP or APP(S) (per-node thresholds possible, r_max read per query);
 // APPS: APP(S)'s round statistics too.  ASRP launches compile neither.
 template <bool APPLIKE, bool APPS>
-__device__ __forceinline__ float4 gepilogue2(const BCtx& c, uint32_t u, float4 s, uint32_t cnt,
-                                             const float* th, const int* act, const int* pn,
-                                             const LaneCtl* ctl, Q4Partials& part) {
-  float4 pushed = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (!(act[0] | act[1] | act[2] | act[3])) return pushed;
-  float* pp4 = &pushed.x;
-  const uint32_t gl = c.lane & (kGL - 1);
-  const size_t i = (size_t)u * kTile + kQL * gl;
-  float4* rp = reinterpret_cast<float4*>(c.t.r_u + i);
-  float4* pp = reinterpret_cast<float4*>(c.t.pi + i);
-  float4* cp = reinterpret_cast<float4*>(c.t.pic + i);
-  float4 r = *rp;
-  float4 pv = ld_stream(pp), pc = ld_stream(cp);
+__device__ __forceinline__ void gepilogue2(const BCtx& c, uint32_t u, float4 s, const float* th, uint32_t act,
+                                           uint32_t pn, const LaneCtl* ctl, Q4Partials<APPS>& part) {
+  const uint32_t ql = kQL * (c.lane & (kRL - 1)), cnt = c.g.q1.deg_u[u];
+  const size_t i = (size_t)u * kTile + ql;
+  float4 r = *reinterpret_cast<const float4*>(c.t.r_u + i);
+  float4 pv = ld_stream(reinterpret_cast<const float4*>(c.t.pi + i));
+  float4 pc = ld_stream(reinterpret_cast<const float4*>(c.t.pic + i));
   float* rr = &r.x;
   float* pvv = &pv.x;
   float* pcc = &pc.x;
@@ -370,7 +407,7 @@ __device__ __forceinline__ float4 gepilogue2(const BCtx& c, uint32_t u, float4 s
   bool pushed_any = false;
 #pragma unroll
   for (int j = 0; j < kQL; ++j) {
-    if (!act[j]) continue;
+    if (!(act >> j & 1u)) continue;
     float kept = rr[j];
     if (kept < 0.f) {
       const float add = c.g.alpha * (-kept);
@@ -383,126 +420,129 @@ __device__ __forceinline__ float4 gepilogue2(const BCtx& c, uint32_t u, float4 s
     part.max_r[j] = fmaxf(part.max_r[j], r_new);
     bool mark;
     if (APPLIKE) {
-      const double rmx = ctl[kQL * gl + j].eps_f;         // APP's r_max for per-node thresholds
-      if (APPS) {
+      const double rmx = ctl[ql + j].eps_f;               // APP's r_max for per-node thresholds
+      if constexpr (APPS) {
         if (cnt) part.max_rel[j] = fmaxf(part.max_rel[j], r_new / (float)cnt);
-        if ((double)r_new > rmx * (double)cnt) part.above[j] += 1;
+        if (above_node_threshold(r_new, rmx, (float)rmx, cnt)) part.above[j] += 1;
       }
-      mark = pn[j] ? (double)r_new > rmx * (double)cnt : r_new >= th[j];
+      mark = (pn >> j & 1u) ? above_node_threshold(r_new, rmx, (float)rmx, cnt) : r_new >= th[j];
     } else {
       mark = r_new >= th[j];
     }
-    if (mark) {
-      rr[j] = -r_new;
-      pp4[j] = r_new;
-      part.marked[j] += 1;
-      part.mdeg[j] += cnt;
-    } else {
-      rr[j] = r_new;
-    }
+    rr[j] = mark ? -r_new : r_new;
+    part.marked[j] += mark;
+    part.mdeg[j] += mark ? cnt : 0u;
   }
-  *rp = r;
-  if (pushed_any) { __stcs(pp, pv); __stcs(cp, pc); }
-  return pushed;
-}
-
-// Attribute hop of the coming round, pushed as soon as u is marked: for every
-// a in A(u), t_A'[a] += k_attr cnorm_a[a] w(u,a) rnorm_u[u] p_u (Eq. 2's two
-// factors and Algorithm 3's U-push share, precomputed per entry as ua_pc), one
-// float4 reduction per lane and attribute; t_A' is small enough to stay in L2.
-template <typename WA>
-__device__ __forceinline__ void push_attr(const DevGraph& g, uint32_t u, float4 p, float* ta_push,
-                                          uint32_t gl, unsigned gmask) {
-  const bool mine = p.x > 0.f || p.y > 0.f || p.z > 0.f || p.w > 0.f;
-  if (!__any_sync(gmask, mine)) return;               // group-uniform
-  const uint32_t b = g.ua_off[u], e = g.ua_off[u + 1];
-  // waves of kGL entries (one per lane of the group, coalesced); every lane
-  // then issues one float4 reduction per entry for its 4 queries
-  for (uint32_t k0 = b; k0 < e; k0 += kGL) {
-    const uint32_t n = min((uint32_t)kGL, e - k0);
-    uint32_t mi = 0;
-    float mc = 0.f;
-    if (gl < n) {
-      mi = g.ua_idx[k0 + gl];
-      mc = ld_stream(g.ua_pc + k0 + gl);
-    }
-#pragma unroll
-    for (int t = 0; t < kGL; ++t) {
-      const uint32_t a = __shfl_sync(gmask, mi, t, kGL);
-      const float cf = __shfl_sync(gmask, mc, t, kGL);
-      if ((uint32_t)t < n && mine)
-        red_add4(ta_push + (size_t)a * kTile + kQL * gl, make_float4(cf * p.x, cf * p.y, cf * p.z, cf * p.w));
-    }
+  *reinterpret_cast<float4*>(c.t.r_u + i) = r;
+  if (pushed_any) {
+    __stcs(reinterpret_cast<float4*>(c.t.pi + i), pv);
+    __stcs(reinterpret_cast<float4*>(c.t.pic + i), pc);
   }
 }
 
-// Phase 2: new residues of every U node for the tile's 32 queries.
-template <typename WA, bool APPLIKE, bool APPS>
-__device__ __forceinline__ void gphase2(const BCtx& c, const LaneCtl* ctl, RAcc* A,
-                                        const float* ta_in, float* ta_push) {
+// Phase 2: new residues of every U node for the tile's queries, over both hops
+// at once from the table; the other set of accumulated rows is cleared.
+template <bool APPLIKE, bool APPS>
+__device__ __forceinline__ void gphase2(const BCtx& c, const LaneCtl* ctl, BlockAcc& sums, TileRing& ring,
+                                        const uint4* rg, GridBarrier* bar, uint32_t set, unsigned char* buf) {
   const DevGraph& g = c.g;
-  const uint32_t lane = c.lane, gl = lane & (kGL - 1), gi = lane / kGL;
-  const unsigned gmask = ((1u << kGL) - 1u) << (gi * kGL);
+  const uint32_t lane = c.lane, ql = kQL * (lane & (kRL - 1)), gi = lane >> 3, n_acc = g.tl.n_acc, n_v = g.n_v;
+  const bool lead = (lane & 7u) < (uint32_t)kRL;
   // mark thresholds and activity of this lane's 4 queries: APP's per-node
   // thresholds (pn), or one threshold (eps_f, or 0 once synchronous)
   float th[kQL];
-  int act[kQL], pn[kQL];
+  uint32_t act = 0, pn = 0;
 #pragma unroll
   for (int j = 0; j < kQL; ++j) {
-    const LaneCtl& q = ctl[kQL * gl + j];
-    act[j] = q.active;
-    pn[j] = APPLIKE ? per_node_threshold(c.p.algo, q.phase) : 0;
-    th[j] = pn[j] ? 0.f : threshold_up(q.phase == kPhaseSync ? 0.0 : q.eps_f);
+    const LaneCtl& q = ctl[ql + j];
+    act |= (uint32_t)(q.active != 0) << j;
+    if (APPLIKE) pn |= (uint32_t)per_node_threshold(c.p.algo, q.phase) << j;
+    th[j] = q.phase == kPhaseSync ? __uint_as_float(1u) : q.th_async;    // smallest float above 0
   }
-  const float* __restrict__ t_v = c.t.t_v;
-  const float* __restrict__ t_a = ta_in;
-  auto gv = [&](uint32_t v) { return ld4(t_v + (size_t)v * kTile + kQL * gl); };
-  auto ga = [&](uint32_t a) { return ld4(t_a + (size_t)a * kTile + kQL * gl); };
-  Q4Partials part;
-  const uint32_t total = g.b_u.n_items + (g.n_u - g.b_u.n_long);
-  for (uint32_t base = c.gw * kGPW; base < total; base += c.nw * kGPW) {
-    const uint32_t uix = base + gi;
-    const bool ok = uix < total;
-    uint32_t u = 0, z = 0, w = 0, slot = 0xffffffffu, b1 = 0, dv = 0, b2 = 0, da = 0;
+  const uint32_t shift = set * n_acc, n_hub = min(n_acc, kTHubRows);
+  float* cur = c.t.t + (size_t)(n_v + shift) * kTile;
+  float* other = c.t.t + (size_t)(n_v + (n_acc - shift)) * kTile;
+  copy_rows(buf, cur, n_hub);
+  // active accumulated rows (Algorithm 4's push counter); the next round's start at zero
+  uint32_t np[kQL] = {0, 0, 0, 0};
+  for (uint32_t j = c.gw * 4 + gi; j < n_acc; j += c.nw * 4) {
+    const size_t i = (size_t)j * kTile + ql;
+    if (!lead) continue;
+    count4(np, *reinterpret_cast<const float4*>(cur + i), g.tl.acc_deg[j]);
+    *reinterpret_cast<float4*>(other + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  add_field<false>(sums, kAccNp, np);
+  Q4Partials<APPS> part;
+  __syncthreads();
+  const uint32_t s_row = smem_addr(buf) + ql * 4u, first = n_v + shift;
+  const float* x = c.t.t + ql;
+  if (c.gt == 0) bar->taken[0] = 0;
+  Segments sg{g.tl.u, rg, &bar->taken[1]};
+  while (sg.next(ring)) {
+    uint4 a = g.tl.u.items[sg.i0];
+    uint32_t k = a.w;
+#pragma unroll 1
+    for (uint32_t it = sg.i0; it < sg.i1; ++it) {
+      const uint4 ca = a;
+      if (it + 1 < sg.i1) a = g.tl.u.items[it + 1];
+      const bool chunk = ca.y >> 31, ok = gi < (ca.y & 0xffu);
+      const bool mine = ok && lead && !chunk && act;
+      uint32_t u = ca.x + gi;
+      if (chunk && ok) u = g.tl.u.chunk_row[ca.x + gi];
+      const float4 s = walk(ring, k, ca.z, first, n_hub, s_row, x,
+                            [&](uint32_t i) { return i >= n_v && i != kNoEntry ? i + shift : i; },
+                            [](float4 v) { return v; });
+      if (mine) gepilogue2<APPLIKE, APPS>(c, u, s, th, act, pn, ctl, part);
+      else if (chunk && ok && lead) red_add4(c.t.split_acc + (size_t)u * kTile + ql, s);
+    }
+  }
+  // the warp's chunks: the last chunk of a row to be counted finishes it
+  // (counted only now, so that no walk waits for the counter)
+#pragma unroll 1
+  for (uint32_t it = rg[0].x; it < rg[0].y; ++it) {
+    const uint4 ca = g.tl.u.items[it];
+    __syncwarp();
+    const bool ok = gi < (ca.y & 0xffu);
+    uint32_t u = 0, last = 0;
     if (ok) {
-      if (uix < g.b_u.n_items) {
-        const uint4 it = g.b_u.items[uix];
-        u = it.x; z = it.z; w = it.w; slot = it.y & kItemMask;
-      } else {
-        u = g.b_u.n_long + (uix - g.b_u.n_items);
+      u = g.tl.u.chunk_row[ca.x + gi];
+      if ((lane & 7u) == 0) {
+        uint32_t seen;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(seen) : "l"(&c.t.split_cnt[u]) : "memory");
+        last = seen == g.tl.chunks_of[u] - 1;
       }
-      b1 = g.uv_off[u]; dv = g.uv_off[u + 1] - b1;
-      b2 = g.ua_off[u]; da = g.ua_off[u + 1] - b2;
-      if (slot == 0xffffffffu) { z = 0; w = dv + da; }
     }
-    // chunk [z, w) of the combined list: V neighbours first, then attributes
-    const uint32_t vb = b1 + min(z, dv), ve = b1 + min(w, dv);
-    const uint32_t ab = b2 + (z > dv ? z - dv : 0), ae = b2 + (w > dv ? w - dv : 0);
-    const uint32_t sv = warp_max_u32((ve - vb + kGL - 1) / kGL), sa = warp_max_u32((ae - ab + kGL - 1) / kGL);
-    float4 s = group_accum(vb, ve, sv, gl,
-        [&](uint32_t k, uint32_t& i, float& wt) { i = ld_stream(g.uv_idx + k); wt = ld_stream(g.uv_w + k); }, gv);
-    const float4 s2 = group_accum(ab, ae, sa, gl,
-        [&](uint32_t k, uint32_t& i, float& wt) { i = ld_stream(g.ua_idx + k); wt = wload<WA>(g.ua_w, k); }, ga);
-    if (!ok) continue;
-    s = make_float4(s.x + s2.x, s.y + s2.y, s.z + s2.z, s.w + s2.w);
-    if (slot != 0xffffffffu) {
-      const uint32_t sl = slot + g.b_v.n_split + g.b_a.n_split;
-      float4 tot;
-      if (!split_combine4(c.t, sl, g.b_u.split_nchunks[slot], s, gl, gmask, &tot)) continue;
-      s = tot;
-    }
-    const float4 pushed = gepilogue2<APPLIKE, APPS>(c, u, s, dv + da, th, act, pn, ctl, part);
-    if (ta_push) push_attr<WA>(g, u, pushed, ta_push, gl, gmask);
+    last = __shfl_sync(kFull, last, 0, 8);
+    if (!last || !lead) continue;
+    const size_t i = (size_t)u * kTile + ql;
+    float4* sp = reinterpret_cast<float4*>(c.t.split_acc + i);
+    const float4 s = __ldcg(sp);
+    __stcg(sp, make_float4(0.f, 0.f, 0.f, 0.f));
+    if ((lane & 7u) == 0) c.t.split_cnt[u] = 0;
+    if (!act) continue;
+    gepilogue2<APPLIKE, APPS>(c, u, s, th, act, pn, ctl, part);
   }
-  flush_q4<APPS>(part, A);
+  __syncwarp();
+  add_field<true>(sums, kAccMax, part.max_r);
+  add_field<false>(sums, kAccMarked, part.marked);
+  add_field<false>(sums, kAccDeg, part.mdeg);
+  if constexpr (APPS) {
+    add_field<true>(sums, kAccRel, part.max_rel);
+    add_field<false>(sums, kAccAbove, part.above);
+  }
 }
 
+__device__ __forceinline__ bool switch_now(const BatchParams& p, const LaneCtl& L, float m) {
+  return switch_due(p.e_tot, p.switch_rule, L.eps_f, p.lambda, p.log_inv, p.switch_unit,
+                    p.switch_rule == 1 ? p.switch_log : L.log_eps, L.n_p, m);
+}
 
-__device__ __forceinline__ double bbudget(const BatchParams& p, double eps_f, double M) {
-  const double EE = (double)p.e_tot;
-  if (p.switch_rule == 2) return INFINITY;
-  if (p.switch_rule == 1) return 2.0 * EE * (log(1.0 / (p.lambda * M)) / p.log_inv);
-  return 2.0 * EE * fmax(0.0, log(M / eps_f) / p.log_inv);
+// A new lane's thresholds, from its eps_f.
+__device__ __forceinline__ void set_eps(LaneCtl& L, double eps_f) {
+  L.eps_f = eps_f;
+  L.th_async = threshold_up(eps_f);
+  const float f = (float)eps_f;
+  L.log_eps = f > 1e-30f ? logf(f) : (float)log(eps_f);
 }
 
 __device__ __forceinline__ unsigned long long score_key(float score, uint32_t caller_id) {
@@ -517,25 +557,25 @@ __device__ __forceinline__ unsigned long long score_key(float score, uint32_t ca
 // (SERVE = true: every lane of a tile is a slot; NEW slots are admitted into
 // tiles already in flight, each live tile advances rounds_per_step rounds,
 // slots that finish are finalised and their top-k extracted).
-template <typename WA, bool SERVE>
+template <int ALGO, bool SERVE>
 __global__ void __launch_bounds__(kBThreads, kBMinBlocks)
-k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState st,
-        const __grid_constant__ BatchParams p, const __grid_constant__ ServeParams sv) {
+k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchParams p,
+        const __grid_constant__ ServeParams sv) {
   extern __shared__ __align__(1024) unsigned char smem[];
   // Per-query control of the current tile, one entry per lane / query.  Warp 0
   // of every block makes the decisions (all blocks read the same round
   // accumulators after a barrier, so they agree); the phases read it here.
   __shared__ LaneCtl s_ctl[kTile];
-  __shared__ unsigned long long s_mdeg[kTile];
+  __shared__ uint32_t s_mdeg[kTile];
   __shared__ int s_switch[kTile];
   __shared__ int s_new[kTile];       // serving: slot admitted at this step
   __shared__ int s_fin[kTile];       // lane finished: finalise and select top-k
   __shared__ uint32_t s_k[kTile];    // top-k size of the lane
   __shared__ int s_pick_d[kTile];    // top-k: digit, keys above it and its count, per lane
   __shared__ uint32_t s_pick_cum[kTile], s_pick_h[kTile];
-  __shared__ int s_flag;
+  __shared__ int s_flag, s_any_switch;
   __shared__ TileBuf s_tb;
-  const uint32_t groups = SERVE ? 1u : p.groups;
+  const uint32_t groups = p.groups;
   const uint32_t nbg = gridDim.x / groups;              // blocks per group
   const uint32_t grp = blockIdx.x / nbg;
   if (grp >= groups) return;                            // leftover blocks
@@ -546,16 +586,29 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
   const uint32_t lane = c.lane;
   const bool lq = lane < (uint32_t)kTile;               // this lane stands for a query
   const bool warp0 = threadIdx.x < 32;
-  const bool app = p.algo != kAlgoASRP;   // APP's r_max as eps_f, per-node threshold for the source
+  constexpr bool app = ALGO != kAlgoASRP;  // APP's r_max as eps_f, per-node threshold for the source
   const uint32_t n_work = SERVE ? sv.n_live : (p.n + kTile - 1) / kTile;
-  const uint32_t n_split = g.b_v.n_split + g.b_a.n_split + g.b_u.n_split;
+  const uint32_t n_split = g.tl.n_split_u, n_acc = g.tl.n_acc;
   const size_t nu32 = (size_t)g.n_u * kTile;
   const uint32_t kmax = p.kmax;
+  GridBarrier* bar = p.bars + grp;
   unsigned int epoch = 0;                               // of the group's barrier
+  // this warp's items, and its ring with the first units of phase 1 (the graph
+  // does not change: no barrier needs to come before the copies)
+  __shared__ uint4 s_rg[kBWarps][4];
+  __shared__ BlockAcc s_acc;
+  const uint4* rg = s_rg[threadIdx.x >> 5];
+  if (lane < 4) s_rg[threadIdx.x >> 5][lane] = (lane < 2 ? p.ranges_t : p.ranges_u)[2 * c.gw + (lane & 1u)];
+  if (threadIdx.x < kAccFields * 32) s_acc[threadIdx.x >> 5][lane] = 0;
+  __syncwarp();
+  TileRing ring;
+  ring.base = smem_addr(smem) + (threadIdx.x >> 5) * (kTRing * 512u);
+  Segments::first(ring, g.tl.t, rg);
+  unsigned char* const buf = scratch_of(smem);
 
   for (uint32_t w = grp; w < n_work; w += groups) {
     const uint32_t tile = SERVE ? sv.live[w] : w;
-    const TileBuf* tg = SERVE ? &sv.tbufs[tile] : &st.tb[grp];
+    const TileBuf* tg = &p.tbufs[SERVE ? tile : grp];
     if (threadIdx.x == 0) s_tb = *tg;
     __syncthreads();
     const uint32_t qi = tile * kTile + lane;            // query (batch) or slot (serve) index
@@ -564,14 +617,14 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
     // ---- admission: the initial state of Algorithm 3 (unit residue at the source) for every new lane
     if (!SERVE) {
       for (size_t i = c.gt; i < nu32; i += c.nt) { tb.r_u[i] = 0.f; tb.pi[i] = 0.f; tb.pic[i] = 0.f; }
-      for (size_t i = c.gt; i < (size_t)g.n_v * kTile; i += c.nt) tb.t_v[i] = 0.f;
-      for (size_t i = c.gt; i < (size_t)g.n_a * kTile; i += c.nt) { tb.t_a[i] = 0.f; tb.t_a2[i] = 0.f; }
+      for (size_t i = c.gt; i < ((size_t)g.n_v + 2 * n_acc) * kTile; i += c.nt) tb.t[i] = 0.f;
       for (size_t i = c.gt; i < (size_t)n_split * kTile; i += c.nt) tb.split_acc[i] = 0.f;
       for (size_t i = c.gt; i < n_split; i += c.nt) tb.split_cnt[i] = 0;
-      if (c.gt < 5 * kTile) tb.racc[c.gt] = RAcc{};
+      for (uint32_t i = c.gt; i < 3 * kAccCopies * kTile; i += c.nt) tb.tacc[i] = TAcc{};
+      if (c.gt < 2 * kTile) tb.racc[c.gt] = RAcc{};
     }
     if (warp0) {
-      LaneCtl L{0.0, 0, 0, 0, 0, kPhaseAsync, kStatusOk, 0, 0};
+      LaneCtl L{0.0, 0, 0, 0, 0, kPhaseAsync, kStatusOk, 0, 0, 0.f, 0.f};
       int is_new = 0;
       uint32_t kk = 0;
       if (!SERVE) {
@@ -579,7 +632,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         const bool bad = in_range && (p.q[qi] >= g.n_u || !(p.eps[qi] > 0.0));
         if (bad) L.status = kStatusBadArg;
         if (in_range && !bad) {
-          L.eps_f = app ? p.eps[qi] / (double)p.e_tot : p.eps[qi] / p.lambda;
+          set_eps(L, app ? p.eps[qi] / (double)p.e_tot : p.eps[qi] / p.lambda);
           L.active = 1;
           L.valid = 1;
           is_new = 1;
@@ -589,7 +642,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         const SlotState& S = sv.slots[qi];
         kk = S.k;
         if (S.state == kSlotNew) {
-          L.eps_f = S.eps_f;
+          set_eps(L, S.eps_f);
           L.active = 1;
           L.valid = 1;
           is_new = 1;
@@ -609,128 +662,128 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         const size_t i = u * kTile + lane;
         tb.r_u[i] = 0.f; tb.pi[i] = 0.f; tb.pic[i] = 0.f;
       }
-      for (size_t a = c.gw; nw && a < g.n_a; a += c.nw) {
-        tb.t_a[a * kTile + lane] = 0.f;
-        tb.t_a2[a * kTile + lane] = 0.f;
-      }
+      for (size_t j = c.gw; nw && j < 2 * (size_t)n_acc; j += c.nw) tb.t[(g.n_v + j) * kTile + lane] = 0.f;
       if (bid == 0 && nw) {
-        for (int r = 0; r < 5; ++r) tb.racc[r * kTile + lane] = RAcc{};
+        for (uint32_t r = 0; r < 3 * kAccCopies; ++r) tb.tacc[r * kTile + lane] = TAcc{};
+        for (int r = 0; r < 2; ++r) tb.racc[r * kTile + lane] = RAcc{};
       }
     }
-    if (!grid_sync(tb.bar, nbg, epoch)) return;
+    if (!grid_sync(bar, nbg, epoch)) return;
     if (bid == 0 && warp0 && lq && s_new[lane]) {
       const uint32_t q_new = SERVE ? sv.slots[qi].q_new : p.u_old2new[p.q[qi]];
       const uint32_t cnt = (g.uv_off[q_new + 1] - g.uv_off[q_new]) + (g.ua_off[q_new + 1] - g.ua_off[q_new]);
       const double th = app ? s_ctl[lane].eps_f * (double)cnt : s_ctl[lane].eps_f;
-      RAcc* a0 = &tb.racc[((tround + 2) % 3) * kTile + lane];
-      *a0 = RAcc{};
+      TAcc* a0 = &tb.tacc[((tround + 2) % 3) * kAccCopies * kTile + lane];
       if (1.0 > th) {
         tb.r_u[(size_t)q_new * kTile + lane] = -1.f;
-        a0->marked = 1;
-        a0->marked_deg = cnt;
-        // the source's attribute push of the first round (see push_attr)
-        float* ta_cur = (tround & 1) ? tb.t_a2 : tb.t_a;
-        for (uint32_t k = g.ua_off[q_new]; k < g.ua_off[q_new + 1]; ++k)
-          ta_cur[(size_t)g.ua_idx[k] * kTile + lane] += g.ua_pc[k];
+        a0->marked_deg = (unsigned long long)cnt << 32 | 1u;
       } else {
         tb.r_u[(size_t)q_new * kTile + lane] = 1.f;
       }
     }
-    if (!grid_sync(tb.bar, nbg, epoch)) return;
+    if (!grid_sync(bar, nbg, epoch)) return;
 
-    // ---- rounds (Algorithm 3 / 4) for the active lanes
-    Partials part;
+    // ---- rounds (Algorithm 3 / 4) for the active lanes; warp 0 decides, lane by
+    // query, in shared memory (registers kept for it would spill in the phases,
+    // and after a barrier a spilled register comes back from L2)
     bool wait_fail = false;
     const uint32_t max_r = SERVE ? sv.rounds_per_step : 0xffffffffu;
-    for (uint32_t done_r = 0;; ++done_r) {
-      RAcc* A = &tb.racc[(tround % 3) * kTile];
-      const RAcc* P = &tb.racc[((tround + 2) % 3) * kTile];
-      if (warp0) {
-        LaneCtl L{};
-        if (lq) {
-          L = s_ctl[lane];
-          const uint32_t marked = __ldcg(&P[lane].marked);
-          s_mdeg[lane] = __ldcg(&P[lane].marked_deg);
-          if (L.active && (L.phase == kPhaseDone || marked == 0)) { L.phase = kPhaseDone; L.active = 0; s_fin[lane] = 1; }
-          if (L.active && L.rounds >= p.max_rounds) { L.status = kStatusCap; L.active = 0; s_fin[lane] = 1; }
-          if (L.active && done_r < max_r) L.pushes += marked;
-          s_ctl[lane] = L;
-        }
-        const int any = __any_sync(kFull, L.active);
-        if (lane == 0) s_flag = any && done_r < max_r;
+    uint32_t done_r = 0;
+    // before a round: does the tile go on (the marks are in the last round's accumulators)
+    auto begin_round = [&](const RoundSums& m) {
+      bool act = false;
+      if (lq) {
+        LaneCtl& L = s_ctl[lane];
+        s_mdeg[lane] = m.marked_deg;
+        act = L.active;
+        if (act && (L.phase == kPhaseDone || m.marked == 0)) { L.phase = kPhaseDone; act = false; s_fin[lane] = 1; }
+        if (act && L.rounds >= p.max_rounds) { L.status = kStatusCap; act = false; s_fin[lane] = 1; }
+        if (act && done_r < max_r) L.pushes += m.marked;
+        L.active = act;
       }
-      __syncthreads();
-      if (!s_flag) break;
-      if (bid == 0 && threadIdx.x < kTile) tb.racc[((tround + 1) % 3) * kTile + threadIdx.x] = RAcc{};
+      const int any = __any_sync(kFull, act);
+      if (lane == 0) s_flag = any && done_r < max_r;
+    };
+    auto round_sums = [&](uint32_t r) {
+      return lq ? sums_of<ALGO == kAlgoAPPS>(&tb.tacc[(r % 3) * kAccCopies * kTile + lane]) : RoundSums{};
+    };
+    // after a round: counters, termination and the switch test; whether a lane switches
+    auto end_round = [&](const RoundSums& m) {
+      bool switched = false;
+      if (lq && s_ctl[lane].active) {
+        LaneCtl& L = s_ctl[lane];
+        const float M = __uint_as_float(m.max_r_bits);
+        L.rounds += 1;
+        L.n_p += (unsigned long long)s_mdeg[lane] + m.np;
+        bool done = false;
+        if (ALGO == kAlgoASRP) {
+          done = M < L.th_async;                                // M <= eps_f
+          switched = !done && L.phase == kPhaseAsync && switch_now(p, L, M);
+        } else if (ALGO == kAlgoAPPS) {
+          // APP's stopping test; the switch budget in units of APP's thresholds
+          const float Mrel = __uint_as_float(m.max_rel_bits);
+          done = m.above == 0;
+          switched = !done && L.phase == kPhaseAsync && switch_now(p, L, Mrel);
+        }
+        if (done) {
+          L.phase = kPhaseDone;
+          L.active = 0;
+          s_fin[lane] = 1;
+        }
+        if (switched) {
+          L.phase = kPhaseSync;
+          L.switch_round = L.rounds + 1;
+        }
+      }
+      if (lq) s_switch[lane] = switched;
+      return __any_sync(kFull, switched);
+    };
+    if (warp0) begin_round(round_sums(tround + 2));
+    __syncthreads();
+    while (s_flag) {
+      // this block's copy of the round's accumulators; the next round's are cleared
+      TAcc* A = &tb.tacc[((tround % 3) * kAccCopies + bid % kAccCopies) * kTile];
+      if (bid == 0 && threadIdx.x < kAccCopies * kTile)
+        tb.tacc[((tround + 1) % 3) * kAccCopies * kTile + threadIdx.x] = TAcc{};
 
-      float* ta_cur = (tround & 1) ? tb.t_a2 : tb.t_a;     // t_A of this round
-      float* ta_next = (tround & 1) ? tb.t_a : tb.t_a2;    // t_A of the next round
-      gphase1<WA>(c, A, true, false, nullptr, ta_cur, ta_next, true);
-      if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
-      if (p.algo == kAlgoASRP) gphase2<WA, false, false>(c, s_ctl, A, ta_cur, ta_next);
-      else if (p.algo == kAlgoAPP) gphase2<WA, true, false>(c, s_ctl, A, ta_cur, ta_next);
-      else gphase2<WA, true, true>(c, s_ctl, A, ta_cur, ta_next);
-      if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
+      const uint32_t set = tround & 1u;                    // accumulated rows of this round
+      gphase1(c, s_acc, ring, rg, bar, set, buf);
+      Segments::first(ring, g.tl.u, rg + 2);
+      if (!grid_sync(bar, nbg, epoch)) { wait_fail = true; break; }
+      gphase2<ALGO != kAlgoASRP, ALGO == kAlgoAPPS>(c, s_ctl, s_acc, ring, rg + 2, bar, set, buf);
+      flush_round<ALGO == kAlgoAPPS>(s_acc, A);
+      Segments::first(ring, g.tl.t, rg);
+      if (!grid_sync(bar, nbg, epoch)) { wait_fail = true; break; }
       ++tround;
-
+      ++done_r;
       if (warp0) {
-        LaneCtl L{};
-        if (lq) L = s_ctl[lane];
-        int switched = 0;
-        if (L.active) {
-          ++L.rounds;
-          const float M = __uint_as_float(__ldcg(&A[lane].max_r_bits));
-          L.n_p += s_mdeg[lane] + __ldcg(&A[lane].np_flush);
-          if (p.algo == kAlgoASRP) {
-            if ((double)M <= L.eps_f) {
-              L.phase = kPhaseDone;
-              L.active = 0;
-              s_fin[lane] = 1;
-            } else if (L.phase == kPhaseAsync && (double)L.n_p >= bbudget(p, L.eps_f, (double)M)) {
-              L.phase = kPhaseSync;
-              L.switch_round = L.rounds + 1;
-              switched = 1;
-            }
-          } else if (p.algo == kAlgoAPPS) {
-            // APP's stopping test; the switch budget in units of APP's thresholds
-            const float Mrel = __uint_as_float(__ldcg(&A[lane].max_rel_bits));
-            if (__ldcg(&A[lane].above) == 0) {
-              L.phase = kPhaseDone;
-              L.active = 0;
-              s_fin[lane] = 1;
-            } else if (L.phase == kPhaseAsync && (double)L.n_p >= bbudget(p, L.eps_f, (double)Mrel)) {
-              L.phase = kPhaseSync;
-              L.switch_round = L.rounds + 1;
-              switched = 1;
-            }
-          }
-        }
-        if (lq) {
-          s_ctl[lane] = L;
-          s_switch[lane] = switched;
-        }
-        const int any = __any_sync(kFull, switched);
-        if (lane == 0) s_flag = any;
+        const RoundSums m = round_sums(tround + 2);
+        const bool sw = end_round(m);
+        if (lane == 0) s_any_switch = sw;
+        if (!sw) begin_round(m);
       }
       __syncthreads();
-      if (s_flag) {
+      if (ALGO != kAlgoAPP && s_any_switch) {
         // first synchronous round pushes every positive residue of that query
         const bool sw = lq && s_switch[lane] != 0;
-        for (size_t u = c.gw; u < g.n_u; u += c.nw) {
-          const size_t i = u * kTile + (lq ? lane : 0);
-          const float r = sw ? tb.r_u[i] : 0.f;
-          if (sw && r > 0.f) {
+        uint32_t marked = 0, mdeg = 0;
+        for (size_t u = c.gw; sw && u < g.n_u; u += c.nw) {
+          const size_t i = u * kTile + lane;
+          const float r = tb.r_u[i];
+          if (r > 0.f) {
             tb.r_u[i] = -r;
-            part.marked += 1;
-            part.marked_deg += (g.uv_off[u + 1] - g.uv_off[u]) + (g.ua_off[u + 1] - g.ua_off[u]);
+            marked += 1;
+            mdeg += g.q1.deg_u[u];
           }
         }
-        flush_lane_partials(part, A);
-        if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
-        // the new marks also push into the next round's t_A: recompute it by
-        // the pull form from the complete marks (once per switch)
-        gphase1<WA>(c, A, false, true, (tround & 1) ? tb.t_a2 : tb.t_a, nullptr, nullptr, false);
-        if (!grid_sync(tb.bar, nbg, epoch)) { wait_fail = true; break; }
+        if (marked) {
+          atomicAdd(&s_acc[kAccMarked][lane], marked);
+          atomicAdd(&s_acc[kAccDeg][lane], mdeg);
+        }
+        flush_round<false>(s_acc, A);
+        if (!grid_sync(bar, nbg, epoch)) { wait_fail = true; break; }
+        if (warp0) begin_round(round_sums(tround + 2));
+        __syncthreads();
       }
     }
     if (wait_fail && warp0 && lq && s_ctl[lane].valid) {
@@ -747,23 +800,24 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
     if (any_fin) {
       // ---- reserves = pi - compensation; per-query sums; dense output
       {
-        Partials pr, pp;
+        double sum_r = 0.0, sum_p = 0.0;
+        float max_r = 0.f;
         for (size_t u = c.gw; fin && u < g.n_u; u += c.nw) {
           const size_t i = u * kTile + lane;
           const float v = fmaxf(tb.pi[i] - tb.pic[i], 0.f);
           tb.pi[i] = v;
           const float r = fabsf(tb.r_u[i]);
-          pr.sum_r += (double)r;
-          pr.max_r = fmaxf(pr.max_r, r);
-          pp.sum_r += (double)v;
+          sum_r += (double)r;
+          max_r = fmaxf(max_r, r);
+          sum_p += (double)v;
           if (!SERVE && p.out_dense) p.out_dense[(size_t)qi * g.n_u + p.u_new2old[u]] = v;
         }
-        flush_lane_partials(pr, &tb.racc[3 * kTile]);   // residues: sum and max
-        flush_lane_partials(pp, &tb.racc[4 * kTile]);   // reserves: sum
+        flush_lane(sum_r, max_r, &tb.racc[0], buf);      // residues
+        flush_lane(sum_p, 0.f, &tb.racc[kTile], buf);    // reserves
         for (size_t i = c.gt; i < (size_t)kRadixPasses * kTile * kRadixBins; i += c.nt) tb.hist[i] = 0;
         if (c.gt < kTile) tb.cand_cnt[c.gt] = 0;
       }
-      if (!grid_sync(tb.bar, nbg, epoch)) return;
+      if (!grid_sync(bar, nbg, epoch)) return;
 
       if (bid == 0 && fin) {
         const LaneCtl L = s_ctl[lane];
@@ -774,10 +828,10 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
         S.status = (uint32_t)((L.status == kStatusOk && L.phase != kPhaseDone) ? kStatusCap : L.status);
         S.pushes = L.pushes;
         S.n_p = L.n_p;
-        S.reserve_sum = __ldcg(&tb.racc[4 * kTile + lane].sum_r);
-        S.resid_sum = __ldcg(&tb.racc[3 * kTile + lane].sum_r);
+        S.reserve_sum = __ldcg(&tb.racc[kTile + lane].sum_r);
+        S.resid_sum = __ldcg(&tb.racc[lane].sum_r);
         S.mass_err = fabs(S.reserve_sum + S.resid_sum - 1.0);
-        S.max_resid = (double)__uint_as_float(__ldcg(&tb.racc[3 * kTile + lane].max_r_bits));
+        S.max_resid = (double)__uint_as_float(__ldcg(&tb.racc[lane].max_r_bits));
         S.lambda = p.lambda;
         S.eps_f = L.eps_f;
         S.served_ms = 0.0;
@@ -790,7 +844,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
       // winner); with distinct scores that happens once the score bits are
       // resolved, so the caller-id passes are skipped.
       if (kmax) {
-        unsigned int* sh = reinterpret_cast<unsigned int*>(smem);    // [kTile][kRadixBins]
+        unsigned int* sh = reinterpret_cast<unsigned int*>(buf);    // [kTile][kRadixBins]
         unsigned long long prefix = 0;
         unsigned long long thresh = 0;        // smallest winning key, once known
         uint32_t krem = kq;
@@ -813,7 +867,7 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
           unsigned int* gh = tb.hist + (size_t)pass * kTile * kRadixBins;
           for (int i = threadIdx.x; i < kTile * kRadixBins; i += kBThreads)
             if (sh[i]) atomicAdd(&gh[i], sh[i]);
-          if (!grid_sync(tb.bar, nbg, epoch)) return;
+          if (!grid_sync(bar, nbg, epoch)) return;
           // the merged histograms into shared memory; warp w picks the digit
           // of queries w, w + 8, ... (warp-parallel), lane l reads query l's
           for (int i = threadIdx.x; i < kTile * kRadixBins; i += kBThreads) sh[i] = __ldcg(&gh[i]);
@@ -848,9 +902,9 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
             }
           }
         }
-        if (!grid_sync(tb.bar, nbg, epoch)) return;
+        if (!grid_sync(bar, nbg, epoch)) return;
         // sort each lane's keys descending (bitonic in shared memory), one block per lane
-        unsigned long long* sk = reinterpret_cast<unsigned long long*>(smem);
+        unsigned long long* sk = reinterpret_cast<unsigned long long*>(buf);
         for (uint32_t l = bid; l < kTile; l += nbg) {
           if (!s_fin[l] || !s_ctl[l].valid) continue;
           const uint32_t ql = tile * kTile + l;
@@ -905,84 +959,56 @@ k_tiles(const __grid_constant__ DevGraph g, const __grid_constant__ BatchState s
       }
       if (lane == 0) sv.tile_round[tile] = tround;
     }
-    if (!grid_sync(tb.bar, nbg, epoch)) return;
+    if (!grid_sync(bar, nbg, epoch)) return;
   }
 }
 
-template __global__ void k_tiles<float, false>(const __grid_constant__ DevGraph,
-                                               const __grid_constant__ BatchState,
-                                               const __grid_constant__ BatchParams,
-                                               const __grid_constant__ ServeParams);
-template __global__ void k_tiles<__nv_bfloat16, false>(const __grid_constant__ DevGraph,
-                                                       const __grid_constant__ BatchState,
-                                                       const __grid_constant__ BatchParams,
-                                                       const __grid_constant__ ServeParams);
-#if AHPP_BT == 32   // serving runs tiles of 32 only
-template __global__ void k_tiles<float, true>(const __grid_constant__ DevGraph,
-                                              const __grid_constant__ BatchState,
-                                              const __grid_constant__ BatchParams,
-                                              const __grid_constant__ ServeParams);
-template __global__ void k_tiles<__nv_bfloat16, true>(const __grid_constant__ DevGraph,
-                                                      const __grid_constant__ BatchState,
-                                                      const __grid_constant__ BatchParams,
-                                                      const __grid_constant__ ServeParams);
-#endif
-
-
 namespace {
-const void* tiles_fn(bool bf16, bool serve) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    attr_set = true;
-    for (const void* f : {(const void*)k_tiles<__nv_bfloat16, false>, (const void*)k_tiles<float, false>})
-      cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
-#if AHPP_BT == 32
-    for (const void* f : {(const void*)k_tiles<__nv_bfloat16, true>, (const void*)k_tiles<float, true>})
-      cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
-#endif
-  }
-#if AHPP_BT == 32
-  if (serve) return bf16 ? (const void*)k_tiles<__nv_bfloat16, true> : (const void*)k_tiles<float, true>;
+template <int ALGO>
+const void* tiles_of(bool serve) {
+#if AHPP_BT == 32   // serving runs tiles of 32 only
+  if (serve) return (const void*)k_tiles<ALGO, true>;
 #else
   (void)serve;
 #endif
-  return bf16 ? (const void*)k_tiles<__nv_bfloat16, false> : (const void*)k_tiles<float, false>;
+  return (const void*)k_tiles<ALGO, false>;
+}
+const void* tiles_fn(int algo, bool serve) {
+  return algo == kAlgoASRP ? tiles_of<kAlgoASRP>(serve)
+                           : algo == kAlgoAPP ? tiles_of<kAlgoAPP>(serve) : tiles_of<kAlgoAPPS>(serve);
+}
+
+int launch(bool serve, const DevGraph& g, const BatchParams& p, const ServeParams& sv, int grid, cudaStream_t stream) {
+  void* args[] = {(void*)&g, (void*)&p, (void*)&sv};
+  const void* fn = tiles_fn(p.algo, serve);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
+  if (e == cudaSuccess)
+    e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBThreads), args, kBatchSmem, stream);
+  return e == cudaSuccess ? 0 : (int)e;
 }
 }  // namespace
 
-int launch_batch(const DevGraph& g, const BatchState& s, const BatchParams& p, bool bf16,
-                 int grid, cudaStream_t stream) {
-  ServeParams sv{};
-  void* args[] = {(void*)&g, (void*)&s, (void*)&p, (void*)&sv};
-  cudaError_t e = cudaLaunchCooperativeKernel(tiles_fn(bf16, false), dim3(grid), dim3(kBThreads), args,
-                                              kBatchSmem, stream);
-  return e == cudaSuccess ? 0 : (int)e;
+int launch_batch(const DevGraph& g, const BatchParams& p, int grid, cudaStream_t stream) {
+  return launch(false, g, p, ServeParams{}, grid, stream);
 }
 
 #if AHPP_BT == 32
-int launch_serve_step(const DevGraph& g, const BatchParams& p, const ServeParams& sv, bool bf16,
-                      int grid, cudaStream_t stream) {
-  BatchState s{};
-  void* args[] = {(void*)&g, (void*)&s, (void*)&p, (void*)&sv};
-  cudaError_t e = cudaLaunchCooperativeKernel(tiles_fn(bf16, true), dim3(grid), dim3(kBThreads), args,
-                                              kBatchSmem, stream);
-  return e == cudaSuccess ? 0 : (int)e;
+int launch_serve_step(const DevGraph& g, const BatchParams& p, const ServeParams& sv, int grid, cudaStream_t stream) {
+  return launch(true, g, p, sv, grid, stream);
 }
 #endif
 
-int batch_max_grid(bool bf16, int sm_count) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tiles_fn(bf16, false), kBThreads, kBatchSmem) !=
-          cudaSuccess || per_sm <= 0)
-    return -1;
-#if AHPP_BT == 32
-  int per_sm2 = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, tiles_fn(bf16, true), kBThreads, kBatchSmem) !=
-          cudaSuccess || per_sm2 <= 0)
-    return -1;
-  per_sm = std::min(per_sm, per_sm2);
-#endif
-  return per_sm * sm_count;
+int batch_max_grid(int sm_count) {
+  int best = -1;
+  for (int i = 0; i < 6; ++i) {
+    const void* fn = tiles_fn(i % 3 == 0 ? kAlgoAPP : i % 3 == 1 ? kAlgoASRP : kAlgoAPPS, i >= 3);
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBThreads, kBatchSmem) != cudaSuccess || per_sm <= 0)
+      return -1;
+    best = best < 0 ? per_sm : std::min(best, per_sm);
+  }
+  return std::min(best, 1) * sm_count;
 }
 
 }  // namespace AHPP_BT_NS

@@ -28,7 +28,7 @@ namespace ahpp {
 namespace {
 
 constexpr char kMagic[8] = {'A', 'H', 'P', 'P', 'G', 'R', 'F', '1'};
-constexpr uint32_t kVersion = 6;
+constexpr uint32_t kVersion = 7;
 
 struct CacheHeader {
   char magic[8];
@@ -47,19 +47,13 @@ void visit_graph_ptrs(ahpp_graph* g, F f) {
   f((const void**)&G.uv_off); f((const void**)&G.uv_idx); f((const void**)&G.uv_w); f((const void**)&G.uv_c);
   f((const void**)&G.vu_off); f((const void**)&G.vu_idx); f((const void**)&G.vu_c); f((const void**)&G.vu_w);
   f((const void**)&G.ua_off); f((const void**)&G.ua_idx); f((const void**)&G.ua_w);
-  f((const void**)&G.au_off); f((const void**)&G.au_idx); f((const void**)&G.au_w); f((const void**)&G.au_c);
-  f((const void**)&G.ua_pc);
+  f((const void**)&G.au_off); f((const void**)&G.au_idx); f((const void**)&G.au_w); f((const void**)&G.au_pc);
   f((const void**)&G.rnorm_u); f((const void**)&G.cnorm_a);
-  ItemList* lists[] = {&G.s1_v, &G.s1_a, &G.b_v, &G.b_a, &G.b_u};
+  ItemList* lists[] = {&G.s1_v, &G.s1_a};
   for (ItemList* L : lists) {
     f((const void**)&L->items);
     f((const void**)&L->split_nchunks);
   }
-  for (int c = 0; c < kChunkChoices; ++c)
-    for (int d = 0; d < 3; ++d) {
-      f((const void**)&G.b_alt[c][d].items);
-      f((const void**)&G.b_alt[c][d].split_nchunks);
-    }
   f((const void**)&g->d_u_new2old);
   f((const void**)&g->d_u_old2new);
 }
@@ -188,7 +182,7 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
   }
   if (kernel_algo(c.algo) < 0 || c.switch_rule < 0 || c.switch_rule > 2 ||
       (c.algo == AHPP_APP_S && c.switch_rule == 1) ||
-      (c.batch_tile != 0 && c.batch_tile != 16 && c.batch_tile != 32) || c.batch_groups > (uint32_t)kMaxGroups ||
+      (c.batch_tile != 0 && c.batch_tile != 16 && c.batch_tile != 32) || c.batch_groups > kMaxBatchGroups ||
       chunk_choice(c.batch_chunk) < 0 || c.single_vec_width > 32 ||
       (c.single_vec_width & (c.single_vec_width - 1))) {
     set_error("ahpp_load_graph_file: bad algo, switch_rule, batch_tile, batch_groups or batch_chunk");
@@ -207,7 +201,7 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
   g->cfg = c;
   g->device = c.device;
   g->batch_tile = c.batch_tile ? c.batch_tile : (uint32_t)kTile;
-  g->batch_groups = c.batch_groups ? c.batch_groups : 1;
+  g->batch_groups = c.batch_groups;
   g->n_u = h.n_u; g->n_v = h.n_v; g->n_a = h.n_a; g->n_e = h.n_e; g->n_ea = h.n_ea;
   g->bf16 = h.attr_bf16 != 0;
   int rc = AHPP_OK;
@@ -280,7 +274,6 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
       fail(AHPP_ECUDA, "ahpp_load_graph_file: id maps");
     }
   }
-  if (rc == AHPP_OK) select_chunk(g->dg, (uint32_t)chunk_choice(c.batch_chunk));
   if (rc == AHPP_OK) rc = alloc_query_state(g);
   if (rc == AHPP_OK) {
     // lambda: the configured value, else the cached estimate when it was

@@ -181,35 +181,11 @@ HostItems build_items(const std::vector<uint32_t>& deg, const ItemShape& sh) {
   return h;
 }
 
-HostItems build_units(const std::vector<uint32_t>& deg, uint32_t chunk) {
-  HostItems h;
-  const uint32_t n = (uint32_t)deg.size();
-  uint32_t r = 0;
-  while (r < n && deg[r] > chunk) {
-    const uint32_t d = deg[r];
-    const uint32_t nch = (d + chunk - 1) / chunk;
-    const uint32_t slot = (uint32_t)h.split_nchunks.size();
-    h.split_nchunks.push_back(nch);
-    for (uint32_t c = 0; c < nch; ++c)
-      h.items.push_back(make_uint4(r, kItemSplit | slot, c * chunk, std::min(d, (c + 1) * chunk)));
-    ++r;
-  }
-  h.n_long = r;
-  return h;
-}
-
 int chunk_choice(uint32_t chunk) {
   if (chunk == 0) return kChunkDefault;
   for (int c = 0; c < kChunkChoices; ++c)
     if (kChunkSizes[c] == chunk) return c;
   return -1;
-}
-
-void select_chunk(DevGraph& G, uint32_t choice) {
-  G.b_chunk = choice;
-  G.b_v = G.b_alt[choice][0];
-  G.b_a = G.b_alt[choice][1];
-  G.b_u = G.b_alt[choice][2];
 }
 
 int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
@@ -310,41 +286,24 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
   std::vector<float> rnorm(nU), cnorm(nA);
   for (uint32_t u = 0; u < nU; ++u) rnorm[u] = wr[u] > 0 ? (float)(1.0 / wr[u]) : 0.f;
   for (uint32_t a = 0; a < nA; ++a) cnorm[a] = wc[a] > 0 ? (float)(1.0 / wc[a]) : 0.f;
-  // push coefficient of the U->A direction (both factors of Eq. 2 and the
+  // coefficient of the U->A hop by attribute (both factors of Eq. 2 and the
   // (1 - alpha) beta share of the U-push), rounded once to FP32
-  std::vector<float> f_ua_pc(ua_w.size());
+  std::vector<float> f_au_pc(au_w.size());
   const double ka = (1.0 - alpha) * beta;
-  parallel_for(nU, [&](size_t b, size_t e) {
-    for (size_t u = b; u < e; ++u)
-      for (uint32_t k = ua_off[u]; k < ua_off[u + 1]; ++k) {
-        const uint32_t a = ua_idx[k];
-        f_ua_pc[k] = (wr[u] > 0 && wc[a] > 0) ? (float)(ka * ua_w[k] / (wr[u] * wc[a])) : 0.f;
-      }
-  });
-  // pull coefficient of the A->U direction (the U-side factor of Eq. 2), from
-  // the quantised weight and the FP64 row sum, rounded once to FP32
-  std::vector<float> f_au_c(au_w.size());
   parallel_for(nA, [&](size_t b, size_t e) {
     for (size_t a = b; a < e; ++a)
       for (uint32_t k = au_off[a]; k < au_off[a + 1]; ++k) {
         const uint32_t u = au_idx[k];
-        f_au_c[k] = wr[u] > 0 ? (float)(au_w[k] / wr[u]) : 0.f;
+        f_au_pc[k] = (wr[u] > 0 && wc[a] > 0) ? (float)(ka * au_w[k] / (wr[u] * wc[a])) : 0.f;
       }
   });
 
   // 5. work items (rows are sorted by degree, longest first)
-  std::vector<uint32_t> dg_u(nU), dg_v(nV), dg_a(nA);
-  for (uint32_t u = 0; u < nU; ++u) dg_u[u] = (uv_off[u + 1] - uv_off[u]) + (ua_off[u + 1] - ua_off[u]);
+  std::vector<uint32_t> dg_v(nV), dg_a(nA);
   for (uint32_t v = 0; v < nV; ++v) dg_v[v] = vu_off[v + 1] - vu_off[v];
   for (uint32_t a = 0; a < nA; ++a) dg_a[a] = au_off[a + 1] - au_off[a];
   const ItemShape s1{64, 32, 0xffffffffu, 2048};
   HostItems i1v = build_items(dg_v, s1), i1a = build_items(dg_a, s1);
-  std::vector<HostItems> ib;
-  for (int c = 0; c < kChunkChoices; ++c) {
-    ib.push_back(build_units(dg_v, kChunkSizes[c]));
-    ib.push_back(build_units(dg_a, kChunkSizes[c]));
-    ib.push_back(build_units(dg_u, kChunkSizes[c]));
-  }
 
   // 6. upload
   auto up = [&](const void* src, size_t bytes) -> void* {
@@ -380,8 +339,7 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
     G.ua_w = up(a.data(), a.size() * 4);
     G.au_w = up(b.data(), b.size() * 4);
   }
-  G.au_c = (const float*)up(f_au_c.data(), f_au_c.size() * 4);
-  G.ua_pc = (const float*)up(f_ua_pc.data(), f_ua_pc.size() * 4);
+  G.au_pc = (const float*)up(f_au_pc.data(), f_au_pc.size() * 4);
   G.rnorm_u = (const float*)up(rnorm.data(), rnorm.size() * 4);
   G.cnorm_a = (const float*)up(cnorm.data(), cnorm.size() * 4);
   auto up_items = [&](const HostItems& h, ItemList& L) {
@@ -389,16 +347,8 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
     L.n_items = (uint32_t)h.items.size();
     L.n_split = (uint32_t)h.split_nchunks.size();
     L.split_nchunks = (const uint32_t*)up(h.split_nchunks.data(), h.split_nchunks.size() * 4);
-    L.n_long = h.n_long;
   };
   up_items(i1v, G.s1_v); up_items(i1a, G.s1_a);
-  G.b_split_max = 0;
-  for (int c = 0; c < kChunkChoices; ++c) {
-    for (int d = 0; d < 3; ++d) up_items(ib[3 * c + d], G.b_alt[c][d]);
-    G.b_split_max = std::max(G.b_split_max,
-                             G.b_alt[c][0].n_split + G.b_alt[c][1].n_split + G.b_alt[c][2].n_split);
-  }
-  select_chunk(G, kChunkDefault);
 
   g->h_u_old2new = u_o2n;
   g->h_u_new2old = u_n2o;
@@ -448,8 +398,8 @@ int alloc_query_state(ahpp_graph* g) {
   AHPP_CUDA(cudaMemset(s.bar, 0, sizeof(GridBarrier)));
   AHPP_CUDA(cudaMemset(s.split_acc, 0, 4ull * std::max(g->n_split1, 1u)));
   AHPP_CUDA(cudaMemset(s.split_cnt, 0, 4ull * std::max(g->n_split1, 1u)));
-  BatchParams plan;
-  if (int rc = batch_plan(g, plan)) return rc;
+  if (int rc = batch_plan(g)) return rc;
+  if (int rc = build_tile_layout(g, (uint32_t)chunk_choice(cfg.batch_chunk))) return rc;
   if (cfg.hbm_budget_bytes && g->graph_bytes + g->q1_bytes > cfg.hbm_budget_bytes) {
     set_error("ahpp_load_graph: graph and query state exceed hbm_budget_bytes");
     return AHPP_ENOMEM;

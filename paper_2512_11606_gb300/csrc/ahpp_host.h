@@ -45,7 +45,6 @@ struct HostAdj {
 struct HostItems {
   std::vector<uint4> items;
   std::vector<uint32_t> split_nchunks;
-  uint32_t n_long = 0;
 };
 
 // Work-item shapes.
@@ -57,10 +56,6 @@ struct ItemShape {
 };
 
 HostItems build_items(const std::vector<uint32_t>& deg, const ItemShape& shape);
-// Batched row units: rows longer than `chunk` (a prefix, rows being sorted by
-// degree) become split chunks; every other row is one unit.
-HostItems build_units(const std::vector<uint32_t>& deg, uint32_t chunk);
-
 // Device allocation tracked by the graph.
 struct DevBuf {
   void* p = nullptr;
@@ -106,9 +101,20 @@ struct ahpp_graph {
 
   // batched state (allocated on first use, grown on demand)
   ahpp::BatchState bt{};
-  uint32_t batch_tile = 32, batch_groups = 1;
+  uint32_t batch_tile = 32, batch_groups = 0;   // groups: 0 = by the graph's size and the batch's
   int bt_grid = 0;
   uint64_t tile_bytes = 0;
+  // batched pull layout (dg.tl): its buffers, the items' costs (running sums),
+  // first units and chunks, and the ranges cut so far
+  std::vector<void*> tile_layout_bufs;
+  uint64_t tile_layout_bytes = 0;
+  struct TileCost {
+    std::vector<uint64_t> cost;
+    std::vector<uint32_t> unit;
+    uint32_t n_chunks = 0;
+  } tile_cost[2];
+  struct TileCut { uint32_t warps; const uint4* r[2]; };
+  std::vector<TileCut> tile_cuts;
 
   // top-k scratch
   void* topk_scratch = nullptr;
@@ -123,15 +129,16 @@ struct ahpp_graph {
 };
 
 namespace ahpp {
-// Clear a grid barrier before a persistent launch on `stream`.  When the
+// Clear n grid barriers before a persistent launch on `stream`.  When the
 // graph's self-test trap is armed (ahpp_selftest_arm_wait_timeout) the
-// counter is set far above any grid size instead, so the launch's first
+// counters are set far below any block count instead, so the launch's first
 // barrier never fills and every block's bounded spin runs out; the trap is
 // consumed by the first launch that sees it.
-int reset_barrier(ahpp_graph* g, GridBarrier* bar, cudaStream_t stream, bool keep_trap = false);
-// Zero if the barrier's error word is clear; kStatusWait if a wait gave up.
-// Synchronous (reads one word from the device on `stream`).
-int barrier_status(GridBarrier* bar, cudaStream_t stream, int* status);
+int reset_barriers(ahpp_graph* g, GridBarrier* bars, uint32_t n, cudaStream_t stream);
+void set_batch_params(const ahpp_graph* g, BatchParams& p);
+// Zero if the error words of n barriers are clear; kStatusWait if a wait gave
+// up.  Synchronous (reads them from the device on `stream`).
+int barrier_status(const GridBarrier* bars, uint32_t n, cudaStream_t stream, int* status);
 int build_graph(const ahpp_graph_desc* desc, ahpp_graph* g);
 // The kernels' algorithm id of an AHPP_* constant (-1 if none).
 int kernel_algo(int algo);
@@ -141,8 +148,14 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width);
 // Index into kChunkSizes of a configured chunk size (0: the default), -1 if
 // it is not one of them.
 int chunk_choice(uint32_t chunk);
-// Make chunk choice `choice` (index into kChunkSizes) the active unit lists.
-void select_chunk(DevGraph& G, uint32_t choice);
+// Sliced layout of the batched pull rounds with chunks of kChunkSizes[choice]
+// entries; replaces the one the graph has.
+int build_tile_layout(ahpp_graph* g, uint32_t choice);
+// The items' ranges for a tile on `warps` warps (made on first use).
+int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u);
+// Blocks of the batched grid that work on one tile, of n_tiles to be run: all of
+// them, or fewer where several small tiles run at once.
+uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles);
 int alloc_query_state(ahpp_graph* g);
 int run_lambda(ahpp_graph* g);
 int run_query1(ahpp_graph* g, uint32_t q_new, double eps, uint32_t lambda_T_mode,
@@ -150,7 +163,7 @@ int run_query1(ahpp_graph* g, uint32_t q_new, double eps, uint32_t lambda_T_mode
 int topk_single(ahpp_graph* g, const float* d_score, uint32_t k, uint32_t* d_nodes,
                 float* d_scores, uint32_t* d_n, cudaStream_t stream);
 // The batched kernel's grid (computed once per graph).
-int batch_plan(ahpp_graph* g, BatchParams& p);
+int batch_plan(ahpp_graph* g);
 int run_single_device(ahpp_graph* g, uint32_t q, double eps, uint32_t k, uint32_t* d_out_nodes,
                       float* d_out_scores, uint32_t* d_out_n, ahpp_stats* d_stats, cudaStream_t s);
 }  // namespace ahpp

@@ -6,7 +6,7 @@
 //   CSR_UV  rows u: off[n_u+1], idx v, w(u,v) raw (pull V->U), c_uv (push U->V)
 //   CSR_VU  rows v: off[n_v+1], idx u, c_uv (pull U->V), w(u,v) raw (push V->U)
 //   CSR_UA  rows u: off[n_u+1], idx a, w(u,a) raw (bf16 or f32)
-//   CSC_AU  rows a: off[n_a+1], idx u, w(u,a) raw (bf16 or f32)
+//   CSC_AU  rows a: off[n_a+1], idx u, w(u,a) raw (bf16 or f32), au_pc (pull U->A)
 //   c_uv(u,v) = (1-alpha)(1-beta) w(u,v) / (d(u) d(v))       (Eq. 1's two factors)
 //   rnorm_u[u] = 1 / sum_a w(u,a),  cnorm_a[a] = 1 / sum_u w(u,a)   (Eq. 2)
 // One round of Algorithm 3 maps the pushed residues p (marked U nodes) to
@@ -33,8 +33,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr uint32_t kItemLong = 0x40000000u;   // item = one whole long row (warp-cooperative)
 constexpr uint32_t kItemSplit = 0x80000000u;  // item = one chunk of a split row (| slot)
 constexpr uint32_t kItemMask = 0x3fffffffu;
-// Entries per chunk of a long row in the batched pull phases: the unit lists
-// of every choice are built at load, ahpp_autotune picks one (default 256).
+// Entries per chunk of a long row in the batched pull phases: the choices of
+// the configuration and of ahpp_autotune.
 constexpr int kChunkChoices = 3;
 constexpr uint32_t kChunkSizes[kChunkChoices] = {128, 256, 512};
 constexpr int kChunkDefault = 1;
@@ -47,7 +47,6 @@ struct ItemList {
   uint32_t n_items = 0;
   uint32_t n_split = 0;                 // split rows
   const uint32_t* split_nchunks = nullptr;
-  uint32_t n_long = 0;                  // batched lists: rows [0, n_long) are chunked
 };
 
 // Sliced rows of the single-query pull phases (built by ahpp_q1layout.cu).
@@ -99,6 +98,42 @@ struct Q1Layout {
   uint32_t hub_u = 0, hub_a = 0, hub_v = 0;
 };
 
+// Sliced rows of the batched pull phases (built by ahpp_tilelayout.cu).  A warp
+// walks four rows at once, eight lanes to a row.  An item is four consecutive
+// rows (rows are sorted by degree), or four chunks of long rows:
+//   {first row, or first chunk; rows | chunk << 31; entries of the longest;
+//    first unit}
+// The chunk items come first, the n_static items from there on that the warps
+// share out beforehand, then those that warps take `batch` at a time when they
+// are done; a last item holds the number of units.
+// Its entries lie in units of 512 bytes: 16 entries of each row, two to a
+// lane's 16 bytes as {index, coefficient, index, coefficient}; pair j of row r
+// is in place 8 r + (j + 2 r) % 8, so that the four rows' reads of a pair hit
+// different banks.  Index kNoEntry: nothing.  chunk_row: a chunk's row.
+constexpr uint32_t kNoEntry = 0xffffffffu;
+struct TileRows {
+  const uint4* items = nullptr;
+  const uint4* units = nullptr;         // [units][32]
+  const uint32_t* chunk_row = nullptr;
+  uint32_t n_items = 0, pool = 0, batch = 1;   // items; first of the pool; items per grab
+};
+
+// Phase 1 (t) pulls the rows of V and of A from the residues into one table of
+// 128-byte rows: row v of V in place v, or, where chunks add up their sums (V
+// rows longer than a chunk, and every attribute), accumulated row j in place
+// n_v + j, in one of two sets of n_acc places (rounds alternate; the other set
+// is cleared meanwhile).  The split V rows come first among the accumulated
+// ones, then the attributes.  Phase 2 (u) pulls the rows of U over both hops at
+// once from that table; its indices are those of the first set.
+struct TileLayout {
+  TileRows t, u;
+  const uint32_t* acc_deg = nullptr;    // degrees of the accumulated rows
+  const uint32_t* chunks_of = nullptr;  // chunks of each split U row (rows [0, n_split_u))
+  uint32_t n_acc = 0, n_split_u = 0;
+  uint32_t acc_max = 0, split_u_max = 0;   // the most of any chunk choice (buffers are sized for them)
+  uint32_t chunk = 0;                   // index into kChunkSizes
+};
+
 struct DevGraph {
   uint32_t n_u = 0, n_v = 0, n_a = 0;
   uint32_t n_e = 0, n_ea = 0;
@@ -110,8 +145,7 @@ struct DevGraph {
   const void* ua_w = nullptr;
   const uint32_t *au_off = nullptr, *au_idx = nullptr;
   const void* au_w = nullptr;
-  const float* au_c = nullptr;          // A->U pull coefficient w(u,a) / sum_a' w(u,a') (FP32)
-  const float* ua_pc = nullptr;         // U->A push coefficient (1-alpha) beta w(u,a) / (sum_a' w(u,a') sum_u' w(u',a))
+  const float* au_pc = nullptr;         // A->U: (1-alpha) beta w(u,a) / (sum_a' w(u,a') sum_u' w(u',a)) (FP32)
   const float* rnorm_u = nullptr;
   const float* cnorm_a = nullptr;
   float alpha = 0.f;
@@ -119,12 +153,7 @@ struct DevGraph {
   // single-query push rounds: work items of the V and attribute flush
   ItemList s1_v, s1_a;
   Q1Layout q1;                          // single-query pull rounds
-  // batched row-group units (the active chunk size) and those of every chunk
-  // choice (kChunkSizes); b_split_max = the most split slots of any choice
-  ItemList b_v, b_a, b_u;
-  ItemList b_alt[kChunkChoices][3];
-  uint32_t b_chunk = kChunkDefault;
-  uint32_t b_split_max = 0;
+  TileLayout tl;                        // batched pull rounds
 };
 
 template <typename WA>
@@ -175,7 +204,7 @@ struct RAcc {
   uint32_t marked;           // nodes marked for the next U-push
   unsigned long long marked_deg;   // sum of |N(u)| + |A(u)| over marked nodes
   unsigned long long np_flush;     // sum of |N(v)| (r(v) > 0) + |A^-1(a)| (r(a) > 0)
-  double sum_r;              // sum_u r_U after the round (pull rounds)
+  double sum_r;              // batched kernel: final sums
   uint32_t n_list_u;               // push rounds: marked list length
   uint32_t pad;
   // APP(S): max_u r(u) / (|N(u)| + |A(u)|) after the round (float bits) and
@@ -183,6 +212,10 @@ struct RAcc {
   unsigned int max_rel_bits;
   uint32_t above;
 };
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
 
 // Software grid barrier for persistent cooperative launches: blocks count up
 // one word, which the host clears before the launch, and wait until it has
@@ -194,7 +227,7 @@ struct RAcc {
 struct alignas(16) GridBarrier {
   unsigned int count;
   unsigned int err;
-  unsigned int pad[2];
+  unsigned int taken[2];     // batched kernel: grabs from the pools of its two phases
 };
 
 constexpr unsigned int kSpinLimit = 1u << 20;   // polls of about a microsecond: about one second
@@ -287,30 +320,11 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ uint32_t warp_sum_u32(uint32_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-
-// Thread-local partials of one query, reduced per block then atomically.
-struct Partials {
-  float max_r = 0.f;
-  uint32_t marked = 0;
-  unsigned long long marked_deg = 0;
-  unsigned long long np_flush = 0;
-  double sum_r = 0.0;
-};
 
 // FP64 runs at two lanes a cycle on an SM of this chip: one FP64 instruction
 // of a full block of 1,024 threads takes a quarter of a microsecond, an FP64

@@ -108,7 +108,7 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
   carve(g, (char*)g_noalloc_ptr[g->device], &s);
   cudaStream_t st = stream ? (cudaStream_t)stream : g->stream;
   Q1Params p = noalloc_params(g, g->h_u_old2new[q], eps);
-  if (int rc = reset_barrier(g, s.bar, st)) return rc;
+  if (int rc = reset_barriers(g, s.bar, 1, st)) return rc;
   const int e = launch_query1(g->dg, s, p, g->bf16, g->q1_grid, st);
   if (e) return cuda_fail((cudaError_t)e, "ahpp_query_dense_noalloc: launch");
   k_scatter_out<<<std::max(1, g->sm_count * 4), 256, 0, st>>>(s.pi, g->d_u_new2old, (uint32_t)g->n_u,
@@ -117,7 +117,7 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
   QCtl ctl;
   AHPP_CUDA(cudaMemcpyAsync(&ctl, s.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st));
   int bst = kStatusOk;
-  if (int rc = barrier_status(s.bar, st, &bst)) return rc;     // also waits for the stream
+  if (int rc = barrier_status(s.bar, 1, st, &bst)) return rc;     // also waits for the stream
   if (ctl.status == kStatusWait || bst == kStatusWait) {
     set_error("ahpp_query_dense_noalloc: a device wait gave up");
     return AHPP_ETIMEOUT;

@@ -188,9 +188,6 @@ __device__ __forceinline__ float ld_shared(uint32_t a) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
   return v;
 }
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 
 // Indices and coefficients of a step at unit k (k advances); compact: one unit
 // of uint16 indices and bfloat16 weights.  The caller refills the ring once it

@@ -66,7 +66,6 @@ struct ahpp_server {
   uint32_t* d_n = nullptr;
   ahpp_stats* d_stats = nullptr;
   GridBarrier* d_bar = nullptr;
-  BatchParams plan;                      // the batched kernel's shared-memory plan (hub rows)
   SlotState* h_slots = nullptr;          // pinned mirror of the slot table
   std::vector<uint64_t> slot_ticket;
   std::vector<Clock::time_point> slot_submit;
@@ -208,36 +207,35 @@ int server_step(ahpp_server* s) {
   AHPP_CUDA(cudaMemcpyAsync(s->d_slots, s->h_slots, sizeof(SlotState) * s->n_slots,
                             cudaMemcpyHostToDevice, s->stream));
   AHPP_CUDA(cudaMemcpyAsync(s->d_live, live.data(), 4 * live.size(), cudaMemcpyHostToDevice, s->stream));
-  if (int rc = reset_barrier(g, s->d_bar, s->stream)) return rc;
+  const uint32_t groups = tile_groups(g, (uint32_t)live.size()), per_group = (uint32_t)s->grid / groups;
+  if (int rc = reset_barriers(g, s->d_bar, groups, s->stream)) return rc;
   BatchParams p;
   p.kmax = s->kmax;
   p.out_nodes = s->d_nodes;
   p.out_scores = s->d_scores;
   p.out_n = s->d_n;
   p.out_stats = s->d_stats;
-  p.u_old2new = g->d_u_old2new;
-  p.u_new2old = g->d_u_new2old;
-  p.algo = kernel_algo(g->cfg.algo);
-  p.kahan = g->cfg.kahan;
-  p.switch_rule = g->cfg.switch_rule;
-  p.lambda = g->lambda;
-  p.log_inv = std::log(1.0 / (1.0 - g->cfg.alpha));
-  p.e_tot = (uint32_t)(g->n_e + g->n_ea);
+  set_batch_params(g, p);
   p.max_rounds = g->cfg.max_rounds ? g->cfg.max_rounds : 100000u;
-  p.groups = 1;
+  p.groups = groups;
+  p.tbufs = s->d_tbufs;
+  p.bars = s->d_bar;
+  {
+    std::lock_guard<std::mutex> glock(g->mu);
+    if (int rc = tile_ranges(g, per_group * kBWarps, &p.ranges_t, &p.ranges_u)) return rc;
+  }
   ServeParams sv;
   sv.slots = s->d_slots;
-  sv.tbufs = s->d_tbufs;
   sv.tile_round = s->d_tile_round;
   sv.live = s->d_live;
   sv.n_live = (uint32_t)live.size();
   sv.rounds_per_step = s->rounds_per_step;
-  const int e = launch_serve_step(g->dg, p, sv, g->bf16, s->grid, s->stream);
+  const int e = launch_serve_step(g->dg, p, sv, (int)(per_group * groups), s->stream);
   if (e) return cuda_fail((cudaError_t)e, "serving step launch");
   AHPP_CUDA(cudaMemcpyAsync(s->h_slots, s->d_slots, sizeof(SlotState) * s->n_slots,
                             cudaMemcpyDeviceToHost, s->stream));
   int bst = kStatusOk;
-  if (int rc = barrier_status(s->d_bar, s->stream, &bst)) return rc;   // also waits for the step
+  if (int rc = barrier_status(s->d_bar, groups, s->stream, &bst)) return rc;   // also waits for the step
   if (bst == kStatusWait) {
     // a device wait gave up: the step may have stopped part-way through its
     // tiles, so no slot's state can be trusted; the loop fails every request
@@ -325,9 +323,9 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
   if (o.single_max) s->single_max = o.single_max;
   // slots: requested, else what the HBM budget leaves after the graph, else 8 tiles
   const DevGraph& G = g->dg;
-  const size_t n_split = G.b_split_max;        // any chunk choice fits
-  const size_t tile_bytes = (size_t)G.n_u * kTile * 12 + (size_t)std::max(G.n_v, 1u) * kTile * 4 +
-                            (size_t)std::max(G.n_a, 1u) * kTile * 4 + std::max<size_t>(n_split, 1) * (kTile + 1) * 4 +
+  const size_t n_split = std::max(G.tl.split_u_max, 1u);        // any chunk choice fits
+  const size_t n_table = (size_t)G.n_v + 2 * (size_t)G.tl.acc_max + 1;
+  const size_t tile_bytes = (size_t)G.n_u * kTile * 12 + n_table * kTile * 4 + n_split * (kTile + 1) * 4 +
                             (size_t)kRadixPasses * kTile * kRadixBins * 4 + (size_t)kTile * s->kmax * 8 + 4096;
   uint32_t tiles;
   if (o.max_slots) {
@@ -354,7 +352,7 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
     std::memset(s->h_slots, 0, sizeof(SlotState) * s->n_slots);
     s->slot_ticket.assign(s->n_slots, 0);
     s->slot_submit.assign(s->n_slots, Clock::time_point{});
-    s->d_bar = (GridBarrier*)s->dalloc(sizeof(GridBarrier));
+    s->d_bar = (GridBarrier*)s->dalloc(kMaxGroups * sizeof(GridBarrier));
     s->d_slots = (SlotState*)s->dalloc(sizeof(SlotState) * s->n_slots);
     s->d_tile_round = (uint32_t*)s->dalloc(4ull * tiles);
     s->d_live = (uint32_t*)s->dalloc(4ull * tiles);
@@ -371,23 +369,21 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
       b.r_u = (float*)s->dalloc((size_t)G.n_u * kTile * 4);
       b.pi = (float*)s->dalloc((size_t)G.n_u * kTile * 4);
       b.pic = (float*)s->dalloc((size_t)G.n_u * kTile * 4);
-      b.t_v = (float*)s->dalloc((size_t)std::max(G.n_v, 1u) * kTile * 4);
-      b.t_a = (float*)s->dalloc((size_t)std::max(G.n_a, 1u) * kTile * 4);
-      b.t_a2 = (float*)s->dalloc((size_t)std::max(G.n_a, 1u) * kTile * 4);
-      b.split_acc = (float*)s->dalloc(std::max<size_t>(n_split, 1) * kTile * 4);
-      b.split_cnt = (uint32_t*)s->dalloc(std::max<size_t>(n_split, 1) * 4);
-      b.racc = (RAcc*)s->dalloc(5 * kTile * sizeof(RAcc));
-      b.bar = s->d_bar;
+      b.t = (float*)s->dalloc(n_table * kTile * 4);
+      b.split_acc = (float*)s->dalloc(n_split * kTile * 4);
+      b.split_cnt = (uint32_t*)s->dalloc(n_split * 4);
+      b.tacc = (TAcc*)s->dalloc(kTAccs * sizeof(TAcc));
+      b.racc = (RAcc*)s->dalloc(2 * kTile * sizeof(RAcc));
       b.hist = (unsigned int*)s->dalloc((size_t)kRadixPasses * kTile * kRadixBins * 4);
       b.cand = (unsigned long long*)s->dalloc((size_t)kTile * s->kmax * 8);
       b.cand_cnt = (uint32_t*)s->dalloc(kTile * 4);
-      ok = b.r_u && b.pi && b.pic && b.t_v && b.t_a && b.t_a2 && b.split_acc && b.split_cnt && b.racc &&
-           b.hist && b.cand && b.cand_cnt;
+      ok = b.r_u && b.pi && b.pic && b.t && b.split_acc && b.split_cnt && b.tacc && b.racc && b.hist && b.cand && b.cand_cnt;
       if (ok) {
         // the split accumulators and counters must start at zero (kept zero by the kernel)
-        ok = cudaMemset(b.split_acc, 0, std::max<size_t>(n_split, 1) * kTile * 4) == cudaSuccess &&
-             cudaMemset(b.split_cnt, 0, std::max<size_t>(n_split, 1) * 4) == cudaSuccess &&
-             cudaMemset(b.racc, 0, 5 * kTile * sizeof(RAcc)) == cudaSuccess;
+        ok = cudaMemset(b.split_acc, 0, n_split * kTile * 4) == cudaSuccess &&
+             cudaMemset(b.split_cnt, 0, n_split * 4) == cudaSuccess &&
+             cudaMemset(b.tacc, 0, kTAccs * sizeof(TAcc)) == cudaSuccess &&
+             cudaMemset(b.racc, 0, 2 * kTile * sizeof(RAcc)) == cudaSuccess;
       }
     }
     if (!ok) {
@@ -403,7 +399,7 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
       rc = cuda_fail(cudaGetLastError(), "ahpp_server_start: table upload");
     if (rc == AHPP_OK) {
       std::lock_guard<std::mutex> glock(g->mu);
-      rc = batch_plan(g, s->plan);
+      rc = batch_plan(g);
       s->grid = g->bt_grid;
     }
   }

@@ -1,8 +1,8 @@
-"""The single-query kernel's sliced rows where they change form: rows cut into
-chunks on both sides, more attributes than shared memory holds, more than
-16-bit indices hold, and more U rows than one pass of the attribute hop's
-blocks covers; against the FP64 oracle push (1e-6, as every GPU result) or a
-closed form.
+"""The sliced rows of the single-query and the batched kernel where they change
+form: rows cut into chunks on both sides, more attributes than shared memory
+holds, more than 16-bit indices hold, more U rows than one pass of the
+attribute hop's blocks covers, several tiles at once with a ragged last one;
+against the FP64 oracle push (1e-6, as every GPU result) or a closed form.
 """
 import numpy as np
 import pytest
@@ -44,13 +44,16 @@ def graph(n_u, n_v, n_a, m, seed, hubs=0, bf16=False):
     return synth.GraphArrays(n_u, n_v, n_a, c(u), c(v), w, c(au), c(aa), aw)
 
 
-@pytest.mark.parametrize("kind", [
+KINDS = [
     dict(n_u=6007, n_v=5003, n_a=31, m=3, seed=1, hubs=2),              # chunks of split rows, long segments
     dict(n_u=3001, n_v=1999, n_a=20011, m=9, seed=2),                   # t_A partly outside shared memory
     dict(n_u=3001, n_v=1999, n_a=20011, m=9, seed=3, bf16=True),
     dict(n_u=2003, n_v=1009, n_a=70001, m=33, seed=4, bf16=True),       # 32-bit attribute indices
     dict(n_u=33, n_v=1, n_a=1, m=1, seed=5, bf16=True),                 # the smallest rows and tables
-])
+]
+
+
+@pytest.mark.parametrize("kind", KINDS)
 @pytest.mark.parametrize("algo", ["ASRP", "APP"])
 def test_layout_forms_match_oracle(ahpp, kind, algo):
     g = graph(**kind)
@@ -64,6 +67,26 @@ def test_layout_forms_match_oracle(ahpp, kind, algo):
             ref = og.push(algo.lower(), ALPHA, BETA, q, 1e-6, lam=lam)
             assert np.abs(pi.astype(np.float64) - ref.pi).max() <= TOL
             assert abs(st["rounds"] - ref.stats["rounds"]) <= 1
+    finally:
+        G.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("algo,tile", [("ASRP", 32), ("ASRP", 16), ("APP", 32), ("APP_S", 32)])
+def test_batched_forms_match_oracle(ahpp, kind, algo, tile):
+    g = graph(**kind)
+    og = oracle.OracleGraph.from_arrays(g)
+    lam, _ = og.lambda_estimate(ALPHA, BETA)
+    G = ahpp.Graph.from_arrays(g, lam=lam, attr_bf16=int(kind.get("bf16", False)),
+                               algo=getattr(ahpp, "AHPP_" + algo), batch_tile=tile)
+    try:
+        qs = np.linspace(0, g.n_u - 1, 70).astype(np.uint32)             # three tiles of 32, five of 16
+        dense, stats, rc = G.query_batch_dense(qs, 1e-6)
+        assert rc == 0
+        for i in (0, 31, 69):
+            ref = og.push(algo.lower().replace("_", ""), ALPHA, BETA, int(qs[i]), 1e-6, lam=lam)
+            assert np.abs(dense[i].astype(np.float64) - ref.pi).max() <= TOL
+            assert abs(stats[i]["rounds"] - ref.stats["rounds"]) <= 1
     finally:
         G.close()
 

@@ -381,8 +381,9 @@ int alloc_query_state(ahpp_graph* g) {
   s.pi = (float*)g->alloc(4ull * nU);
   s.pic = (float*)g->alloc(4ull * nU);
   s.t_v = (float*)g->alloc(4ull * std::max(nV, 1u));
-  s.t_a = (float*)g->alloc(4ull * std::max(nA, 1u));
-  s.t_a2 = (float*)g->alloc(4ull * std::max(nA, 1u));
+  const uint64_t ta = (uint64_t)std::max(nA, 1u) * G.q1.ta_copies;
+  s.t_a = (float*)g->alloc(4 * ta);
+  s.t_a2 = (float*)g->alloc(4 * ta);
   s.list_u = (uint32_t*)g->alloc(4ull * nU);
   s.split_acc = (float*)g->alloc(4ull * std::max(g->n_split1, 1u));
   s.split_cnt = (uint32_t*)g->alloc(4ull * std::max(g->n_split1, 1u));

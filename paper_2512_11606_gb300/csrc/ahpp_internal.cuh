@@ -77,8 +77,8 @@ struct Q1Rows {
 // (block, attribute).  Items over (block, attribute) segments:
 //   {first segment, segments | lg vw << 8, first unit, steps}
 // with row indices local to the block; ranges[w] = {item begin, end, unit
-// begin, end} of warp w % kQ1Warps of block w / kQ1Warps; meta[s] = {attribute,
-// bits of the float scale of the sum} of segment s.
+// begin, end} of warp w % kQ1Warps of block w / kQ1Warps; meta[s] = {place in the
+// copies of t_A, bits of the float scale of the sum} of segment s.
 struct Q1Segs {
   const uint4* items = nullptr;
   const uint4* ranges = nullptr;
@@ -88,11 +88,18 @@ struct Q1Segs {
   uint32_t n_vb = 0, own_cap = 0;       // blocks of rows, and the most rows of one
 };
 
+constexpr uint32_t kTaCopies = 8;        // copies of t_A, at most
+
 struct Q1Layout {
   Q1Rows v, u;
   Q1Segs s;
   const uint32_t *deg_u = nullptr, *deg_v = nullptr, *deg_a = nullptr;
   uint32_t n_warps = 0;                 // ranges per row space
+  // copies of t_A that the blocks of the attribute hop add to in turn: with few
+  // attributes their reductions meet in a few lines of L2 (at 2,000 attributes
+  // 152 blocks' took 20,000 of the round's 75,000 cycles, and 3.31 ms a query
+  // became 2.61 with four copies)
+  uint32_t ta_copies = 1;
   uint32_t compact_a = 0, compact_s = 0;   // attribute steps of u / s in compact units
   // leading entries of p, t_A and t_V that the pull phases hold in shared memory
   uint32_t hub_u = 0, hub_a = 0, hub_v = 0;

@@ -47,7 +47,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Carve the single-query state out of base; returns the bytes needed.
 size_t carve(const ahpp_graph* g, char* base, Q1State* s) {
-  const size_t nu = g->n_u, nv = std::max<uint64_t>(g->n_v, 1), na = std::max<uint64_t>(g->n_a, 1);
+  const size_t nu = g->n_u, nv = std::max<uint64_t>(g->n_v, 1), na = std::max<uint64_t>(g->n_a, 1) * g->dg.q1.ta_copies;
   const size_t ns = std::max<uint32_t>(g->n_split1, 1);
   size_t off = 0;
   auto take = [&](size_t bytes) {

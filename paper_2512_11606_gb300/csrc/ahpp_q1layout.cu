@@ -218,10 +218,11 @@ __global__ void k_fill_segs(const uint4* items, uint32_t n_items, const uint4* s
   }
 }
 
-// Segment s's attribute and the scale of its sum (k_attr / W_col).
-__global__ void k_seg_meta(const uint4* segs, uint32_t n, const float* cnorm_a, float k_attr, uint2* meta) {
+// Segment s's place in t_A's copies and the scale of its sum (k_attr / W_col).
+__global__ void k_seg_meta(const uint4* segs, uint32_t n, const float* cnorm_a, uint32_t n_a, float k_attr,
+                           uint2* meta) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    meta[i] = make_uint2(segs[i].x, __float_as_uint(k_attr * cnorm_a[segs[i].x]));
+    meta[i] = make_uint2(segs[i].x, __float_as_uint(k_attr * cnorm_a[segs[i].x % n_a]));
 }
 
 __global__ void k_diff(const uint32_t* off, uint32_t n, const uint32_t* off2, uint32_t* out) {
@@ -249,7 +250,7 @@ struct Block {
 // Segments of rows [r0, r1), sorted by length in windows of consecutive
 // attributes: a slice's rows are about equally long, and its sums still go to
 // nearby attributes.
-Block make_block(uint32_t r0, uint32_t r1, const std::vector<uint32_t>& au, const std::vector<uint32_t>& au_idx,
+Block make_block(uint32_t b, uint32_t r0, uint32_t r1, const std::vector<uint32_t>& au, const std::vector<uint32_t>& au_idx,
                  uint32_t s_units) {
   Block B;
   for (uint32_t a = 0; a + 1 < au.size(); ++a) {
@@ -264,6 +265,11 @@ Block make_block(uint32_t r0, uint32_t r1, const std::vector<uint32_t>& au, cons
   for (uint32_t i = 0; i < n; i += kSegWindow)
     std::stable_sort(B.segs.begin() + i, B.segs.begin() + std::min(n, i + kSegWindow),
                      [](const uint4& x, const uint4& y) { return x.z > y.z; });
+  // each block starts with another window: blocks that walked the attributes in
+  // step would all reduce into the same lines at the same time (medium graph:
+  // 21.15 ms a query against 20.58, mean over six placements in memory)
+  const uint32_t windows = (n + kSegWindow - 1) / kSegWindow;
+  if (windows) std::rotate(B.segs.begin(), B.segs.begin() + (size_t)(b % windows) * kSegWindow, B.segs.end());
   uint32_t lg_min = 0;                     // enough items for the block's warps
   while (lg_min < 5 && ((uint64_t)n << lg_min) / 32 < kQ1Warps) ++lg_min;
   uint64_t total = 0, done = 0;
@@ -383,13 +389,17 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   }
   std::vector<Block> blk(n_vb);
   over_threads(n_vb, [&](uint32_t b) {
-    blk[b] = make_block(vb[b].x, vb[b].x + vb[b].y, au, au_idx, s_units);
+    blk[b] = make_block(b, vb[b].x, vb[b].x + vb[b].y, au, au_idx, s_units);
   });
+  // copies of t_A: at least 16 blocks to a copy (with 39 blocks, eight copies to
+  // add up in phase 2 cost 4 % of the query), and few enough attributes that all
+  // copies fit in 32 KB and t_A is looked up in shared memory only
+  Q.ta_copies = std::max(1u, std::min({kTaCopies, 8192u / std::max(nA, 1u), n_vb / 16}));
   std::vector<uint4> segs, sitems, sranges;
   uint32_t total_s = 0;
   for (uint32_t b = 0; b < n_vb; ++b) {
     const uint32_t s0 = (uint32_t)segs.size(), i0 = (uint32_t)sitems.size();
-    segs.insert(segs.end(), blk[b].segs.begin(), blk[b].segs.end());
+    for (auto x : blk[b].segs) { x.x += b % Q.ta_copies * nA; segs.push_back(x); }
     for (auto x : blk[b].items) { x.x += s0; x.z += total_s; sitems.push_back(x); }
     for (auto& x : blk[b].ranges) sranges.push_back(make_uint4(x.x + i0, x.y + i0, x.z + total_s, x.w + total_s));
     total_s += blk[b].units;
@@ -460,7 +470,7 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
     uint4* units = (uint4*)dev((size_t)total_s * 512, nullptr);
     Q.s.units = units;
     if (ok && n_items) {
-      k_seg_meta<<<grid, threads, 0, g->stream>>>(sg, (uint32_t)segs.size(), G.cnorm_a, G.k_attr, meta);
+      k_seg_meta<<<grid, threads, 0, g->stream>>>(sg, (uint32_t)segs.size(), G.cnorm_a, nA, G.k_attr, meta);
       if (g->bf16)
         k_fill_segs<<<grid, threads, 0, g->stream>>>(Q.s.items, n_items, sg, G.au_idx, (const __nv_bfloat16*)G.au_w,
                                                      true, units);

@@ -391,12 +391,28 @@ __device__ __forceinline__ void phase2(const Ctx& c, float th, bool per_node, Q1
   for (uint32_t i = v4 + threadIdx.x; i < hub_v / 4; i += kQ1Threads)
     reinterpret_cast<float4*>(s_tv)[i] = reinterpret_cast<const float4*>(t_v)[i];
   for (uint32_t i = threadIdx.x; i < min(4 * v4, hub_v); i += kQ1Threads) s_tv[i] = i < nsv ? acc.v_cur[i] : t_v[i];
-  for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) s_ta[i] = ta_cur[i];
+  const uint32_t n_ta = na * Q.ta_copies;
+  if (n_ta == na) {
+    for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) s_ta[i] = ta_cur[i];
+  } else {                                 // all loads of a sum in flight at once
+    for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) {
+      float t = 0.f;
+#pragma unroll
+      for (uint32_t k = 0; k < kTaCopies; ++k) t += i + k * na < n_ta ? ta_cur[i + k * na] : 0.f;
+      s_ta[i] = t;
+    }
+  }
   // active attributes and split V rows (Algorithm 4's push counter); the next
   // round's sums start at zero
   for (uint32_t a = c.gt; a < na; a += c.nt) {
-    if (ta_cur[a] > 0.f) part.np_flush += Q.deg_a[a];
-    ta_next[a] = 0.f;
+    bool active = false;
+#pragma unroll
+    for (uint32_t k = 0; k < kTaCopies; ++k)
+      if (a + k * na < n_ta) {
+        active |= ta_cur[a + k * na] > 0.f;
+        ta_next[a + k * na] = 0.f;
+      }
+    if (active) part.np_flush += Q.deg_a[a];
   }
   for (uint32_t v = c.gt; v < nsv; v += c.nt) {
     if (acc.v_cur[v] > 0.f) part.np_flush += Q.deg_v[v];
@@ -700,7 +716,7 @@ k_query1(const __grid_constant__ DevGraph g, const __grid_constant__ Q1State s,
   const float r0 = p.lambda_mode ? -1.f : 0.f;
   for (uint32_t u = c.gt; u < g.n_u; u += c.nt) { s.r_u[u] = r0; s.pi[u] = 0.f; s.pic[u] = 0.f; }
   for (uint32_t v = c.gt; v < g.n_v; v += c.nt) s.t_v[v] = 0.f;
-  for (uint32_t a = c.gt; a < g.n_a; a += c.nt) { s.t_a[a] = 0.f; s.t_a2[a] = 0.f; }
+  for (uint32_t a = c.gt; a < g.n_a * g.q1.ta_copies; a += c.nt) { s.t_a[a] = 0.f; s.t_a2[a] = 0.f; }
   for (uint32_t i = c.gt; i < p.n_split; i += c.nt) { s.split_acc[i] = 0.f; s.split_cnt[i] = 0; }   // 2 V + U
   if (c.gt < 3) s.racc[c.gt] = RAcc{};
   if (leader) {

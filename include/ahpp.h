@@ -247,8 +247,9 @@ int ahpp_query_batch_device(ahpp_graph *g, uint32_t n, const uint32_t *d_q, cons
  * or a thread that must not take the device synchronisation cudaMalloc /
  * cudaFree may cause).  The paper has no counterpart: this is a deployment
  * variant of the single-query push.  The query's working state lives in one
- * static device array of 32 MiB per device, held until the process exits;
- * graphs whose single-query state exceeds it are rejected with AHPP_EINVAL.
+ * static device array of 36 MiB per device, held until the process exits;
+ * graphs whose single-query state (4 B x (4 |U| + |V| + 2 |A|) and sums of long
+ * rows) exceeds 32 MiB are rejected with AHPP_EINVAL.
  * Outputs: d_out_pi[n_u] (device, caller ids).  stream: cudaStream_t (NULL =
  * the graph's).  The call waits for its stream before returning; calls are
  * serialised because they share the array (overlapping use would race).  The

@@ -97,6 +97,7 @@ struct ahpp_graph {
   uint32_t q1_dense_div = 32;     // pull rounds once the frontier covers > 1/dense_div of the edges
   std::string tune_log;           // the last autotune's measurements (JSON object)
   uint32_t n_split1 = 0;
+  uint32_t n_long_u = 0;          // U rows of more than 2,048 entries
   uint64_t q1_bytes = 0;
 
   // batched state (allocated on first use, grown on demand)

@@ -11,9 +11,12 @@
 // the buffers they pass in.
 //
 // Limits and sharing:
-//   - the array holds kNoAllocBytes (32 MiB) on every device that loads the
-//     library, for the life of the process;
-//   - graphs whose single-query state does not fit are rejected (AHPP_EINVAL);
+//   - the array holds kNoAllocBytes (32 MiB) and kLayoutBytes on every device
+//     that loads the library, for the life of the process;
+//   - graphs whose single-query state (the vectors, and the sums of rows of more
+//     than 2,048 entries) exceeds 32 MiB are rejected (AHPP_EINVAL).  What the
+//     layout of the pull rounds needs beyond that (both sets of sums, copies of
+//     t_A) has room of its own, so which graphs are taken does not depend on it;
 //   - every call uses the same array and leaves its contents behind; the
 //     kernel clears everything that must start at zero.  Calls that overlap
 //     on the GPU would race on the array: this entry point serialises its own
@@ -30,9 +33,10 @@ namespace ahpp {
 namespace {
 
 constexpr size_t kNoAllocBytes = 32ull << 20;
+constexpr size_t kLayoutBytes = 4ull << 20;
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes + kLayoutBytes];
 
 std::mutex g_noalloc_mu;
 void* g_noalloc_ptr[kMaxDevices] = {};
@@ -71,6 +75,15 @@ size_t carve(const ahpp_graph* g, char* base, Q1State* s) {
   return off;
 }
 
+// Bytes of query state by which graphs are taken or rejected.
+size_t state_bytes(const ahpp_graph* g) {
+  const size_t nv = std::max<uint64_t>(g->n_v, 1), na = std::max<uint64_t>(g->n_a, 1);
+  const size_t ns = std::max<size_t>((size_t)g->dg.s1_v.n_split + g->dg.s1_a.n_split + g->n_long_u, 1);
+  return 4 * align256(4 * g->n_u) + align256(4 * nv) + 2 * align256(4 * na) + 2 * align256(4 * ns) +
+         align256(sizeof(QCtl)) + align256(3 * sizeof(RAcc)) + align256(sizeof(GridBarrier)) +
+         align256(2 * sizeof(unsigned int));
+}
+
 }  // namespace
 
 // Parameters of a single query (shared with the allocating entry points).
@@ -89,8 +102,8 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
     return AHPP_EINVAL;
   }
   Q1State s;
-  const size_t need = carve(g, nullptr, &s);
-  if (need > kNoAllocBytes) {
+  const size_t need = state_bytes(g);
+  if (need > kNoAllocBytes || carve(g, nullptr, &s) > kNoAllocBytes + kLayoutBytes) {
     set_error("ahpp_query_dense_noalloc: the graph needs " + std::to_string(need) +
               " bytes of query state; the static scratch holds " + std::to_string(kNoAllocBytes) +
               " (use ahpp_query_dense)");

@@ -317,6 +317,8 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   auto la = [&](uint32_t u) { return ua[u + 1] - ua[u]; };
   auto lw = [&](uint32_t v) { return vu[v + 1] - vu[v]; };
   auto none = [](uint32_t) { return 0u; };
+  g->n_long_u = 0;
+  while (g->n_long_u < nU && lv(g->n_long_u) + la(g->n_long_u) > 2048) ++g->n_long_u;
   Q.compact_a = g->bf16 && nA <= 65536;
   Q.compact_s = g->bf16;
   const uint32_t a_units = Q.compact_a ? 1 : 2, s_units = Q.compact_s ? 1 : 2;

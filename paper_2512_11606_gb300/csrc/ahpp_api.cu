@@ -152,10 +152,15 @@ int barrier_status(const GridBarrier* bars, uint32_t n, cudaStream_t stream, int
   return AHPP_OK;
 }
 
+int launch_single(const ahpp_graph* g, const Q1State& s, const Q1Params& p, cudaStream_t stream) {
+  if (g->cl.n_blocks) return launch_cluster(g->dg, g->cl, s, p, stream);
+  return launch_query1(g->dg, s, p, g->bf16, g->q1_grid, stream);
+}
+
 int run_query1_launch(ahpp_graph* g, uint32_t q_new, double eps, cudaStream_t stream) {
   Q1Params p = q1_params(g, q_new, eps);
   if (int rc = reset_barriers(g, g->q1.bar, 1, stream)) return rc;
-  int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, stream);
+  int e = launch_single(g, g->q1, p, stream);
   if (e) return cuda_fail((cudaError_t)e, "k_query1 launch");
   return AHPP_OK;
 }
@@ -174,7 +179,7 @@ int run_lambda(ahpp_graph* g) {
   p.kahan = 1;
   p.max_rounds = T;
   if (int rc = reset_barriers(nullptr, g->q1.bar, 1, g->stream)) return rc;
-  int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, g->stream);
+  int e = launch_single(g, g->q1, p, g->stream);
   if (e) return cuda_fail((cudaError_t)e, "lambda launch");
   unsigned int bits[2] = {0, 0};
   QCtl ctl;
@@ -549,7 +554,7 @@ int ahpp_power_iteration(ahpp_graph* g, uint32_t q, uint32_t T, float* out_pi, a
   set_tests(p);
   p.max_rounds = T;
   if (int rc = reset_barriers(g, g->q1.bar, 1, g->stream)) return rc;
-  int e = launch_query1(g->dg, g->q1, p, g->bf16, g->q1_grid, g->stream);
+  int e = launch_single(g, g->q1, p, g->stream);
   if (e) return cuda_fail((cudaError_t)e, "power iteration launch");
   int rc;
   if ((rc = ensure(g, io->dense, 4ull * g->n_u))) return rc;
@@ -827,7 +832,7 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     return set(best_v);
   };
   const uint32_t saved_div = g->q1_dense_div, saved_vw = g->q1_vw_max;
-  rc = tune_single("single_vec_width", [&](uint32_t v) { return build_q1_layout(g, v); }, {32u, 8u, 2u, 1u});
+  if (!g->cl.n_blocks) rc = tune_single("single_vec_width", [&](uint32_t v) { return build_q1_layout(g, v); }, {32u, 8u, 2u, 1u});
   if (rc == AHPP_OK)
     rc = tune_single("single_dense_div", [&](uint32_t v) { g->q1_dense_div = v; return AHPP_OK; }, {32u, 8u, 16u, 64u, 128u});
   if (rc != AHPP_OK) {

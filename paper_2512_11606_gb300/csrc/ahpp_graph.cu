@@ -374,6 +374,9 @@ int alloc_query_state(ahpp_graph* g) {
   if (max_blocks <= 0) { set_error("ahpp_load_graph: occupancy query failed"); return AHPP_ECUDA; }
   g->q1_max_blocks = (uint32_t)max_blocks;
   if (int rc = build_q1_layout(g, cfg.single_vec_width)) return rc;
+  // a lane width asks for the grid kernel, whose rows it is about
+  if (!cfg.single_vec_width)
+    if (int rc = build_cluster_layout(g)) return rc;
   g->n_split1 = 2 * G.q1.v.n_split + G.q1.u.n_split;
   const size_t before = g->bufs.size();
   Q1State& s = g->q1;

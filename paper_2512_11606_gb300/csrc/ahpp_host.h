@@ -14,6 +14,7 @@
 #include "ahpp_internal.cuh"
 #include "ahpp_query1.cuh"
 #include "ahpp_batch.cuh"
+#include "ahpp_cluster.cuh"
 
 namespace ahpp {
 
@@ -89,6 +90,7 @@ struct ahpp_graph {
   // single-query state
   ahpp::Q1State q1{};
   int q1_grid = 0;
+  ahpp::ClusterLayout cl{};       // small graphs: the layout of the cluster kernel, which then runs them
   // single-query pull layout (dg.q1): its buffers, the most blocks the device
   // keeps resident, shared memory per block, lanes of the shortest rows
   std::vector<void*> q1_layout_bufs;
@@ -146,6 +148,9 @@ int kernel_algo(int algo);
 // Sliced layout of the single-query pull rounds with at least vec_width lanes
 // per row (0: by the graph's size); replaces the one the graph has.
 int build_q1_layout(ahpp_graph* g, uint32_t vec_width);
+int build_cluster_layout(ahpp_graph* g);
+// A single query's launch, on the cluster kernel where the graph has its layout.
+int launch_single(const ahpp_graph* g, const Q1State& s, const Q1Params& p, cudaStream_t stream);
 // Index into kChunkSizes of a configured chunk size (0: the default), -1 if
 // it is not one of them.
 int chunk_choice(uint32_t chunk);

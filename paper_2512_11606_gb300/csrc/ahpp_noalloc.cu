@@ -122,7 +122,7 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
   cudaStream_t st = stream ? (cudaStream_t)stream : g->stream;
   Q1Params p = noalloc_params(g, g->h_u_old2new[q], eps);
   if (int rc = reset_barriers(g, s.bar, 1, st)) return rc;
-  const int e = launch_query1(g->dg, s, p, g->bf16, g->q1_grid, st);
+  const int e = launch_single(g, s, p, st);
   if (e) return cuda_fail((cudaError_t)e, "ahpp_query_dense_noalloc: launch");
   k_scatter_out<<<std::max(1, g->sm_count * 4), 256, 0, st>>>(s.pi, g->d_u_new2old, (uint32_t)g->n_u,
                                                               d_out_pi);

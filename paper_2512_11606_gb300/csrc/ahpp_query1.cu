@@ -37,6 +37,7 @@
 
 #include "ahpp_internal.cuh"
 #include "ahpp_query1.cuh"
+#include "ahpp_rounds.cuh"
 
 namespace ahpp {
 
@@ -66,14 +67,6 @@ struct Ctx {
 };
 
 // -------------------------------------------------- partials of a block
-
-// Per-round sums of a thread; every sum stays below |E| + |E_A| < 2^32.
-struct Q1Part {
-  float max_r = 0.f;
-  uint32_t marked = 0, marked_deg = 0, np_flush = 0;
-  float max_rel = 0.f;       // APP(S) statistics (see RAcc)
-  uint32_t above = 0;
-};
 
 // Block reduction of p into acc, one atomic per field and block: one redux
 // per field in each warp (the floats are >= 0, so their bits order them),
@@ -341,13 +334,6 @@ __device__ __forceinline__ void phase1(const Ctx& c, Q1Part& part, Ring& ring, c
 // r_U'[u] = kept_u + sum_v w(u,v) t_V[v] + sum_a w(u,a) t_A[a]; reserve update of
 // the nodes pushed this round; marking of the next frontier with threshold th.
 
-// APP(S)'s round statistics of a residue r of a node with cnt = |N(u)| + |A(u)|:
-// the largest r / cnt, and whether r exceeds APP's threshold r_max cnt.
-__device__ __forceinline__ void app_stats(const Ctx& c, float r, uint32_t cnt, Q1Part& part) {
-  if (cnt) part.max_rel = fmaxf(part.max_rel, r / (float)cnt);
-  if (above_node_threshold(r, c.p.eps_f, c.p.eps_f32, cnt)) part.above += 1;
-}
-
 // Residue r_old (reserve pv, compensation pc) of row u takes in s.
 template <bool APPS>
 __device__ __forceinline__ void finish_row(const Ctx& c, uint32_t u, float s, float r_old, float pv, float pc,
@@ -366,7 +352,7 @@ __device__ __forceinline__ void finish_row(const Ctx& c, uint32_t u, float s, fl
   }
   const float r_new = kept + s;
   part.max_r = fmaxf(part.max_r, r_new);
-  if (APPS) app_stats(c, r_new, cnt, part);
+  if (APPS) app_stats(c.p, r_new, cnt, part);
   const bool mark = per_node ? above_node_threshold(r_new, c.p.eps_f, c.p.eps_f32, cnt) : r_new >= th;
   if (mark) {
     part.marked += 1;
@@ -529,7 +515,7 @@ __device__ __forceinline__ void flush_row(const Ctx& c, bool is_a, uint32_t b, u
     // APP(S): a node's last update sees its new residue (counts of nodes
     // above threshold may repeat a node; only zero is tested)
     if (APPS)
-      app_stats(c, old + add, (g.uv_off[j + 1] - g.uv_off[j]) + (g.ua_off[j + 1] - g.ua_off[j]), part);
+      app_stats(c.p, old + add, (g.uv_off[j + 1] - g.uv_off[j]) + (g.ua_off[j + 1] - g.ua_off[j]), part);
   }
 }
 
@@ -616,63 +602,17 @@ __device__ void mark_remaining(const Ctx& c, Q1Part& part) {
   }
 }
 
-// The query's control, kept in shared memory by thread 0 of every block (all
-// read the same round accumulators after a barrier, so all blocks agree).
-struct Q1Loop {
-  unsigned long long n_p, pushes, marked_deg;
-  uint32_t rounds, switch_round, dense_rounds, marked;
-  int phase, status, dense, switched, per_node, go;
-  float theta;
-};
-
-__device__ __forceinline__ bool switch_now(const Q1Params& p, unsigned long long n_p, float m) {
-  return switch_due(p.e_tot, p.switch_rule, p.eps_f, p.lambda, p.log_inv, p.switch_unit, p.switch_log, n_p, m);
-}
-
-// Before a round: stop, or how it runs (the marks are in the last round's accumulators).
+// Before and after a round, from its accumulators in global memory.
 __device__ void begin_round(const Q1State& s, const Q1Params& p, Q1Loop& L) {
   const RAcc* P = &s.racc[(L.rounds + 2) % 3];
-  L.marked = __ldcg(&P->marked);
-  L.marked_deg = __ldcg(&P->marked_deg);
-  L.go = 0;
-  if (L.phase == kPhaseDone || L.marked == 0) { L.phase = kPhaseDone; return; }
-  if (L.rounds >= p.max_rounds) { L.status = kStatusCap; return; }
-  L.go = 1;
-  if (blockIdx.x == 0) s.racc[(L.rounds + 1) % 3] = RAcc{};
-  if (!L.dense && L.marked_deg * (unsigned long long)p.dense_div > (unsigned long long)p.e_tot) L.dense = 1;
-  L.pushes += L.marked;
-  L.per_node = per_node_threshold(p.algo, L.phase);
-  L.theta = L.phase == kPhaseSync ? p.th_sync : p.th_async;
+  begin_round(p, L, __ldcg(&P->marked), __ldcg(&P->marked_deg));
+  if (L.go && blockIdx.x == 0) s.racc[(L.rounds + 1) % 3] = RAcc{};
 }
-
-// After a round: its counters, the termination and the switch test.
 template <bool APPS>
 __device__ void end_round(const Q1State& s, const Q1Params& p, Q1Loop& L) {
   const RAcc* A = &s.racc[L.rounds % 3];
-  const float M = __uint_as_float(__ldcg(&A->max_r_bits));
-  const unsigned long long np = __ldcg(&A->np_flush);
-  ++L.rounds;
-  L.n_p += L.marked_deg + np;
-  L.switched = 0;
-  bool due = false;
-  if (APPS) {
-    // APP's stopping test; the switch budget in units of APP's thresholds
-    const float Mrel = __uint_as_float(__ldcg(&A->max_rel_bits));
-    if (__ldcg(&A->above) == 0) L.phase = kPhaseDone;
-    else due = L.phase == kPhaseAsync && switch_now(p, L.n_p, Mrel);
-  } else if (p.algo == kAlgoASRP) {
-    if (M < p.th_async) L.phase = kPhaseDone;            // M <= eps_f
-    else due = L.phase == kPhaseAsync && switch_now(p, L.n_p, M);
-  }
-  if (due) {
-    L.phase = kPhaseSync;
-    L.switch_round = L.rounds + 1;
-    L.switched = 1;
-  }
-  L.go = L.phase != kPhaseDone;
-  // marking of the next frontier in a push round
-  L.per_node = per_node_threshold(p.algo, L.phase);
-  L.theta = L.phase == kPhaseSync ? p.th_sync : p.th_async;
+  end_round<APPS>(p, L, __uint_as_float(__ldcg(&A->max_r_bits)), __ldcg(&A->np_flush),
+                  APPS ? __uint_as_float(__ldcg(&A->max_rel_bits)) : 0.f, APPS ? __ldcg(&A->above) : 0u);
 }
 
 }  // namespace

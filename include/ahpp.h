@@ -96,8 +96,9 @@ typedef struct {
                                   256 or 512 (less on graphs too small for it); 0: 256
                                   (ahpp_autotune picks one) */
     uint32_t single_vec_width; /* single-query kernel: at least this many lanes walk one row
-                                  (1, 2, 4, 8, 16 or 32); 0: 1, 2, 8 or 32 by the graph's size
-                                  (ahpp_autotune picks one of those) */
+                                  (1, 2, 4, 8, 16 or 32); 0: 1 or 2 by the graph's size
+                                  (ahpp_autotune picks 1, 2, 8 or 32), and graphs that one
+                                  thread-block cluster holds run there instead */
 } ahpp_config;
 
 /* Per-query statistics. */
@@ -134,7 +135,8 @@ typedef struct {
      * U->A of pull rounds added up in shared memory (single_attr_push, always
      * 1); the shortest rows walked by single_vec_width lanes each (1 = one row
      * per lane), longer ones by more; single_smem_bytes of shared memory per
-     * block. */
+     * block.  (Of the whole-GPU kernel: graphs that one thread-block cluster
+     * holds run there.) */
     uint32_t single_dense_div, single_attr_push, single_vec_width, single_smem_bytes;
 } ahpp_graph_info;
 

@@ -329,13 +329,13 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   const uint32_t nb = (uint32_t)std::min<uint64_t>(g->q1_max_blocks, std::max<uint64_t>(8, 4 * steps / kQ1Warps));
   Q.n_warps = nb * kQ1Warps;
   g->q1_grid = (int)nb;
-  // lanes per short row: enough that the slices cover the warps
-  uint32_t vw = vec_width;
-  if (!vw)
-    for (uint32_t w : {1u, 2u, 8u, 32u}) {
-      vw = w;
-      if ((uint64_t)nU * w / 32 >= Q.n_warps) break;
-    }
+  // lanes per short row: one (16,000 nodes: 1.77 ms a query with eight lanes, 1.69
+  // with one; 44,000: 2.62, 1.70; 100,000: 2.94, 2.64), unless that leaves the
+  // warps a long slice of U rows or two each (200,000 nodes of 40 entries: 5.35 with
+  // one, 4.89 with two; 277,000 of 36: 10.0, 9.28; but 176,000 of 22: 3.86, 4.85)
+  const uint64_t slices = nU / 32;
+  const bool uneven = slices > Q.n_warps && 10 * slices < 19 * (uint64_t)Q.n_warps;
+  const uint32_t vw = vec_width ? vec_width : uneven && (uint64_t)G.n_e + G.n_ea >= 30ull * nU ? 2 : 1;
   g->q1_vw_max = vw;
   uint32_t lg_min = 0;
   while ((1u << lg_min) < vw) ++lg_min;

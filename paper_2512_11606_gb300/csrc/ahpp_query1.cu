@@ -377,28 +377,26 @@ __device__ __forceinline__ void phase2(const Ctx& c, float th, bool per_node, Q1
   for (uint32_t i = v4 + threadIdx.x; i < hub_v / 4; i += kQ1Threads)
     reinterpret_cast<float4*>(s_tv)[i] = reinterpret_cast<const float4*>(t_v)[i];
   for (uint32_t i = threadIdx.x; i < min(4 * v4, hub_v); i += kQ1Threads) s_tv[i] = i < nsv ? acc.v_cur[i] : t_v[i];
-  const uint32_t n_ta = na * Q.ta_copies;
-  if (n_ta == na) {
-    for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) s_ta[i] = ta_cur[i];
-  } else {                                 // all loads of a sum in flight at once
-    for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) {
-      float t = 0.f;
-#pragma unroll
-      for (uint32_t k = 0; k < kTaCopies; ++k) t += i + k * na < n_ta ? ta_cur[i + k * na] : 0.f;
-      s_ta[i] = t;
-    }
-  }
   // active attributes and split V rows (Algorithm 4's push counter); the next
   // round's sums start at zero
-  for (uint32_t a = c.gt; a < na; a += c.nt) {
-    bool active = false;
+  if (Q.ta_copies == 1) {
+    for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) s_ta[i] = ta_cur[i];
+    for (uint32_t a = c.gt; a < na; a += c.nt) {
+      if (ta_cur[a] > 0.f) part.np_flush += Q.deg_a[a];
+      ta_next[a] = 0.f;
+    }
+  } else {                                 // all loads of a sum in flight at once
+    const uint32_t n_ta = na * Q.ta_copies;
+    auto sum = [&](uint32_t a) {
+      float t = 0.f;
 #pragma unroll
-    for (uint32_t k = 0; k < kTaCopies; ++k)
-      if (a + k * na < n_ta) {
-        active |= ta_cur[a + k * na] > 0.f;
-        ta_next[a + k * na] = 0.f;
-      }
-    if (active) part.np_flush += Q.deg_a[a];
+      for (uint32_t k = 0; k < kTaCopies; ++k) t += a + k * na < n_ta ? ta_cur[a + k * na] : 0.f;
+      return t;
+    };
+    for (uint32_t i = threadIdx.x; i < hub_a; i += kQ1Threads) s_ta[i] = sum(i);
+    for (uint32_t a = c.gt; a < na; a += c.nt)
+      if (sum(a) > 0.f) part.np_flush += Q.deg_a[a];
+    for (uint32_t a = c.gt; a < n_ta; a += c.nt) ta_next[a] = 0.f;
   }
   for (uint32_t v = c.gt; v < nsv; v += c.nt) {
     if (acc.v_cur[v] > 0.f) part.np_flush += Q.deg_v[v];

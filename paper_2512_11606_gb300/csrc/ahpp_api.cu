@@ -467,6 +467,7 @@ void ahpp_free_graph(ahpp_graph* g) {
   for (void* p : g->q1_layout_bufs) cudaFree(p);
   for (void* p : g->tile_layout_bufs) cudaFree(p);
   g->release_all();
+  if (g->host_out) cudaFreeHost(g->host_out);
   if (g->stream) cudaStreamDestroy(g->stream);
   io_drop(g);
   delete g;
@@ -508,14 +509,25 @@ int ahpp_query_device(ahpp_graph* g, uint32_t q, double eps, uint32_t k, uint32_
   return ahpp::run_single_device(g, q, eps, k, d_out_nodes, d_out_scores, d_out_n, d_stats, s);
 }
 
-static int finish_single(ahpp_graph* g, double eps, ahpp_stats* st) {
+// Waits for a single query: one copy into pinned memory brings its control block,
+// maxima and barrier, and k nodes and scores (the copies into pageable memory that
+// it replaces cost 8 us each).
+static int finish_single(ahpp_graph* g, double eps, ahpp_stats* st, uint32_t k = 0, uint32_t* out_nodes = nullptr,
+                         float* out_scores = nullptr) {
+  const size_t bytes = k ? kOutTop + 8ull * k : kOutTop;
+  AHPP_CUDA(cudaMemcpyAsync(g->host_out, g->d_out, bytes, cudaMemcpyDeviceToHost, g->stream));
+  AHPP_CUDA(cudaStreamSynchronize(g->stream));
   QCtl ctl;
+  GridBarrier bar;
   unsigned int bits[2];
-  AHPP_CUDA(cudaMemcpyAsync(&ctl, g->q1.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, g->stream));
-  AHPP_CUDA(cudaMemcpyAsync(bits, g->q1.final_maxr_bits, sizeof(bits), cudaMemcpyDeviceToHost, g->stream));
-  int bst = kStatusOk;
-  if (int rc = barrier_status(g->q1.bar, 1, g->stream, &bst)) return rc;
-  if (bst == kStatusWait) ctl.status = kStatusWait;
+  std::memcpy(&ctl, g->host_out, sizeof(ctl));
+  std::memcpy(bits, g->host_out + kOutBits, sizeof(bits));
+  std::memcpy(&bar, g->host_out + kOutBar, sizeof(bar));
+  if (k) {
+    std::memcpy(out_nodes, g->host_out + kOutTop, 4ull * k);
+    std::memcpy(out_scores, g->host_out + kOutTop + 4ull * k, 4ull * k);
+  }
+  if (bar.err) ctl.status = kStatusWait;
   if (st) {
     st->rounds = ctl.rounds;
     st->switch_round = ctl.switch_round;
@@ -584,17 +596,13 @@ int ahpp_query(ahpp_graph* g, uint32_t q, double eps, uint32_t k, uint32_t* out_
   if (rc) return rc;
   const uint32_t kk = (uint32_t)std::min<uint64_t>(k, g->n_u);
   if (kk) {
-    if ((rc = ensure(g, io->nodes, 4ull * AHPP_MAX_K)) || (rc = ensure(g, io->scores, 4ull * AHPP_MAX_K)) ||
-        (rc = ensure(g, io->n, 16)))
-      return rc;
-    rc = topk_single(g, g->q1.pi, kk, (uint32_t*)io->nodes.p, (float*)io->scores.p,
+    if ((rc = ensure(g, io->n, 16))) return rc;
+    rc = topk_single(g, g->q1.pi, kk, (uint32_t*)(g->d_out + kOutTop), (float*)(g->d_out + kOutTop + 4ull * kk),
                      (uint32_t*)io->n.p, g->stream);
     if (rc) return rc;
-    AHPP_CUDA(cudaMemcpyAsync(out_nodes, io->nodes.p, 4ull * kk, cudaMemcpyDeviceToHost, g->stream));
-    AHPP_CUDA(cudaMemcpyAsync(out_scores, io->scores.p, 4ull * kk, cudaMemcpyDeviceToHost, g->stream));
   }
   if (out_n) *out_n = kk;
-  return finish_single(g, eps, st);
+  return finish_single(g, eps, st, kk, out_nodes, out_scores);
 }
 
 int ahpp_query_dense(ahpp_graph* g, uint32_t q, double eps, float* out_pi, ahpp_stats* st) {

@@ -390,15 +390,17 @@ int alloc_query_state(ahpp_graph* g) {
   s.list_u = (uint32_t*)g->alloc(4ull * nU);
   s.split_acc = (float*)g->alloc(4ull * std::max(g->n_split1, 1u));
   s.split_cnt = (uint32_t*)g->alloc(4ull * std::max(g->n_split1, 1u));
-  s.ctl = (QCtl*)g->alloc(sizeof(QCtl));
+  g->d_out = (char*)g->alloc(kOutBytes);
+  s.ctl = (QCtl*)g->d_out;
+  s.final_maxr_bits = (unsigned int*)(g->d_out + kOutBits);
+  s.bar = (GridBarrier*)(g->d_out + kOutBar);
   s.racc = (RAcc*)g->alloc(3 * sizeof(RAcc));
-  s.bar = (GridBarrier*)g->alloc(sizeof(GridBarrier));
-  s.final_maxr_bits = (unsigned int*)g->alloc(2 * sizeof(unsigned int));
   g->q1_bytes = 0;
   for (size_t i = before; i < g->bufs.size(); ++i) {
     if (!g->bufs[i].p) { set_error("ahpp_load_graph: device allocation failed"); return AHPP_ENOMEM; }
     g->q1_bytes += g->bufs[i].bytes;
   }
+  AHPP_CUDA(cudaMallocHost((void**)&g->host_out, kOutBytes));
   AHPP_CUDA(cudaMemset(s.bar, 0, sizeof(GridBarrier)));
   AHPP_CUDA(cudaMemset(s.split_acc, 0, 4ull * std::max(g->n_split1, 1u)));
   AHPP_CUDA(cudaMemset(s.split_cnt, 0, 4ull * std::max(g->n_split1, 1u)));

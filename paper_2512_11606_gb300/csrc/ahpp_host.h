@@ -65,6 +65,14 @@ struct DevBuf {
 
 }  // namespace ahpp
 
+namespace ahpp {
+// Places in a single query's result block (the barrier, which blocks poll, has a
+// line of its own).
+constexpr size_t kOutBits = 128, kOutBar = 256, kOutTop = 384;
+static_assert(sizeof(QCtl) <= kOutBits, "control block");
+constexpr size_t kOutBytes = kOutTop + 8 * (size_t)AHPP_MAX_K;
+}  // namespace ahpp
+
 struct ahpp_graph {
   ahpp_config cfg{};
   int device = 0;
@@ -98,6 +106,9 @@ struct ahpp_graph {
   uint32_t q1_max_blocks = 0, q1_smem = 0, q1_vw_max = 0;
   uint32_t q1_dense_div = 32;     // pull rounds once the frontier covers > 1/dense_div of the edges
   std::string tune_log;           // the last autotune's measurements (JSON object)
+  // what a single query leaves for the host, in one block that one copy fetches:
+  // control, final maxima, barrier, then nodes and scores; host_out: its pinned copy
+  char *d_out = nullptr, *host_out = nullptr;
   uint32_t n_split1 = 0;
   uint32_t n_long_u = 0;          // U rows of more than 2,048 entries
   uint64_t q1_bytes = 0;

@@ -20,7 +20,7 @@
 //
 // What bounds a pull round, and what the layout does about it (GB300, one
 // query, 20M edges and 20M attribute entries; a round took 0.320 ms with
-// rows of CSR walked by two lanes each, 0.190 ms now; 2M + 2M: 0.077, 0.035):
+// rows of CSR walked by two lanes each, 0.190 ms now; 2M + 2M: 0.077, 0.028):
 //   - looking up 4-byte values at random: an SM finds one L1 line a cycle, so a
 //     warp's 32 lookups take 32 cycles from L2.  The entries most looked up
 //     (degree order: the first ones) are copied to shared memory each phase,
@@ -30,8 +30,10 @@
 //     shared memory, across the barrier too;
 //   - uneven shares: cut by measured cost at load (ahpp_q1layout.cu);
 //   - FP64: see switch_due; a log in every thread was 25 us of every round.
+//   - reductions that meet in a few lines: see Q1Layout::ta_copies.
 // Two barriers a round take about 2,500 cycles each; a small graph's round is
-// mostly those and the few L2 latencies between them.
+// mostly those and the few L2 latencies between them (the smallest graphs run
+// on one cluster instead: ahpp_cluster.cu).
 #include <algorithm>
 #include <type_traits>
 

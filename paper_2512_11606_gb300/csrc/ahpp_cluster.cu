@@ -402,10 +402,11 @@ using ClusterFn = void (*)(const DevGraph, const ClusterLayout, const Q1State, c
 
 ClusterFn cluster_fn(bool apps) { return apps ? k_cluster<true> : k_cluster<false>; }
 
-// Dynamic shared memory limit and cluster size of an instance.
-cudaError_t allow(ClusterFn fn, uint32_t smem_bytes) {
+// Dynamic shared memory limit and cluster size of an instance (the limit of all
+// graphs, so that threads that launch for different ones do not undo each other's).
+cudaError_t allow(ClusterFn fn) {
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
   return e;
 }
 
@@ -429,7 +430,7 @@ bool cluster_fits(uint32_t blocks, uint32_t smem_bytes) {
     ClusterFn fn = cluster_fn(apps != 0);
     cudaLaunchAttribute attr;
     int n = 0;
-    cudaError_t e = allow(fn, smem_bytes);
+    cudaError_t e = allow(fn);
     if (e == cudaSuccess) {
       const cudaLaunchConfig_t c = config(blocks, smem_bytes, nullptr, &attr);
       e = cudaOccupancyMaxActiveClusters(&n, fn, &c);
@@ -650,7 +651,7 @@ int launch_cluster(const DevGraph& g, const ClusterLayout& c, const Q1State& s, 
   ClusterFn fn = cluster_fn(p.algo == kAlgoAPPS);
   cudaLaunchAttribute attr;
   const cudaLaunchConfig_t cfg = config(c.n_blocks, c.smem_bytes, stream, &attr);
-  cudaError_t e = allow(fn, c.smem_bytes);
+  cudaError_t e = allow(fn);
   if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fn, g, c, s, p);
   return (int)e;
 }

@@ -788,7 +788,8 @@ const void* q1_fn(int form, bool apps) { return apps ? q1_form<true>(form) : q1_
 // Carve out of the SM's unified memory just the shared memory the block needs
 // (with 1 KB reserved by the system); the rest stays L1, which holds the lines
 // of the gathers in flight.  Sets the dynamic shared memory limit of the
-// instance too.
+// instance too, to that of all graphs: threads that launch for different ones must
+// not undo each other's.
 int prepare(const void* fn, uint32_t smem_bytes) {
   int dev = 0, per_sm = 0;
   cudaFuncAttributes fa{};
@@ -796,7 +797,7 @@ int prepare(const void* fn, uint32_t smem_bytes) {
       cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
       cudaFuncGetAttributes(&fa, fn) != cudaSuccess || per_sm <= 0)
     return (int)cudaGetLastError();
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQ1SmemMax);
   if (e != cudaSuccess) return (int)e;
   const uint64_t need = (uint64_t)kQ1Blocks * (smem_bytes + fa.sharedSizeBytes + 1024);
   const int pct = (int)std::min<uint64_t>(100, (100 * need + per_sm - 1) / per_sm);

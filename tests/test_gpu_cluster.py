@@ -91,3 +91,34 @@ def test_lambda_and_power_iteration_match_grid_kernel(ahpp, kind):
     finally:
         G.close()
         H.close()
+
+
+def test_threads_on_graphs_of_different_sizes(ahpp):
+    """Launches for graphs whose kernels ask for different amounts of shared
+    memory, from a thread each: every call works and answers as it does alone."""
+    import threading
+
+    specs = [(KINDS[3], 0), (KINDS[6], 0), (KINDS[3], 2), (KINDS[7], 2)]
+    graphs = [ahpp.Graph.from_arrays(graph(**k), attr_bf16=0, single_vec_width=w) for k, w in specs]
+    alone = [G.query_dense(5, 1e-6)[0].astype(np.float64) for G in graphs]
+    bad = []
+
+    def work(i):
+        try:
+            for _ in range(30):
+                pi, _, rc = graphs[i].query_dense(5, 1e-6)
+                if rc != 0 or np.abs(pi - alone[i]).max() > TOL:
+                    bad.append((i, rc))
+        except Exception as e:  # noqa: BLE001
+            bad.append((i, repr(e)))
+
+    try:
+        threads = [threading.Thread(target=work, args=(i,)) for i in range(len(graphs))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert not bad
+    finally:
+        for G in graphs:
+            G.close()

@@ -16,7 +16,7 @@
 // What bounds it: the chain of a round, about 7,500 cycles (two walks, a row's
 // sum, two exchanges of 1,200 cycles that end when the remote writes have
 // arrived; tiny graph of 2,000 nodes).  One query there: 1.38 ms on the grid
-// kernel, 0.43 here; 4,000 nodes and 160,000 entries: 0.95, 0.58.  Graphs whose
+// kernel, 0.40 here; 4,000 nodes and 160,000 entries: 0.95, 0.58.  Graphs whose
 // entries do not fit are left to the grid kernel: read from L2 by 16 SMs (24
 // cycles of the SM's data path for a step, and blocks sending each other 17 bytes a
 // cycle) they were no faster here (6,000 nodes 0.97 against 1.01 ms, 20,000 nodes

@@ -207,28 +207,31 @@ int batch_plan(ahpp_graph* g) {
   return AHPP_OK;
 }
 
+// Buffers for `groups` tiles at once and kmax results a query.  A launch reads the
+// table of its tiles on the device as it goes, and the call that made it may have
+// returned (ahpp_query_batch_device): growing makes a new table, and buffers and
+// tables that launches were given live as long as the graph.  On failure the
+// state stays as it was.
 int ensure_batch(ahpp_graph* g, uint32_t groups, uint32_t kmax) {
-  BatchState& s = g->bt;
   kmax = std::max<uint32_t>(kmax, 1);
-  if (s.n_groups >= groups && s.kmax_cap >= kmax) return AHPP_OK;
+  if (g->bt.n_groups >= groups && g->bt.kmax_cap >= kmax) return AHPP_OK;
+  BatchState s = g->bt;
   const DevGraph& G = g->dg;
   const size_t n_split = std::max(G.tl.split_u_max, 1u);        // any chunk choice fits
   const uint32_t kcap = std::max(kmax, s.kmax_cap);
   const uint32_t ng = std::max(groups, s.n_groups);
+  const size_t before = g->bufs.size();
   uint64_t bytes = 0;
   bool ok = true;
   auto A = [&](size_t b) {
     bytes += b;
-    void* p = g->alloc(b);
+    void* p = ok ? g->alloc(b) : nullptr;
     ok = ok && p;
     return p;
   };
-  if (!s.bars) {
-    s.bars = (GridBarrier*)A(kMaxGroups * sizeof(GridBarrier));
-    s.d_tb = (TileBuf*)A(kMaxGroups * sizeof(TileBuf));
-    if (ok) AHPP_CUDA(cudaMemset(s.bars, 0, kMaxGroups * sizeof(GridBarrier)));
-    bytes = 0;
-  }
+  if (!s.bars) s.bars = (GridBarrier*)A(kMaxGroups * sizeof(GridBarrier));
+  s.d_tb = (TileBuf*)A(kMaxGroups * sizeof(TileBuf));
+  bytes = 0;
   for (uint32_t i = 0; i < ng && ok; ++i) {
     TileBuf& t = s.tb[i];
     const bool fresh = i >= s.n_groups;
@@ -246,11 +249,16 @@ int ensure_batch(ahpp_graph* g, uint32_t groups, uint32_t kmax) {
     }
     if (fresh || kcap > s.kmax_cap) t.cand = (unsigned long long*)A((size_t)kTile * kcap * 8);
   }
-  if (!ok) { set_error("batched state allocation failed"); return AHPP_ENOMEM; }
+  if (!ok) {
+    for (; g->bufs.size() > before; g->bufs.pop_back()) cudaFree(g->bufs.back().p);
+    set_error("batched state allocation failed");
+    return AHPP_ENOMEM;
+  }
   AHPP_CUDA(cudaMemcpy(s.d_tb, s.tb, ng * sizeof(TileBuf), cudaMemcpyHostToDevice));
   if (s.n_groups == 0) g->tile_bytes = bytes / ng;
   s.n_groups = ng;
   s.kmax_cap = kcap;
+  g->bt = s;
   return AHPP_OK;
 }
 

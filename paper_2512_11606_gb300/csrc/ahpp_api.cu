@@ -133,6 +133,11 @@ Q1Params noalloc_params(const ahpp_graph* g, uint32_t q_new, double eps) {
   return q1_params(g, q_new, eps);
 }
 
+cudaError_t upload(ahpp_graph* g, void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, g->upload_stream) : cudaSuccess;
+  return e == cudaSuccess ? cudaStreamSynchronize(g->upload_stream) : e;
+}
+
 int reset_barriers(ahpp_graph* g, GridBarrier* bars, uint32_t n, cudaStream_t stream) {
   AHPP_CUDA(cudaMemsetAsync(bars, 0, n * sizeof(GridBarrier), stream));
   if (g && g->wait_trap.exchange(0)) {
@@ -254,7 +259,7 @@ int ensure_batch(ahpp_graph* g, uint32_t groups, uint32_t kmax) {
     set_error("batched state allocation failed");
     return AHPP_ENOMEM;
   }
-  AHPP_CUDA(cudaMemcpy(s.d_tb, s.tb, ng * sizeof(TileBuf), cudaMemcpyHostToDevice));
+  AHPP_CUDA(upload(g, s.d_tb, s.tb, ng * sizeof(TileBuf)));
   if (s.n_groups == 0) g->tile_bytes = bytes / ng;
   s.n_groups = ng;
   s.kmax_cap = kcap;
@@ -450,7 +455,8 @@ int ahpp_load_graph(const ahpp_graph_desc* desc, const ahpp_config* cfg, ahpp_gr
   g->batch_groups = c.batch_groups;
   int rc = AHPP_OK;
   if (cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&g->upload_stream, cudaStreamNonBlocking) != cudaSuccess) {
     rc = cuda_fail(cudaGetLastError(), "ahpp_load_graph: device setup");
   }
   if (rc == AHPP_OK) rc = build_graph(desc, g);
@@ -477,6 +483,7 @@ void ahpp_free_graph(ahpp_graph* g) {
   g->release_all();
   if (g->host_out) cudaFreeHost(g->host_out);
   if (g->stream) cudaStreamDestroy(g->stream);
+  if (g->upload_stream) cudaStreamDestroy(g->upload_stream);
   io_drop(g);
   delete g;
 }

@@ -209,7 +209,8 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
     if (rc == AHPP_OK) { set_error(msg); rc = code; }
   };
   if (cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&g->upload_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     fail(AHPP_ECUDA, "ahpp_load_graph_file: device setup failed");
   }
@@ -230,7 +231,7 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
     if (!rd(in.f, host.data(), n, cs)) { fail(AHPP_EINVAL, "ahpp_load_graph_file: truncated file"); break; }
     void* p = g->alloc(n ? n : 4);
     if (!p) { fail(AHPP_ENOMEM, "ahpp_load_graph_file: device allocation failed"); break; }
-    if (n && cudaMemcpy(p, host.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (upload(g, p, host.data(), n) != cudaSuccess) {
       cudaGetLastError();
       fail(AHPP_ECUDA, "ahpp_load_graph_file: upload failed");
     }

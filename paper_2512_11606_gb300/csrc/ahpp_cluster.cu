@@ -611,7 +611,7 @@ int build_cluster_layout(ahpp_graph* g) {
     const size_t before = g->graph_bytes;
     auto put = [&](const void* p, size_t bytes) -> void* {
       void* d = g->alloc(std::max<size_t>(bytes, 16));
-      if (!d || (bytes && cudaMemcpy(d, p, bytes, cudaMemcpyHostToDevice) != cudaSuccess)) ok = false;
+      if (!d || upload(g, d, p, bytes) != cudaSuccess) ok = false;
       g->graph_bytes += std::max<size_t>(bytes, 16);
       return d;
     };

@@ -308,7 +308,7 @@ int build_graph(const ahpp_graph_desc* d, ahpp_graph* g) {
   // 6. upload
   auto up = [&](const void* src, size_t bytes) -> void* {
     void* p = g->alloc(bytes ? bytes : 4);
-    if (p && bytes && cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return nullptr;
+    if (p && upload(g, p, src, bytes) != cudaSuccess) return nullptr;
     return p;
   };
   DevGraph& G = g->dg;
@@ -401,9 +401,6 @@ int alloc_query_state(ahpp_graph* g) {
     g->q1_bytes += g->bufs[i].bytes;
   }
   AHPP_CUDA(cudaMallocHost((void**)&g->host_out, kOutBytes));
-  AHPP_CUDA(cudaMemset(s.bar, 0, sizeof(GridBarrier)));
-  AHPP_CUDA(cudaMemset(s.split_acc, 0, 4ull * std::max(g->n_split1, 1u)));
-  AHPP_CUDA(cudaMemset(s.split_cnt, 0, 4ull * std::max(g->n_split1, 1u)));
   if (int rc = batch_plan(g)) return rc;
   if (int rc = build_tile_layout(g, (uint32_t)chunk_choice(cfg.batch_chunk))) return rc;
   if (cfg.hbm_budget_bytes && g->graph_bytes + g->q1_bytes > cfg.hbm_budget_bytes) {

@@ -78,6 +78,7 @@ struct ahpp_graph {
   int device = 0;
   int sm_count = 0;
   cudaStream_t stream = nullptr;
+  cudaStream_t upload_stream = nullptr;   // see ahpp::upload
   std::mutex mu;
 
   uint64_t n_u = 0, n_v = 0, n_a = 0, n_e = 0, n_ea = 0;
@@ -143,6 +144,10 @@ struct ahpp_graph {
 };
 
 namespace ahpp {
+// Host memory to the device, there when this returns: a plain cudaMemcpy from
+// pageable memory may return before its copy has arrived, and the library's
+// streams (and most callers') do not wait for the default stream it is on.
+cudaError_t upload(ahpp_graph* g, void* dst, const void* src, size_t bytes);
 // Clear n grid barriers before a persistent launch on `stream`.  When the
 // graph's self-test trap is armed (ahpp_selftest_arm_wait_timeout) the
 // counters are set far below any block count instead, so the launch's first

@@ -416,7 +416,7 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
     if (cudaMalloc(&p, n) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
     g->q1_layout_bufs.push_back(p);
     g->q1_layout_bytes += n;
-    if (src && bytes && cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+    if (src && upload(g, p, src, bytes) != cudaSuccess) ok = false;
     return p;
   };
   auto put = [&](auto& v) -> void* { return dev(v.size() * sizeof(v[0]), v.data()); };
@@ -426,7 +426,7 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
     const size_t n = v.size() * sizeof(v[0]);
     if (cudaMalloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
     tmp.push_back(p);
-    if (n && cudaMemcpy(p, v.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+    if (upload(g, p, v.data(), n) != cudaSuccess) ok = false;
     return p;
   };
   const int grid = std::max(1, 8 * g->sm_count), threads = 256;

@@ -380,10 +380,10 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
       ok = b.r_u && b.pi && b.pic && b.t && b.split_acc && b.split_cnt && b.tacc && b.racc && b.hist && b.cand && b.cand_cnt;
       if (ok) {
         // the split accumulators and counters must start at zero (kept zero by the kernel)
-        ok = cudaMemset(b.split_acc, 0, n_split * kTile * 4) == cudaSuccess &&
-             cudaMemset(b.split_cnt, 0, n_split * 4) == cudaSuccess &&
-             cudaMemset(b.tacc, 0, kTAccs * sizeof(TAcc)) == cudaSuccess &&
-             cudaMemset(b.racc, 0, 2 * kTile * sizeof(RAcc)) == cudaSuccess;
+        ok = cudaMemsetAsync(b.split_acc, 0, n_split * kTile * 4, s->stream) == cudaSuccess &&
+             cudaMemsetAsync(b.split_cnt, 0, n_split * 4, s->stream) == cudaSuccess &&
+             cudaMemsetAsync(b.tacc, 0, kTAccs * sizeof(TAcc), s->stream) == cudaSuccess &&
+             cudaMemsetAsync(b.racc, 0, 2 * kTile * sizeof(RAcc), s->stream) == cudaSuccess;
       }
     }
     if (!ok) {
@@ -392,10 +392,11 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
     }
   }
   if (rc == AHPP_OK) {
-    if (cudaMemcpy(s->d_tbufs, s->h_tbufs.data(), sizeof(TileBuf) * tiles, cudaMemcpyHostToDevice) !=
+    // on the stream of the steps, which read them
+    if (cudaMemcpyAsync(s->d_tbufs, s->h_tbufs.data(), sizeof(TileBuf) * tiles, cudaMemcpyHostToDevice, s->stream) !=
             cudaSuccess ||
-        cudaMemset(s->d_tile_round, 0, 4ull * tiles) != cudaSuccess ||
-        cudaMemset(s->d_slots, 0, sizeof(SlotState) * s->n_slots) != cudaSuccess)
+        cudaMemsetAsync(s->d_tile_round, 0, 4ull * tiles, s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->d_slots, 0, sizeof(SlotState) * s->n_slots, s->stream) != cudaSuccess)
       rc = cuda_fail(cudaGetLastError(), "ahpp_server_start: table upload");
     if (rc == AHPP_OK) {
       std::lock_guard<std::mutex> glock(g->mu);

@@ -210,7 +210,7 @@ int build_tile_layout(ahpp_graph* g, uint32_t choice) {
     if (cudaMalloc(&p, n) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
     g->tile_layout_bufs.push_back(p);
     g->tile_layout_bytes += n;
-    if (src && bytes && cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+    if (src && upload(g, p, src, bytes) != cudaSuccess) ok = false;
     return p;
   };
   auto put = [&](auto& v) -> void* { return dev(v.size() * sizeof(v[0]), v.data()); };
@@ -220,7 +220,7 @@ int build_tile_layout(ahpp_graph* g, uint32_t choice) {
     const size_t n = v.size() * sizeof(v[0]);
     if (cudaMalloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
     tmp.push_back(p);
-    if (n && cudaMemcpy(p, v.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+    if (upload(g, p, v.data(), n) != cudaSuccess) ok = false;
     return p;
   };
   const int grid = std::max(1, 8 * g->sm_count), threads = 256;
@@ -305,7 +305,7 @@ int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u)
     g->tile_layout_bufs.push_back(p);
     g->tile_layout_bytes += bytes;
     g->graph_bytes += bytes;
-    AHPP_CUDA(cudaMemcpy(p, r.data(), bytes, cudaMemcpyHostToDevice));
+    AHPP_CUDA(upload(g, p, r.data(), bytes));
     cut.r[k] = (const uint4*)p;
   }
   g->tile_cuts.push_back(cut);

@@ -220,7 +220,7 @@ k_cluster(const __grid_constant__ DevGraph g, const __grid_constant__ ClusterLay
   grid_sync(s.bar, nb, epoch);
   cluster_sync();
   if (tid == 0) {
-    s_fine = (ld_barrier(s.bar) >> 32) == 0;
+    s_fine = ld_barrier(s.bar).err == 0;
     if (p.lambda_mode) {
       begin_round(p, L, g.n_u, p.e_tot);
     } else {

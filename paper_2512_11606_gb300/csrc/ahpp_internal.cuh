@@ -240,10 +240,15 @@ struct alignas(16) GridBarrier {
 constexpr unsigned int kSpinLimit = 1u << 20;   // polls of about a microsecond: about one second
 constexpr unsigned int kSpinEager = 64;         // polls before the wait backs off
 
-// Arrivals (low word) and error flag (high word) in one acquiring load.
-__device__ __forceinline__ unsigned long long ld_barrier(const GridBarrier* b) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(b) : "memory");
+// Arrivals and error flag in one acquiring load, as two words: an acquire is
+// ordered behind a release of the same width only, and blocks arrive with a
+// 32-bit one.
+struct BarrierWords {
+  unsigned int count, err;
+};
+__device__ __forceinline__ BarrierWords ld_barrier(const GridBarrier* b) {
+  BarrierWords v;
+  asm volatile("ld.acquire.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.count), "=r"(v.err) : "l"(b) : "memory");
   return v;
 }
 
@@ -261,13 +266,13 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned int nblocks, 
     // would add about 500 cycles each to the 2,500 that this takes
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
     unsigned int spins = 0;
-    unsigned long long w = ld_barrier(b);
-    while ((w >> 32) == 0 && (int)((unsigned int)w - epoch) < 0) {
-      if (++spins > kSpinLimit) { atomicOr(&b->err, 1u); w = 1ull << 32; break; }
+    BarrierWords w = ld_barrier(b);
+    while (w.err == 0 && (int)(w.count - epoch) < 0) {
+      if (++spins > kSpinLimit) { atomicOr(&b->err, 1u); w.err = 1u; break; }
       if (spins > kSpinEager) __nanosleep(40);
       w = ld_barrier(b);
     }
-    s_ok = (w >> 32) == 0;
+    s_ok = w.err == 0;
     if (s_ok) then();
   }
   __syncthreads();

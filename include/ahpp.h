@@ -281,8 +281,10 @@ int ahpp_query_device(ahpp_graph *g, uint32_t q, double eps, uint32_t k,
  * stored in the graph and reported by ahpp_get_graph_info; the measured
  * times by ahpp_autotune_report.  Do not run it while a server on g is
  * running.  q_sample: host array of n_sample query ids (n_sample == 0
- * changes nothing).  AHPP_EINVAL for a NULL g or q_sample, an id outside U
- * or a bad eps. */
+ * changes nothing).  On failure (AHPP_ENOMEM among them) the graph keeps the
+ * shapes it had.  Launches captured before stay valid: the layouts that were in
+ * use keep their memory (a chosen one adds to graph_bytes).  AHPP_EINVAL for a
+ * NULL g or q_sample, an id outside U or a bad eps. */
 int ahpp_autotune(ahpp_graph *g, uint32_t n_sample, const uint32_t *q_sample, double eps);
 
 /* The last ahpp_autotune's measurements as a JSON object text, one entry
@@ -354,6 +356,13 @@ int ahpp_selftest_wait_timeout(int device, int *blocks_gave_up, int *context_ok)
  * the server fails every request with AHPP_ETIMEOUT and stops), and the
  * graph stays usable for the next call.  AHPP_EINVAL for a NULL g. */
 int ahpp_selftest_arm_wait_timeout(ahpp_graph *g);
+
+/* Self-test of running out of device memory (nothing is really exhausted): of
+ * the device allocations made for g from here on, the first `skip` go through
+ * and the next one fails, once, as if memory had run out.  The call that made
+ * it must report AHPP_ENOMEM and leave the graph as it was.  AHPP_EINVAL for a
+ * NULL g. */
+int ahpp_selftest_arm_alloc_failure(ahpp_graph *g, uint32_t skip);
 
 #ifdef __cplusplus
 }

@@ -127,6 +127,7 @@ SIGNATURES = {
     "ahpp_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_int, ctypes.POINTER(ctypes.c_int),
                                                   ctypes.POINTER(ctypes.c_int)]),
     "ahpp_selftest_arm_wait_timeout": (ctypes.c_int, [_vp]),
+    "ahpp_selftest_arm_alloc_failure": (ctypes.c_int, [_vp, ctypes.c_uint32]),
 }
 
 
@@ -333,6 +334,11 @@ class Graph:
         grid barrier that can never fill, so its call reports AHPP_ETIMEOUT
         after about a second (ahpp_selftest_arm_wait_timeout)."""
         _check(lib().ahpp_selftest_arm_wait_timeout(self._h))
+
+    def arm_alloc_failure(self, skip: int) -> None:
+        """Self-test: after `skip` more, one device allocation of this graph
+        fails as if memory had run out (ahpp_selftest_arm_alloc_failure)."""
+        _check(lib().ahpp_selftest_arm_alloc_failure(self._h, skip))
 
     def autotune(self, q_sample, eps: float) -> dict:
         q = np.ascontiguousarray(q_sample, np.uint32)

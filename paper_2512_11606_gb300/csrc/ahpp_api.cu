@@ -109,7 +109,7 @@ Q1Params q1_params(const ahpp_graph* g, uint32_t q_new, double eps) {
   p.max_rounds = g->cfg.max_rounds ? g->cfg.max_rounds : auto_rounds(p.eps_f, g->cfg.alpha);
   p.dense_div = g->q1_dense_div;
   p.n_split = g->n_split1;
-  p.smem_bytes = g->q1_smem;
+  p.smem_bytes = g->q1_layouts.cur->smem;
   return p;
 }
 
@@ -159,7 +159,7 @@ int barrier_status(const GridBarrier* bars, uint32_t n, cudaStream_t stream, int
 
 int launch_single(const ahpp_graph* g, const Q1State& s, const Q1Params& p, cudaStream_t stream) {
   if (g->cl.n_blocks) return launch_cluster(g->dg, g->cl, s, p, stream);
-  return launch_query1(g->dg, s, p, g->bf16, g->q1_grid, stream);
+  return launch_query1(g->dg, s, p, g->bf16, (int)g->q1_layouts.cur->grid, stream);
 }
 
 int run_query1_launch(ahpp_graph* g, uint32_t q_new, double eps, cudaStream_t stream) {
@@ -202,6 +202,31 @@ int run_lambda(ahpp_graph* g) {
   // term |U| (1-alpha)^T is added exactly as in Theorem 3.
   g->lambda = (double)maxpi * (1.0 + 1e-4) + (double)g->n_u * std::pow(1.0 - alpha, (double)T);
   return AHPP_OK;
+}
+
+Layout::~Layout() {
+  for (void* p : bufs) cudaFree(p);
+  g->graph_bytes -= bytes;
+}
+
+void* Layout::put(size_t n, const void* src) {
+  void* p = nullptr;
+  const size_t size = std::max<size_t>(n, 16);
+  if (g->dev_malloc(&p, size) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  bufs.push_back(p);
+  bytes += size;
+  g->graph_bytes += size;
+  return src && upload(g, p, src, n) != cudaSuccess ? nullptr : p;
+}
+
+void settle_layouts(ahpp_graph* g) {
+  g->q1_layouts.cur->kept = true;
+  g->q1_layouts.drop();
+  g->tile_layouts.cur->kept = true;
+  g->tile_layouts.drop();
 }
 
 int batch_plan(ahpp_graph* g) {
@@ -344,9 +369,14 @@ int run_single_device(ahpp_graph* g, uint32_t q, double eps, uint32_t k, uint32_
 
 using namespace ahpp;
 
+cudaError_t ahpp_graph::dev_malloc(void** p, size_t bytes) {
+  if (alloc_trap.load() >= 0 && alloc_trap.fetch_sub(1) == 0) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
 void* ahpp_graph::alloc(size_t bytes) {
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+  if (dev_malloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
     bufs.push_back({nullptr, bytes});
     return nullptr;
@@ -478,8 +508,8 @@ void ahpp_free_graph(ahpp_graph* g) {
   if (!g) return;
   cudaSetDevice(g->device);
   if (g->stream) cudaStreamSynchronize(g->stream);
-  for (void* p : g->q1_layout_bufs) cudaFree(p);
-  for (void* p : g->tile_layout_bufs) cudaFree(p);
+  g->q1_layouts.all.clear();
+  g->tile_layouts.all.clear();
   g->release_all();
   if (g->host_out) cudaFreeHost(g->host_out);
   if (g->stream) cudaStreamDestroy(g->stream);
@@ -504,8 +534,8 @@ int ahpp_get_graph_info(const ahpp_graph* g, ahpp_graph_info* info) {
   info->batch_chunk = kChunkSizes[g->dg.tl.chunk];
   info->single_dense_div = g->q1_dense_div;
   info->single_attr_push = 1;
-  info->single_vec_width = g->q1_vw_max;
-  info->single_smem_bytes = g->q1_smem;
+  info->single_vec_width = g->q1_layouts.cur->vw;
+  info->single_smem_bytes = g->q1_layouts.cur->smem;
   return AHPP_OK;
 }
 
@@ -827,21 +857,18 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     }
     return set(best_v);
   };
-  const uint32_t saved_groups = g->batch_groups, saved_chunk = g->dg.tl.chunk, saved_tile = g->batch_tile;
+  // the shapes in use, which come back if anything fails (their layouts are kept)
+  const uint32_t saved_groups = g->batch_groups, saved_tile = g->batch_tile, saved_div = g->q1_dense_div;
+  TileBuilt* const saved_tiles = g->tile_layouts.cur;
+  Q1Built* const saved_rows = g->q1_layouts.cur;
   rc = tune_batch("batch_tile", [&](uint32_t v) { g->batch_tile = v; return AHPP_OK; }, {(uint32_t)kTile, (uint32_t)kTileNarrow});
   if (rc == AHPP_OK)
-    rc = tune_batch("batch_chunk_choice", [&](uint32_t v) { return build_tile_layout(g, v); }, {1u, 0u, 2u});
+    rc = tune_batch("batch_chunk_choice", [&](uint32_t v) { return use_tile_layout(g, v); }, {1u, 0u, 2u});
   if (rc == AHPP_OK) rc = tune_batch("batch_groups", [&](uint32_t v) { g->batch_groups = v; return AHPP_OK; }, {0u, 1u, 2u, 4u});
-  if (rc != AHPP_OK) {
-    g->batch_groups = saved_groups;
-    build_tile_layout(g, saved_chunk);
-    g->batch_tile = saved_tile;
-    return rc;
-  }
   // ---- single-query path (up to four sample queries, one warm-up pass):
   // the frontier fraction 1/dense_div at which rounds switch from push to pull
   std::vector<uint32_t> q1(q_sample, q_sample + std::min<uint32_t>(n_sample, 4));
-  if ((rc = time_single(g, q1, eps, &ms)) != AHPP_OK) return rc;
+  if (rc == AHPP_OK) rc = time_single(g, q1, eps, &ms);
   auto tune_single = [&](const char* knob, auto set, const std::vector<uint32_t>& values) -> int {
     float best = -1.f;
     uint32_t best_v = values[0];
@@ -854,15 +881,19 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     }
     return set(best_v);
   };
-  const uint32_t saved_div = g->q1_dense_div, saved_vw = g->q1_vw_max;
-  if (!g->cl.n_blocks) rc = tune_single("single_vec_width", [&](uint32_t v) { return build_q1_layout(g, v); }, {32u, 8u, 2u, 1u});
+  if (rc == AHPP_OK && !g->cl.n_blocks)
+    rc = tune_single("single_vec_width", [&](uint32_t v) { return use_q1_layout(g, v); }, {32u, 8u, 2u, 1u});
   if (rc == AHPP_OK)
     rc = tune_single("single_dense_div", [&](uint32_t v) { g->q1_dense_div = v; return AHPP_OK; }, {32u, 8u, 16u, 64u, 128u});
   if (rc != AHPP_OK) {
+    g->batch_groups = saved_groups;
+    g->batch_tile = saved_tile;
     g->q1_dense_div = saved_div;
-    build_q1_layout(g, saved_vw);
-    return rc;
+    use_tile_layout(g, saved_tiles);
+    use_q1_layout(g, saved_rows);
   }
+  settle_layouts(g);
+  if (rc != AHPP_OK) return rc;
   g->tune_log = log + "}";
   return AHPP_OK;
 }

@@ -373,7 +373,7 @@ int alloc_query_state(ahpp_graph* g) {
   const int max_blocks = query1_max_grid(g->sm_count, kQ1SmemMax);
   if (max_blocks <= 0) { set_error("ahpp_load_graph: occupancy query failed"); return AHPP_ECUDA; }
   g->q1_max_blocks = (uint32_t)max_blocks;
-  if (int rc = build_q1_layout(g, cfg.single_vec_width)) return rc;
+  if (int rc = use_q1_layout(g, cfg.single_vec_width)) return rc;
   // a lane width asks for the grid kernel, whose rows it is about
   if (!cfg.single_vec_width)
     if (int rc = build_cluster_layout(g)) return rc;
@@ -402,7 +402,8 @@ int alloc_query_state(ahpp_graph* g) {
   }
   AHPP_CUDA(cudaMallocHost((void**)&g->host_out, kOutBytes));
   if (int rc = batch_plan(g)) return rc;
-  if (int rc = build_tile_layout(g, (uint32_t)chunk_choice(cfg.batch_chunk))) return rc;
+  if (int rc = use_tile_layout(g, (uint32_t)chunk_choice(cfg.batch_chunk))) return rc;
+  settle_layouts(g);
   if (cfg.hbm_budget_bytes && g->graph_bytes + g->q1_bytes > cfg.hbm_budget_bytes) {
     set_error("ahpp_load_graph: graph and query state exceed hbm_budget_bytes");
     return AHPP_ENOMEM;

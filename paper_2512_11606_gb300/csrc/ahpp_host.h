@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -73,6 +74,52 @@ static_assert(sizeof(QCtl) <= kOutBits, "control block");
 constexpr size_t kOutBytes = kOutTop + 8 * (size_t)AHPP_MAX_K;
 }  // namespace ahpp
 
+namespace ahpp {
+// A pull layout: its device arrays and what the host keeps of it.  `kept`: a
+// launch that a caller made or captured may hold its addresses.
+struct Layout {
+  ahpp_graph* g;
+  std::vector<void*> bufs;
+  uint64_t bytes = 0;
+  bool kept = false;
+  explicit Layout(ahpp_graph* graph) : g(graph) {}
+  Layout(const Layout&) = delete;
+  Layout& operator=(const Layout&) = delete;
+  ~Layout();
+  // Device memory of the layout, filled from src if given (nullptr on failure).
+  void* put(size_t n, const void* src);
+};
+struct Q1Built : Layout {
+  using Layout::Layout;
+  Q1Layout q;
+  // lanes of the shortest rows, blocks of the grid, shared memory per block
+  uint32_t vw = 0, grid = 0, smem = 0;
+};
+struct TileBuilt : Layout {
+  using Layout::Layout;
+  TileLayout t;
+  // the items' costs (running sums), first units and chunks, and the ranges cut so far
+  struct Cost {
+    std::vector<uint64_t> cost;
+    std::vector<uint32_t> unit;
+    uint32_t n_chunks = 0;
+  } cost[2];
+  struct Cut { uint32_t warps; const uint4* r[2]; };
+  std::vector<Cut> cuts;
+};
+// The layouts of one kind that a graph has; `cur` is the one in use.
+template <typename L>
+struct Layouts {
+  std::vector<std::unique_ptr<L>> all;
+  L* cur = nullptr;
+  // Frees those that nothing may refer to any more.
+  void drop() {
+    for (size_t i = all.size(); i-- > 0;)
+      if (!all[i]->kept && all[i].get() != cur) all.erase(all.begin() + i);
+  }
+};
+}  // namespace ahpp
+
 struct ahpp_graph {
   ahpp_config cfg{};
   int device = 0;
@@ -98,13 +145,9 @@ struct ahpp_graph {
 
   // single-query state
   ahpp::Q1State q1{};
-  int q1_grid = 0;
   ahpp::ClusterLayout cl{};       // small graphs: the layout of the cluster kernel, which then runs them
-  // single-query pull layout (dg.q1): its buffers, the most blocks the device
-  // keeps resident, shared memory per block, lanes of the shortest rows
-  std::vector<void*> q1_layout_bufs;
-  uint64_t q1_layout_bytes = 0;
-  uint32_t q1_max_blocks = 0, q1_smem = 0, q1_vw_max = 0;
+  ahpp::Layouts<ahpp::Q1Built> q1_layouts;   // single-query pull layouts (dg.q1: the current one's)
+  uint32_t q1_max_blocks = 0;     // the most blocks of k_query1 that the device keeps resident
   uint32_t q1_dense_div = 32;     // pull rounds once the frontier covers > 1/dense_div of the edges
   std::string tune_log;           // the last autotune's measurements (JSON object)
   // what a single query leaves for the host, in one block that one copy fetches:
@@ -119,17 +162,7 @@ struct ahpp_graph {
   uint32_t batch_tile = 32, batch_groups = 0;   // groups: 0 = by the graph's size and the batch's
   int bt_grid = 0;
   uint64_t tile_bytes = 0;
-  // batched pull layout (dg.tl): its buffers, the items' costs (running sums),
-  // first units and chunks, and the ranges cut so far
-  std::vector<void*> tile_layout_bufs;
-  uint64_t tile_layout_bytes = 0;
-  struct TileCost {
-    std::vector<uint64_t> cost;
-    std::vector<uint32_t> unit;
-    uint32_t n_chunks = 0;
-  } tile_cost[2];
-  struct TileCut { uint32_t warps; const uint4* r[2]; };
-  std::vector<TileCut> tile_cuts;
+  ahpp::Layouts<ahpp::TileBuilt> tile_layouts;   // batched pull layouts (dg.tl: the current one's)
 
   // top-k scratch
   void* topk_scratch = nullptr;
@@ -138,8 +171,11 @@ struct ahpp_graph {
   // failure-detection self-test: the next launch's grid barriers start with
   // a counter that can never reach the block count (see reset_barrier)
   std::atomic<int> wait_trap{0};
+  // and the allocation after this many more fails (< 0: none does)
+  std::atomic<int64_t> alloc_trap{-1};
 
-  void* alloc(size_t bytes);          // cudaMalloc + track (nullptr on failure)
+  cudaError_t dev_malloc(void** p, size_t bytes);   // every device allocation of the graph
+  void* alloc(size_t bytes);          // the same, tracked (nullptr on failure)
   void release_all();
 };
 
@@ -161,18 +197,23 @@ int barrier_status(const GridBarrier* bars, uint32_t n, cudaStream_t stream, int
 int build_graph(const ahpp_graph_desc* desc, ahpp_graph* g);
 // The kernels' algorithm id of an AHPP_* constant (-1 if none).
 int kernel_algo(int algo);
-// Sliced layout of the single-query pull rounds with at least vec_width lanes
-// per row (0: by the graph's size); replaces the one the graph has.
-int build_q1_layout(ahpp_graph* g, uint32_t vec_width);
+// Makes the sliced layout of the single-query pull rounds with at least vec_width
+// lanes per row (0: by the graph's size) the current one: one that the graph has,
+// else a new one.  On failure the current one stays.
+int use_q1_layout(ahpp_graph* g, uint32_t vec_width);
+void use_q1_layout(ahpp_graph* g, Q1Built* b);
 int build_cluster_layout(ahpp_graph* g);
 // A single query's launch, on the cluster kernel where the graph has its layout.
 int launch_single(const ahpp_graph* g, const Q1State& s, const Q1Params& p, cudaStream_t stream);
 // Index into kChunkSizes of a configured chunk size (0: the default), -1 if
 // it is not one of them.
 int chunk_choice(uint32_t chunk);
-// Sliced layout of the batched pull rounds with chunks of kChunkSizes[choice]
-// entries; replaces the one the graph has.
-int build_tile_layout(ahpp_graph* g, uint32_t choice);
+// The same for the batched pull rounds, with chunks of kChunkSizes[choice] entries.
+int use_tile_layout(ahpp_graph* g, uint32_t choice);
+void use_tile_layout(ahpp_graph* g, TileBuilt* b);
+// The current layouts are those that calls work on from here on; candidates that
+// none did are freed.
+void settle_layouts(ahpp_graph* g);
 // The items' ranges for a tile on `warps` warps (made on first use).
 int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u);
 // Blocks of the batched grid that work on one tile, of n_tiles to be run: all of

@@ -294,16 +294,26 @@ Block make_block(uint32_t b, uint32_t r0, uint32_t r1, const std::vector<uint32_
   return B;
 }
 
-}  // namespace
+// Blocks of the grid and lanes per short row.
+void shape_of(const ahpp_graph* g, uint32_t vec_width, uint32_t* grid, uint32_t* lanes) {
+  const DevGraph& G = g->dg;
+  // the barrier costs the same from 8 blocks on, so a step of phase 2 is dealt to
+  // every fourth warp at least
+  const uint64_t steps = ((uint64_t)G.n_e + G.n_ea) / kStep + 1;
+  const uint32_t nb = (uint32_t)std::min<uint64_t>(g->q1_max_blocks, std::max<uint64_t>(8, 4 * steps / kQ1Warps));
+  // lanes per short row: one (16,000 nodes: 1.77 ms a query with eight lanes, 1.69
+  // with one; 44,000: 2.62, 1.70; 100,000: 2.94, 2.64), unless that leaves the
+  // warps a long slice of U rows or two each (200,000 nodes of 40 entries: 5.35 with
+  // one, 4.89 with two; 277,000 of 36: 10.0, 9.28; but 176,000 of 22: 3.86, 4.85)
+  const uint64_t slices = G.n_u / 32, warps = (uint64_t)nb * kQ1Warps;
+  const bool uneven = slices > warps && 10 * slices < 19 * warps;
+  *grid = nb;
+  *lanes = vec_width ? vec_width : uneven && (uint64_t)G.n_e + G.n_ea >= 30ull * G.n_u ? 2 : 1;
+}
 
-int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
-  DevGraph& G = g->dg;
-  Q1Layout& Q = G.q1;
-  for (void* p : g->q1_layout_bufs) cudaFree(p);
-  g->q1_layout_bufs.clear();
-  g->graph_bytes -= g->q1_layout_bytes;
-  g->q1_layout_bytes = 0;
-  Q = Q1Layout();
+int build_q1_layout(ahpp_graph* g, Q1Built* b) {
+  const DevGraph& G = g->dg;
+  Q1Layout& Q = b->q;
   const uint32_t nU = G.n_u, nV = G.n_v, nA = G.n_a;
   auto down = [&](std::vector<uint32_t>& v, const uint32_t* p, size_t n) {
     v.resize(n);
@@ -323,22 +333,10 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   Q.compact_s = g->bf16;
   const uint32_t a_units = Q.compact_a ? 1 : 2, s_units = Q.compact_s ? 1 : 2;
 
-  // blocks of the grid: the barrier costs the same from 8 blocks on, so a step
-  // of phase 2 is dealt to every fourth warp at least
-  const uint64_t steps = ((uint64_t)G.n_e + G.n_ea) / kStep + 1;
-  const uint32_t nb = (uint32_t)std::min<uint64_t>(g->q1_max_blocks, std::max<uint64_t>(8, 4 * steps / kQ1Warps));
+  const uint32_t nb = b->grid;
   Q.n_warps = nb * kQ1Warps;
-  g->q1_grid = (int)nb;
-  // lanes per short row: one (16,000 nodes: 1.77 ms a query with eight lanes, 1.69
-  // with one; 44,000: 2.62, 1.70; 100,000: 2.94, 2.64), unless that leaves the
-  // warps a long slice of U rows or two each (200,000 nodes of 40 entries: 5.35 with
-  // one, 4.89 with two; 277,000 of 36: 10.0, 9.28; but 176,000 of 22: 3.86, 4.85)
-  const uint64_t slices = nU / 32;
-  const bool uneven = slices > Q.n_warps && 10 * slices < 19 * (uint64_t)Q.n_warps;
-  const uint32_t vw = vec_width ? vec_width : uneven && (uint64_t)G.n_e + G.n_ea >= 30ull * nU ? 2 : 1;
-  g->q1_vw_max = vw;
   uint32_t lg_min = 0;
-  while ((1u << lg_min) < vw) ++lg_min;
+  while ((1u << lg_min) < b->vw) ++lg_min;
   // a lane's walk of a V row: at most half the steps a warp has in the phase, so
   // that the warps' shares can be cut evenly (2M edges: phase 1 from 38,000 to
   // 35,000 cycles); U items and segments, with more to do at their ends, are
@@ -364,7 +362,7 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   }
   const uint32_t n_vb = (uint32_t)vb.size();
   uint32_t own = 0;
-  for (const uint2& b : vb) own = std::max(own, b.y);
+  for (const uint2& x : vb) own = std::max(own, x.y);
 
   // shared memory: t_A first (every U row looks it up), then the leading
   // entries of t_V and p that are looked up often enough by each SM to repay
@@ -379,7 +377,7 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   Q.hub_u = std::min(leading(nU, lv), kTableFloats - Q.s.own_cap) / 4 * 4;
   Q.hub_a = std::min(nA, kTaEntries);
   Q.hub_v = std::min(leading(nV, lw), kTableFloats - (Q.hub_a + 3) / 4 * 4) / 4 * 4;
-  g->q1_smem = kQ1RingBytes + 4 * std::max(Q.s.own_cap + Q.hub_u, (Q.hub_a + 3) / 4 * 4 + Q.hub_v);
+  b->smem = kQ1RingBytes + 4 * std::max(Q.s.own_cap + Q.hub_u, (Q.hub_a + 3) / 4 * 4 + Q.hub_v);
 
   HostRows hv, hu;
   {
@@ -390,8 +388,8 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
     t.join();
   }
   std::vector<Block> blk(n_vb);
-  over_threads(n_vb, [&](uint32_t b) {
-    blk[b] = make_block(b, vb[b].x, vb[b].x + vb[b].y, au, au_idx, s_units);
+  over_threads(n_vb, [&](uint32_t i) {
+    blk[i] = make_block(i, vb[i].x, vb[i].x + vb[i].y, au, au_idx, s_units);
   });
   // copies of t_A: at least 16 blocks to a copy (with 39 blocks, eight copies to
   // add up in phase 2 cost 4 % of the query), and few enough attributes that all
@@ -399,24 +397,20 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   Q.ta_copies = std::max(1u, std::min({kTaCopies, 8192u / std::max(nA, 1u), n_vb / 16}));
   std::vector<uint4> segs, sitems, sranges;
   uint32_t total_s = 0;
-  for (uint32_t b = 0; b < n_vb; ++b) {
+  for (uint32_t k = 0; k < n_vb; ++k) {
     const uint32_t s0 = (uint32_t)segs.size(), i0 = (uint32_t)sitems.size();
-    for (auto x : blk[b].segs) { x.x += b % Q.ta_copies * nA; segs.push_back(x); }
-    for (auto x : blk[b].items) { x.x += s0; x.z += total_s; sitems.push_back(x); }
-    for (auto& x : blk[b].ranges) sranges.push_back(make_uint4(x.x + i0, x.y + i0, x.z + total_s, x.w + total_s));
-    total_s += blk[b].units;
-    blk[b] = Block();
+    for (auto x : blk[k].segs) { x.x += k % Q.ta_copies * nA; segs.push_back(x); }
+    for (auto x : blk[k].items) { x.x += s0; x.z += total_s; sitems.push_back(x); }
+    for (auto& x : blk[k].ranges) sranges.push_back(make_uint4(x.x + i0, x.y + i0, x.z + total_s, x.w + total_s));
+    total_s += blk[k].units;
+    blk[k] = Block();
   }
 
   // ---- device arrays
   bool ok = true;
   auto dev = [&](size_t bytes, const void* src) -> void* {
-    void* p = nullptr;
-    const size_t n = std::max<size_t>(bytes, 16);
-    if (cudaMalloc(&p, n) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
-    g->q1_layout_bufs.push_back(p);
-    g->q1_layout_bytes += n;
-    if (src && upload(g, p, src, bytes) != cudaSuccess) ok = false;
+    void* p = b->put(bytes, src);
+    ok = ok && p;
     return p;
   };
   auto put = [&](auto& v) -> void* { return dev(v.size() * sizeof(v[0]), v.data()); };
@@ -424,7 +418,7 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   auto scratch = [&](auto& v) -> void* {
     void* p = nullptr;
     const size_t n = v.size() * sizeof(v[0]);
-    if (cudaMalloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
+    if (g->dev_malloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
     tmp.push_back(p);
     if (upload(g, p, v.data(), n) != cudaSuccess) ok = false;
     return p;
@@ -495,9 +489,28 @@ int build_q1_layout(ahpp_graph* g, uint32_t vec_width) {
   const cudaError_t e = cudaStreamSynchronize(g->stream);
   const cudaError_t le = cudaGetLastError();
   for (void* p : tmp) cudaFree(p);
-  g->graph_bytes += g->q1_layout_bytes;
   if (e != cudaSuccess || le != cudaSuccess) return cuda_fail(e != cudaSuccess ? e : le, "single-query layout");
   if (!ok) { set_error("single-query layout: device allocation failed"); return AHPP_ENOMEM; }
+  return AHPP_OK;
+}
+
+}  // namespace
+
+void use_q1_layout(ahpp_graph* g, Q1Built* b) {
+  g->q1_layouts.cur = b;
+  g->dg.q1 = b->q;
+}
+
+int use_q1_layout(ahpp_graph* g, uint32_t vec_width) {
+  Layouts<Q1Built>& L = g->q1_layouts;
+  L.drop();
+  std::unique_ptr<Q1Built> b(new Q1Built(g));
+  shape_of(g, vec_width, &b->grid, &b->vw);
+  for (auto& x : L.all)
+    if (x->vw == b->vw) { use_q1_layout(g, x.get()); return AHPP_OK; }
+  if (int rc = build_q1_layout(g, b.get())) return rc;
+  L.all.push_back(std::move(b));
+  use_q1_layout(g, L.all.back().get());
   return AHPP_OK;
 }
 

@@ -79,3 +79,13 @@ extern "C" int ahpp_selftest_arm_wait_timeout(ahpp_graph* g) {
   g->wait_trap.store(1);
   return AHPP_OK;
 }
+
+// Arms the graph's allocation trap (see ahpp_graph::dev_malloc).
+extern "C" int ahpp_selftest_arm_alloc_failure(ahpp_graph* g, uint32_t skip) {
+  if (!g) {
+    set_error("ahpp_selftest_arm_alloc_failure: null graph");
+    return AHPP_EINVAL;
+  }
+  g->alloc_trap.store(skip);
+  return AHPP_OK;
+}

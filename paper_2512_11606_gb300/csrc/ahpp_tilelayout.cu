@@ -140,23 +140,14 @@ __global__ void k_fill_tiles(const uint4* items, const Piece* pieces, uint32_t n
   }
 }
 
-}  // namespace
-
-int build_tile_layout(ahpp_graph* g, uint32_t choice) {
-  DevGraph& G = g->dg;
-  TileLayout& T = G.tl;
-  for (void* p : g->tile_layout_bufs) cudaFree(p);
-  g->tile_layout_bufs.clear();
-  g->tile_cuts.clear();
-  g->graph_bytes -= g->tile_layout_bytes;
-  g->tile_layout_bytes = 0;
-  T = TileLayout();
-  T.chunk = choice;
+int build_tile_layout(ahpp_graph* g, TileBuilt* b) {
+  const DevGraph& G = g->dg;
+  TileLayout& T = b->t;
   // a chunk is walked by one warp: on a small graph the configured size would be
   // more than the warps' shares
   uint32_t fine = 64;
   while (fine < 512 && (uint64_t)fine * 16 * g->bt_grid * kBWarps < (uint64_t)G.n_e + G.n_ea) fine *= 2;
-  const uint32_t nU = G.n_u, nV = G.n_v, nA = G.n_a, chunk = std::min(kChunkSizes[choice], fine);
+  const uint32_t nU = G.n_u, nV = G.n_v, nA = G.n_a, chunk = std::min(kChunkSizes[T.chunk], fine);
   auto down = [&](std::vector<uint32_t>& v, const uint32_t* p, size_t n) {
     v.resize(n);
     return cudaMemcpy(v.data(), p, 4 * n, cudaMemcpyDeviceToHost) == cudaSuccess;
@@ -205,12 +196,8 @@ int build_tile_layout(ahpp_graph* g, uint32_t choice) {
 
   bool ok = true;
   auto dev = [&](size_t bytes, const void* src) -> void* {
-    void* p = nullptr;
-    const size_t n = std::max<size_t>(bytes, 16);
-    if (cudaMalloc(&p, n) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
-    g->tile_layout_bufs.push_back(p);
-    g->tile_layout_bytes += n;
-    if (src && upload(g, p, src, bytes) != cudaSuccess) ok = false;
+    void* p = b->put(bytes, src);
+    ok = ok && p;
     return p;
   };
   auto put = [&](auto& v) -> void* { return dev(v.size() * sizeof(v[0]), v.data()); };
@@ -218,7 +205,7 @@ int build_tile_layout(ahpp_graph* g, uint32_t choice) {
   auto scratch = [&](auto& v) -> void* {
     void* p = nullptr;
     const size_t n = v.size() * sizeof(v[0]);
-    if (cudaMalloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
+    if (g->dev_malloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
     tmp.push_back(p);
     if (upload(g, p, v.data(), n) != cudaSuccess) ok = false;
     return p;
@@ -239,7 +226,7 @@ int build_tile_layout(ahpp_graph* g, uint32_t choice) {
       ok = cudaStreamSynchronize(g->stream) == cudaSuccess &&
            cudaMemcpy(cost.data(), d_cost, 4ull * n, cudaMemcpyDeviceToHost) == cudaSuccess;
     }
-    ahpp_graph::TileCost& c = g->tile_cost[which];
+    TileBuilt::Cost& c = b->cost[which];
     c.n_chunks = h.n_chunks;
     c.unit.clear();
     for (const uint4& x : h.items) c.unit.push_back(x.w);
@@ -263,21 +250,41 @@ int build_tile_layout(ahpp_graph* g, uint32_t choice) {
   T.chunks_of = (const uint32_t*)put(chunks_of);
   const cudaError_t e = cudaStreamSynchronize(g->stream), le = cudaGetLastError();
   for (void* p : tmp) cudaFree(p);
-  g->graph_bytes += g->tile_layout_bytes;
   if (e != cudaSuccess || le != cudaSuccess) return cuda_fail(e != cudaSuccess ? e : le, "batched layout");
   if (!ok) { set_error("batched layout: device allocation failed"); return AHPP_ENOMEM; }
   return AHPP_OK;
 }
 
+}  // namespace
+
+void use_tile_layout(ahpp_graph* g, TileBuilt* b) {
+  g->tile_layouts.cur = b;
+  g->dg.tl = b->t;
+}
+
+int use_tile_layout(ahpp_graph* g, uint32_t choice) {
+  Layouts<TileBuilt>& L = g->tile_layouts;
+  L.drop();
+  for (auto& x : L.all)
+    if (x->t.chunk == choice) { use_tile_layout(g, x.get()); return AHPP_OK; }
+  std::unique_ptr<TileBuilt> b(new TileBuilt(g));
+  b->t.chunk = choice;
+  if (int rc = build_tile_layout(g, b.get())) return rc;
+  L.all.push_back(std::move(b));
+  use_tile_layout(g, L.all.back().get());
+  return AHPP_OK;
+}
+
 int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u) {
-  for (const auto& c : g->tile_cuts)
+  TileBuilt* const b = g->tile_layouts.cur;
+  for (const auto& c : b->cuts)
     if (c.warps == warps) { *t = c.r[0]; *u = c.r[1]; return AHPP_OK; }
-  ahpp_graph::TileCut cut{warps, {nullptr, nullptr}};
+  TileBuilt::Cut cut{warps, {nullptr, nullptr}};
   for (int k = 0; k < 2; ++k) {
     // chunks evenly, then the slices before the pool so that every warp's cost is
     // about the same: {chunk begin, end, slice begin, end}, and the first units
     // of those four
-    const ahpp_graph::TileCost& c = g->tile_cost[k];
+    const TileBuilt::Cost& c = b->cost[k];
     const uint32_t n = k ? g->dg.tl.u.pool : g->dg.tl.t.pool;
     std::vector<uint4> r;
     uint32_t i = c.n_chunks;
@@ -295,20 +302,13 @@ int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u)
       r.push_back(make_uint4(c0, c1, i0, i));
       r.push_back(make_uint4(c.unit[c0], c.unit[c1], c.unit[i0], c.unit[i]));
     }
-    const size_t bytes = r.size() * sizeof(uint4);
-    void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
+    cut.r[k] = (const uint4*)b->put(r.size() * sizeof(uint4), r.data());
+    if (!cut.r[k]) {
       set_error("batched ranges: device allocation failed");
       return AHPP_ENOMEM;
     }
-    g->tile_layout_bufs.push_back(p);
-    g->tile_layout_bytes += bytes;
-    g->graph_bytes += bytes;
-    AHPP_CUDA(upload(g, p, r.data(), bytes));
-    cut.r[k] = (const uint4*)p;
   }
-  g->tile_cuts.push_back(cut);
+  b->cuts.push_back(cut);
   *t = cut.r[0];
   *u = cut.r[1];
   return AHPP_OK;

@@ -118,12 +118,17 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
     if (e != cudaSuccess || !ptr) return cuda_fail(e, "ahpp_query_dense_noalloc: cudaGetSymbolAddress");
     g_noalloc_ptr[g->device] = ptr;
   }
-  carve(g, (char*)g_noalloc_ptr[g->device], &s);
   cudaStream_t st = stream ? (cudaStream_t)stream : g->stream;
-  Q1Params p = noalloc_params(g, g->h_u_old2new[q], eps);
-  if (int rc = reset_barriers(g, s.bar, 1, st)) return rc;
-  const int e = launch_single(g, s, p, st);
-  if (e) return cuda_fail((cudaError_t)e, "ahpp_query_dense_noalloc: launch");
+  {
+    // the layout that the launch is given is one that the graph keeps: the
+    // autotuner, which tries others and frees them, holds this lock throughout
+    std::lock_guard<std::mutex> glock(g->mu);
+    carve(g, (char*)g_noalloc_ptr[g->device], &s);
+    Q1Params p = noalloc_params(g, g->h_u_old2new[q], eps);
+    if (int rc = reset_barriers(g, s.bar, 1, st)) return rc;
+    const int e = launch_single(g, s, p, st);
+    if (e) return cuda_fail((cudaError_t)e, "ahpp_query_dense_noalloc: launch");
+  }
   k_scatter_out<<<std::max(1, g->sm_count * 4), 256, 0, st>>>(s.pi, g->d_u_new2old, (uint32_t)g->n_u,
                                                               d_out_pi);
   AHPP_CUDA(cudaGetLastError());

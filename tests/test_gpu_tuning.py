@@ -56,3 +56,40 @@ def test_a_build_that_runs_out_of_memory_changes_nothing(ahpp, arrays):
     finally:
         G.arm_alloc_failure(1 << 30)
         G.close()
+
+
+def test_no_allocation_queries_while_another_thread_tunes(ahpp, arrays):
+    """Every launch works on a layout that stays, whatever the autotuner tries
+    and frees meanwhile."""
+    import threading
+
+    torch = pytest.importorskip("torch")
+    og = oracle.OracleGraph.from_arrays(arrays)
+    lam, _ = og.lambda_estimate(ALPHA, BETA)
+    G = ahpp.Graph.from_arrays(arrays, lam=lam, attr_bf16=0)
+    try:
+        qs = [int(x) for x in synth.draw_queries(arrays.n_u, 16, seed=33)]
+        ref = og.push("asrp", ALPHA, BETA, qs[1], EPS, lam=lam).pi
+        out = torch.empty(arrays.n_u, dtype=torch.float32, device="cuda")
+        G.query_dense_noalloc(qs[1], EPS, out)
+        failed = []
+
+        def tune():
+            try:
+                G.autotune(qs, EPS)
+            except Exception as e:  # noqa: BLE001
+                failed.append(e)
+
+        t = threading.Thread(target=tune)
+        t.start()
+        calls = 0
+        while t.is_alive() or calls < 3:
+            out.fill_(-1.0)
+            torch.cuda.synchronize()
+            assert G.query_dense_noalloc(qs[1], EPS, out) == 0
+            assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= TOL
+            calls += 1
+        t.join()
+        assert not failed
+    finally:
+        G.close()

@@ -89,9 +89,10 @@ typedef struct {
     uint32_t max_rounds;       /* round cap per query; 0: automatic */
     uint32_t batch_tile;       /* queries per batched tile: 16 or 32; 0: 32 (ahpp_autotune picks one);
                                   serving always uses tiles of 32 */
-    uint32_t batch_groups;     /* tiles processed concurrently, 1..8; 0: as many as share the GPU well,
-                                  by the graph's size and the batch's (ahpp_autotune keeps that or
-                                  picks 1, 2 or 4) */
+    uint32_t batch_groups;     /* tiles processed concurrently, 1..8 (no more than a batch has); 0: as
+                                  many as share the GPU well, by the graph's size and the batch's
+                                  (ahpp_autotune keeps that or picks 1, 2 or 4).  A server's steps
+                                  follow that rule, with a number given here as its limit */
     uint32_t batch_chunk;      /* entries per chunk of a long row in the batched kernel, at most: 128,
                                   256 or 512 (less on graphs too small for it); 0: 256
                                   (ahpp_autotune picks one) */

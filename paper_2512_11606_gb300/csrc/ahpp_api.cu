@@ -311,7 +311,7 @@ int run_batch_launch(ahpp_graph* g, uint32_t n, const uint32_t* d_q, const doubl
                      uint32_t* d_n, ahpp_stats* d_stats, float* d_dense, cudaStream_t stream) {
   int rc = batch_plan(g);
   if (rc) return rc;
-  const uint32_t groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile);
+  const uint32_t groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile, false);
   if ((rc = ensure_batch(g, groups, kmax))) return rc;
   BatchParams p;
   const uint32_t per_group = (uint32_t)g->bt_grid / groups;

@@ -16,6 +16,7 @@
 #include "ahpp_query1.cuh"
 #include "ahpp_batch.cuh"
 #include "ahpp_cluster.cuh"
+#include "ahpp_groups.h"
 
 namespace ahpp {
 
@@ -216,9 +217,8 @@ void use_tile_layout(ahpp_graph* g, TileBuilt* b);
 void settle_layouts(ahpp_graph* g);
 // The items' ranges for a tile on `warps` warps (made on first use).
 int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u);
-// Blocks of the batched grid that work on one tile, of n_tiles to be run: all of
-// them, or fewer where several small tiles run at once.
-uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles);
+// Tiles that run at once, of n_tiles to be run (see groups_of).
+uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles, bool serving);
 int alloc_query_state(ahpp_graph* g);
 int run_lambda(ahpp_graph* g);
 int run_query1(ahpp_graph* g, uint32_t q_new, double eps, uint32_t lambda_T_mode,

@@ -207,7 +207,7 @@ int server_step(ahpp_server* s) {
   AHPP_CUDA(cudaMemcpyAsync(s->d_slots, s->h_slots, sizeof(SlotState) * s->n_slots,
                             cudaMemcpyHostToDevice, s->stream));
   AHPP_CUDA(cudaMemcpyAsync(s->d_live, live.data(), 4 * live.size(), cudaMemcpyHostToDevice, s->stream));
-  const uint32_t groups = tile_groups(g, (uint32_t)live.size()), per_group = (uint32_t)s->grid / groups;
+  const uint32_t groups = tile_groups(g, (uint32_t)live.size(), true), per_group = (uint32_t)s->grid / groups;
   if (int rc = reset_barriers(g, s->d_bar, groups, s->stream)) return rc;
   BatchParams p;
   p.kmax = s->kmax;

@@ -314,17 +314,10 @@ int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u)
   return AHPP_OK;
 }
 
-uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles) {
-  const uint32_t most = std::min<uint32_t>(kMaxGroups, (uint32_t)std::max(1, g->bt_grid));
-  if (g->batch_groups) return std::min(g->batch_groups, most);
-  // tiles that run at once share L2: their gathered tables stay within its size
-  // (100k nodes, 20 MB a tile: 106 us a tile and round one at a time, 91 with
-  // two, 84 with four; 300k nodes, 60 MB: 270 with one or two)
+uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles, bool serving) {
   const uint64_t table = 128ull * ((uint64_t)g->n_u + g->n_v + 2ull * g->dg.tl.n_acc);
-  const uint64_t fit = std::max<uint64_t>(1, (128ull << 20) / std::max<uint64_t>(table, 1));
-  const uint32_t at_once = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({most, n_tiles, fit}));
-  const uint32_t waves = (n_tiles + at_once - 1) / at_once;
-  return (n_tiles + waves - 1) / waves;    // the same number of waves, evenly
+  return groups_of(g->batch_groups, n_tiles, std::min<uint32_t>(kMaxGroups, (uint32_t)std::max(1, g->bt_grid)), table,
+                   serving);
 }
 
 }  // namespace ahpp

@@ -121,8 +121,9 @@ struct IoBuf {
 
 int ensure(ahpp_graph* g, IoBuf& b, size_t bytes) {
   if (b.bytes >= bytes) return AHPP_OK;
-  b.p = g->alloc(bytes);
-  if (!b.p) { set_error("device allocation failed"); return AHPP_ENOMEM; }
+  void* p = g->alloc(bytes);
+  if (!p) { set_error("device allocation failed"); return AHPP_ENOMEM; }
+  b.p = p;
   b.bytes = bytes;
   return AHPP_OK;
 }

@@ -239,7 +239,11 @@ int ahpp_query_batch_dense(ahpp_graph *g, uint32_t n, const uint32_t *q, const d
  * i * kmax), d_out_n[n]; d_stats (n entries, device) may be NULL.  kmax is
  * the largest k in d_k (at most AHPP_MAX_K).  stream is a cudaStream_t (NULL
  * = the graph's own stream); the call is asynchronous with respect to the
- * host except for internal bookkeeping. */
+ * host except for internal bookkeeping.  Working buffers are allocated by the
+ * first call and by one with a larger kmax, or more tiles than before that can
+ * run at once; without memory for more tiles the call runs with those it has.
+ * It may be captured into a CUDA graph (buffers that it then allocates, like all
+ * others, live as long as g). */
 int ahpp_query_batch_device(ahpp_graph *g, uint32_t n, const uint32_t *d_q, const double *d_eps,
                             const uint32_t *d_k, uint32_t kmax, uint32_t *d_out_nodes,
                             float *d_out_scores, uint32_t *d_out_n, ahpp_stats *d_stats,

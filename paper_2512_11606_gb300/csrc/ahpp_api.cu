@@ -246,6 +246,7 @@ int batch_plan(ahpp_graph* g) {
 int ensure_batch(ahpp_graph* g, uint32_t groups, uint32_t kmax) {
   kmax = std::max<uint32_t>(kmax, 1);
   if (g->bt.n_groups >= groups && g->bt.kmax_cap >= kmax) return AHPP_OK;
+  GrowInCapture grow;
   BatchState s = g->bt;
   const DevGraph& G = g->dg;
   const size_t n_split = std::max(G.tl.split_u_max, 1u);        // any chunk choice fits
@@ -312,11 +313,16 @@ int run_batch_launch(ahpp_graph* g, uint32_t n, const uint32_t* d_q, const doubl
                      uint32_t* d_n, ahpp_stats* d_stats, float* d_dense, cudaStream_t stream) {
   int rc = batch_plan(g);
   if (rc) return rc;
-  const uint32_t groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile, false);
-  if ((rc = ensure_batch(g, groups, kmax))) return rc;
+  // with no memory for so many tiles at once, as many as there are buffers for
+  uint32_t groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile, false), per_group;
+  rc = ensure_batch(g, groups, kmax);
+  if (rc == AHPP_ENOMEM && groups > std::max(1u, g->bt.n_groups)) {
+    groups = std::max(1u, g->bt.n_groups);
+    rc = ensure_batch(g, groups, kmax);
+  }
+  if (rc) return rc;
   BatchParams p;
-  const uint32_t per_group = (uint32_t)g->bt_grid / groups;
-  if ((rc = tile_ranges(g, per_group * kBWarps, &p.ranges_t, &p.ranges_u))) return rc;
+  if ((rc = plan_groups(g, (uint32_t)g->bt_grid, &groups, &per_group, p))) return rc;
   p.n = n;
   p.q = d_q;
   p.eps = d_eps;
@@ -331,7 +337,6 @@ int run_batch_launch(ahpp_graph* g, uint32_t n, const uint32_t* d_q, const doubl
   // one cap for the whole launch: generous enough for eps down to 1e-14 / lambda
   p.max_rounds = g->cfg.max_rounds ? g->cfg.max_rounds
                                    : auto_rounds(1e-14 / std::max(g->lambda, 1.0), g->cfg.alpha);
-  p.groups = groups;
   p.tbufs = g->bt.d_tb;
   p.bars = g->bt.bars;
   p.tile = g->batch_tile;

@@ -181,6 +181,16 @@ struct ahpp_graph {
 };
 
 namespace ahpp {
+// Lets this thread allocate while a stream is being captured (by it or, in the
+// global mode, by any thread): what grows during a call lives as long as the
+// graph, so a launch that is only recorded may hold it.
+struct GrowInCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  GrowInCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~GrowInCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  GrowInCapture(const GrowInCapture&) = delete;
+  GrowInCapture& operator=(const GrowInCapture&) = delete;
+};
 // Host memory to the device, there when this returns: a plain cudaMemcpy from
 // pageable memory may return before its copy has arrived, and the library's
 // streams (and most callers') do not wait for the default stream it is on.
@@ -215,8 +225,12 @@ void use_tile_layout(ahpp_graph* g, TileBuilt* b);
 // The current layouts are those that calls work on from here on; candidates that
 // none did are freed.
 void settle_layouts(ahpp_graph* g);
-// The items' ranges for a tile on `warps` warps (made on first use).
+// The items' ranges for a tile on `warps` warps (made on first use; those of the
+// whole grid's warps with the layout).
 int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u);
+// A launch's groups of `grid` blocks: *groups, or one where there is no memory for
+// the ranges of so many; their blocks each and ranges.
+int plan_groups(ahpp_graph* g, uint32_t grid, uint32_t* groups, uint32_t* per_group, BatchParams& p);
 // Tiles that run at once, of n_tiles to be run (see groups_of).
 uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles, bool serving);
 int alloc_query_state(ahpp_graph* g);

@@ -207,9 +207,13 @@ int server_step(ahpp_server* s) {
   AHPP_CUDA(cudaMemcpyAsync(s->d_slots, s->h_slots, sizeof(SlotState) * s->n_slots,
                             cudaMemcpyHostToDevice, s->stream));
   AHPP_CUDA(cudaMemcpyAsync(s->d_live, live.data(), 4 * live.size(), cudaMemcpyHostToDevice, s->stream));
-  const uint32_t groups = tile_groups(g, (uint32_t)live.size(), true), per_group = (uint32_t)s->grid / groups;
-  if (int rc = reset_barriers(g, s->d_bar, groups, s->stream)) return rc;
   BatchParams p;
+  uint32_t groups = tile_groups(g, (uint32_t)live.size(), true), per_group;
+  {
+    std::lock_guard<std::mutex> glock(g->mu);
+    if (int rc = plan_groups(g, (uint32_t)s->grid, &groups, &per_group, p)) return rc;
+  }
+  if (int rc = reset_barriers(g, s->d_bar, groups, s->stream)) return rc;
   p.kmax = s->kmax;
   p.out_nodes = s->d_nodes;
   p.out_scores = s->d_scores;
@@ -217,13 +221,8 @@ int server_step(ahpp_server* s) {
   p.out_stats = s->d_stats;
   set_batch_params(g, p);
   p.max_rounds = g->cfg.max_rounds ? g->cfg.max_rounds : 100000u;
-  p.groups = groups;
   p.tbufs = s->d_tbufs;
   p.bars = s->d_bar;
-  {
-    std::lock_guard<std::mutex> glock(g->mu);
-    if (int rc = tile_ranges(g, per_group * kBWarps, &p.ranges_t, &p.ranges_u)) return rc;
-  }
   ServeParams sv;
   sv.slots = s->d_slots;
   sv.tile_round = s->d_tile_round;

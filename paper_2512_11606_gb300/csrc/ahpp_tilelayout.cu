@@ -255,38 +255,17 @@ int build_tile_layout(ahpp_graph* g, TileBuilt* b) {
   return AHPP_OK;
 }
 
-}  // namespace
-
-void use_tile_layout(ahpp_graph* g, TileBuilt* b) {
-  g->tile_layouts.cur = b;
-  g->dg.tl = b->t;
-}
-
-int use_tile_layout(ahpp_graph* g, uint32_t choice) {
-  Layouts<TileBuilt>& L = g->tile_layouts;
-  L.drop();
-  for (auto& x : L.all)
-    if (x->t.chunk == choice) { use_tile_layout(g, x.get()); return AHPP_OK; }
-  std::unique_ptr<TileBuilt> b(new TileBuilt(g));
-  b->t.chunk = choice;
-  if (int rc = build_tile_layout(g, b.get())) return rc;
-  L.all.push_back(std::move(b));
-  use_tile_layout(g, L.all.back().get());
-  return AHPP_OK;
-}
-
-int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u) {
-  TileBuilt* const b = g->tile_layouts.cur;
+int tile_ranges(TileBuilt* b, uint32_t warps, const uint4** t, const uint4** u) {
   for (const auto& c : b->cuts)
     if (c.warps == warps) { *t = c.r[0]; *u = c.r[1]; return AHPP_OK; }
-  TileBuilt::Cut cut{warps, {nullptr, nullptr}};
+  GrowInCapture grow;
+  std::vector<uint4> r;                    // of phase 1, then of phase 2
   for (int k = 0; k < 2; ++k) {
     // chunks evenly, then the slices before the pool so that every warp's cost is
     // about the same: {chunk begin, end, slice begin, end}, and the first units
     // of those four
     const TileBuilt::Cost& c = b->cost[k];
-    const uint32_t n = k ? g->dg.tl.u.pool : g->dg.tl.t.pool;
-    std::vector<uint4> r;
+    const uint32_t n = k ? b->t.u.pool : b->t.t.pool;
     uint32_t i = c.n_chunks;
     uint64_t done = 0;
     for (uint32_t w = 0; w < warps; ++w) {
@@ -302,16 +281,54 @@ int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u)
       r.push_back(make_uint4(c0, c1, i0, i));
       r.push_back(make_uint4(c.unit[c0], c.unit[c1], c.unit[i0], c.unit[i]));
     }
-    cut.r[k] = (const uint4*)b->put(r.size() * sizeof(uint4), r.data());
-    if (!cut.r[k]) {
-      set_error("batched ranges: device allocation failed");
-      return AHPP_ENOMEM;
-    }
   }
-  b->cuts.push_back(cut);
-  *t = cut.r[0];
-  *u = cut.r[1];
+  const uint4* d = (const uint4*)b->put(r.size() * sizeof(uint4), r.data());
+  if (!d) {
+    set_error("batched ranges: device allocation failed");
+    return AHPP_ENOMEM;
+  }
+  b->cuts.push_back(TileBuilt::Cut{warps, {d, d + 2 * warps}});
+  *t = d;
+  *u = d + 2 * warps;
   return AHPP_OK;
+}
+
+}  // namespace
+
+void use_tile_layout(ahpp_graph* g, TileBuilt* b) {
+  g->tile_layouts.cur = b;
+  g->dg.tl = b->t;
+}
+
+int use_tile_layout(ahpp_graph* g, uint32_t choice) {
+  Layouts<TileBuilt>& L = g->tile_layouts;
+  L.drop();
+  for (auto& x : L.all)
+    if (x->t.chunk == choice) { use_tile_layout(g, x.get()); return AHPP_OK; }
+  std::unique_ptr<TileBuilt> b(new TileBuilt(g));
+  b->t.chunk = choice;
+  if (int rc = build_tile_layout(g, b.get())) return rc;
+  const uint4 *t, *u;
+  if (int rc = tile_ranges(b.get(), (uint32_t)g->bt_grid * kBWarps, &t, &u)) return rc;
+  L.all.push_back(std::move(b));
+  use_tile_layout(g, L.all.back().get());
+  return AHPP_OK;
+}
+
+int tile_ranges(ahpp_graph* g, uint32_t warps, const uint4** t, const uint4** u) {
+  return tile_ranges(g->tile_layouts.cur, warps, t, u);
+}
+
+int plan_groups(ahpp_graph* g, uint32_t grid, uint32_t* groups, uint32_t* per_group, BatchParams& p) {
+  *per_group = grid / *groups;
+  int rc = tile_ranges(g, *per_group * kBWarps, &p.ranges_t, &p.ranges_u);
+  if (rc == AHPP_ENOMEM && *groups > 1) {
+    *groups = 1;
+    *per_group = grid;
+    rc = tile_ranges(g, grid * kBWarps, &p.ranges_t, &p.ranges_u);
+  }
+  p.groups = *groups;
+  return rc;
 }
 
 uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles, bool serving) {

@@ -64,3 +64,78 @@ def test_a_larger_k_while_a_batch_runs(ahpp, groups):
             c.check(G)
     finally:
         G.close()
+
+
+def test_a_larger_batch_without_memory_for_more_tiles(ahpp):
+    """A batch that would like more tiles at once than there is memory for runs
+    on those there are: buffers for one tile are all that a batch needs."""
+    torch = pytest.importorskip("torch")
+    g = synth.make_graph(**synth.TINY)
+    G = ahpp.Graph.from_arrays(g, attr_bf16=0)
+    try:
+        qs = [int(x) for x in synth.draw_queries(g.n_u, 300, seed=81)]
+        small, large = Batch(torch, ahpp, qs[:20], 10), Batch(torch, ahpp, qs, 10)
+        assert small.start(G, None) == 0
+        torch.cuda.synchronize()
+        for skip in (0, 5, 9):                 # of a tile's buffers, of the next one's
+            G.arm_alloc_failure(skip)
+            assert large.start(G, None) == 0
+            torch.cuda.synchronize()
+            G.arm_alloc_failure(1 << 30)
+            large.check(G)
+    finally:
+        G.close()
+
+
+def test_a_server_without_memory_for_more_tiles(ahpp):
+    """The same for a serving step with more live tiles than before."""
+    g = synth.make_graph(**synth.TINY)
+    G = ahpp.Graph.from_arrays(g, attr_bf16=0)
+    try:
+        qs = [int(x) for x in synth.draw_queries(g.n_u, 120, seed=82)]
+        srv = ahpp.Server(G, max_slots=128, rounds_per_step=4, single_max=-1)
+        try:
+            G.arm_alloc_failure(0)
+            got = [srv.wait(t, 10) for t in [srv.submit(q, EPS, 10) for q in qs]]
+        finally:
+            srv.stop()
+        G.arm_alloc_failure(1 << 30)
+        dense, _, _ = G.query_batch_dense(qs, EPS)
+        for i, r in enumerate(got):
+            assert r.rc == 0
+            check_topk(r.nodes, r.scores, dense[i], 10, EPS)
+    finally:
+        G.close()
+
+
+def test_a_larger_batch_while_its_stream_is_captured(ahpp):
+    """After a small batch, a larger one is only recorded: it takes what memory
+    it needs as it is recorded, and its replays give its results."""
+    torch = pytest.importorskip("torch")
+    g = synth.make_graph(**synth.TINY)
+    G = ahpp.Graph.from_arrays(g, attr_bf16=0)
+    try:
+        qs = [int(x) for x in synth.draw_queries(g.n_u, 300, seed=83)]
+        small, large, after = Batch(torch, ahpp, qs[:20], 10), Batch(torch, ahpp, qs, 10), Batch(torch, ahpp, qs, 900)
+        stream = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            assert small.start(G, stream) == 0
+            stream.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                assert large.start(G, stream) == 0
+        # what grows or is tuned later leaves the recorded launch's memory alone
+        assert after.start(G, stream) == 0
+        stream.synchronize()
+        G.autotune(qs[:8], EPS)
+        for _ in range(2):
+            large.nodes.fill_(-1)
+            large.n.zero_()
+            torch.cuda.synchronize()
+            graph.replay()
+            torch.cuda.synchronize()
+            large.check(G)
+        after.check(G)
+    finally:
+        G.close()

@@ -84,7 +84,12 @@ typedef struct {
     int attr_bf16;             /* store attribute weights as bfloat16 (default 1) */
     int kahan;                 /* Kahan-compensated FP32 reserves (default 1) */
     int switch_rule;           /* switch test: 0 corrected (default), 1 as printed (ASRP only), 2 never */
-    uint64_t hbm_budget_bytes; /* cap on device memory of graph + query state; 0 = no cap */
+    uint64_t hbm_budget_bytes; /* cap on the device memory of the graph's arrays (graph_bytes), a single
+                                  query's state and a server's slots; 0 = no cap.  Not counted, so that
+                                  they decide neither which graphs load nor how many slots there are:
+                                  the layouts built from the arrays for the pull rounds (about as much
+                                  again: ahpp_get_layout_info), and the further tiles that a batch of
+                                  several runs at once on a small graph (at most about 0.5 GB) */
     int device;                /* CUDA device ordinal (default 0) */
     uint32_t max_rounds;       /* round cap per query; 0: automatic */
     uint32_t batch_tile;       /* queries per batched tile: 16 or 32; 0: 32 (ahpp_autotune picks one);
@@ -123,7 +128,7 @@ typedef struct {
     uint64_t n_u, n_v, n_a, n_e, n_ea;   /* after merging duplicates */
     double lambda;                       /* Theorem 3 estimate (or the configured value) */
     uint32_t lambda_T;
-    uint64_t graph_bytes;                /* device bytes held by the graph */
+    uint64_t graph_bytes;                /* device bytes of the graph's arrays */
     uint64_t query_state_bytes;          /* device bytes per single-query state */
     uint64_t tile_state_bytes;           /* device bytes per batched tile */
     int device;
@@ -288,7 +293,7 @@ int ahpp_query_device(ahpp_graph *g, uint32_t q, double eps, uint32_t k,
  * running.  q_sample: host array of n_sample query ids (n_sample == 0
  * changes nothing).  On failure (AHPP_ENOMEM among them) the graph keeps the
  * shapes it had.  Launches captured before stay valid: the layouts that were in
- * use keep their memory (a chosen one adds to graph_bytes).  AHPP_EINVAL for a
+ * use keep their memory (a newly chosen one comes on top).  AHPP_EINVAL for a
  * NULL g or q_sample, an id outside U or a bad eps. */
 int ahpp_autotune(ahpp_graph *g, uint32_t n_sample, const uint32_t *q_sample, double eps);
 

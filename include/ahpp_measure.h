@@ -1,8 +1,8 @@
 /*
  * Measurement helpers of the AHPP library: device rates that roofline
- * reports divide by.  None of them touches a graph or a query; they live in
- * the same shared library as the query API (include/ahpp.h), whose status
- * codes they return.
+ * reports divide by, and what a loaded graph was laid out as.  They live in the
+ * same shared library as the query API (include/ahpp.h), whose status codes they
+ * return.
  */
 #ifndef AHPP_MEASURE_H
 #define AHPP_MEASURE_H
@@ -24,6 +24,13 @@ extern "C" {
  * op not 0/1, table_bytes outside [128, 8 GiB], device < 0 or a NULL output;
  * AHPP_ENOMEM if the table cannot be allocated; AHPP_ECUDA otherwise. */
 int ahpp_row_access_peak(int device, uint64_t table_bytes, int op, double *rows_per_s);
+
+/* What the library built from a graph's arrays (graph_bytes of ahpp_graph_info)
+ * for its pull rounds. */
+typedef struct {
+    uint64_t layout_bytes;               /* device bytes of the layouts, on top of graph_bytes */
+} ahpp_layout_info;
+int ahpp_get_layout_info(const ahpp_graph *g, ahpp_layout_info *info);
 
 #ifdef __cplusplus
 }

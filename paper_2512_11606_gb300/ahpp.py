@@ -73,6 +73,10 @@ class GraphInfo(ctypes.Structure):
                 ("single_vec_width", ctypes.c_uint32), ("single_smem_bytes", ctypes.c_uint32)]
 
 
+class LayoutInfo(ctypes.Structure):
+    _fields_ = [("layout_bytes", ctypes.c_uint64)]
+
+
 class ServerOpts(ctypes.Structure):
     _fields_ = [("max_slots", ctypes.c_uint32), ("queue_capacity", ctypes.c_uint32),
                 ("tile", ctypes.c_uint32), ("rounds_per_step", ctypes.c_uint32),
@@ -96,6 +100,7 @@ SIGNATURES = {
     "ahpp_load_graph_file": (ctypes.c_int, [ctypes.c_char_p, ctypes.POINTER(Config), ctypes.POINTER(_vp)]),
     "ahpp_free_graph": (None, [_vp]),
     "ahpp_get_graph_info": (ctypes.c_int, [_vp, ctypes.POINTER(GraphInfo)]),
+    "ahpp_get_layout_info": (ctypes.c_int, [_vp, ctypes.POINTER(LayoutInfo)]),
     "ahpp_query": (ctypes.c_int, [_vp, ctypes.c_uint32, ctypes.c_double, ctypes.c_uint32,
                                   _u32p, _f32p, _u32p, ctypes.POINTER(Stats)]),
     "ahpp_query_dense": (ctypes.c_int, [_vp, ctypes.c_uint32, ctypes.c_double, _f32p,
@@ -244,6 +249,12 @@ class Graph:
         i = GraphInfo()
         _check(lib().ahpp_get_graph_info(self._h, ctypes.byref(i)))
         return {k.rstrip("_"): getattr(i, k) for k, _ in i._fields_}
+
+    def get_layout_info(self) -> dict:
+        """What the pull rounds' layouts of this graph are (ahpp_measure.h)."""
+        i = LayoutInfo()
+        _check(lib().ahpp_get_layout_info(self._h, ctypes.byref(i)))
+        return {k: getattr(i, k) for k, _ in i._fields_}
 
     @property
     def n_u(self) -> int:

@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "../../include/ahpp_measure.h"
 #include "ahpp_host.h"
 
 namespace ahpp {
@@ -207,7 +208,7 @@ int run_lambda(ahpp_graph* g) {
 
 Layout::~Layout() {
   for (void* p : bufs) cudaFree(p);
-  g->graph_bytes -= bytes;
+  g->layout_bytes -= bytes;
 }
 
 void* Layout::put(size_t n, const void* src) {
@@ -219,7 +220,7 @@ void* Layout::put(size_t n, const void* src) {
   }
   bufs.push_back(p);
   bytes += size;
-  g->graph_bytes += size;
+  g->layout_bytes += size;
   return src && upload(g, p, src, n) != cudaSuccess ? nullptr : p;
 }
 
@@ -545,6 +546,12 @@ int ahpp_get_graph_info(const ahpp_graph* g, ahpp_graph_info* info) {
   return AHPP_OK;
 }
 
+
+int ahpp_get_layout_info(const ahpp_graph* g, ahpp_layout_info* info) {
+  if (!g || !info) { set_error("null argument"); return AHPP_EINVAL; }
+  info->layout_bytes = g->layout_bytes;
+  return AHPP_OK;
+}
 
 int ahpp_query_device(ahpp_graph* g, uint32_t q, double eps, uint32_t k, uint32_t* d_out_nodes,
                       float* d_out_scores, uint32_t* d_out_n, ahpp_stats* d_stats, void* stream) {

@@ -608,11 +608,11 @@ int build_cluster_layout(ahpp_graph* g) {
                           up16(8ull * t.rows_max) + up16(8ull * u.rows_max) + steps * kClStepBytes;
     if (smem > kClSmemMax || !cluster_fits(blocks, (uint32_t)smem)) continue;
 
-    const size_t before = g->graph_bytes;
+    const uint64_t before = g->layout_bytes;
     auto put = [&](const void* p, size_t bytes) -> void* {
       void* d = g->alloc(std::max<size_t>(bytes, 16));
       if (!d || upload(g, d, p, bytes) != cudaSuccess) ok = false;
-      g->graph_bytes += std::max<size_t>(bytes, 16);
+      g->layout_bytes += std::max<size_t>(bytes, 16);
       return d;
     };
     auto rows = [&](const HostPhase& h, uint32_t step0, ClusterRows& R) {
@@ -636,7 +636,7 @@ int build_cluster_layout(ahpp_graph* g) {
     C.n_blocks = blocks;
     C.smem_bytes = (uint32_t)smem;
     if (!ok) {
-      g->graph_bytes = before;
+      g->layout_bytes = before;
       set_error("cluster layout: device allocation failed");
       return AHPP_ENOMEM;
     }

@@ -404,7 +404,7 @@ int alloc_query_state(ahpp_graph* g) {
   if (int rc = batch_plan(g)) return rc;
   if (int rc = use_tile_layout(g, (uint32_t)chunk_choice(cfg.batch_chunk))) return rc;
   settle_layouts(g);
-  if (cfg.hbm_budget_bytes && g->graph_bytes + g->q1_bytes > cfg.hbm_budget_bytes) {
+  if (cfg.hbm_budget_bytes && g->graph_bytes + single_state_bytes(g) > cfg.hbm_budget_bytes) {
     set_error("ahpp_load_graph: graph and query state exceed hbm_budget_bytes");
     return AHPP_ENOMEM;
   }

@@ -137,7 +137,8 @@ struct ahpp_graph {
   ahpp::DevGraph dg{};
   std::vector<ahpp::DevBuf> bufs;   // everything allocated for the graph
   size_t n_graph_bufs = 0;          // bufs[0, n_graph_bufs): the graph's own arrays (what a cache saves)
-  uint64_t graph_bytes = 0;
+  uint64_t graph_bytes = 0;       // the graph's own arrays
+  uint64_t layout_bytes = 0;      // what is built from them for the pull rounds
 
   // internal <-> caller id maps of U
   std::vector<uint32_t> h_u_old2new, h_u_new2old;
@@ -234,6 +235,10 @@ int plan_groups(ahpp_graph* g, uint32_t grid, uint32_t* groups, uint32_t* per_gr
 // Tiles that run at once, of n_tiles to be run (see groups_of).
 uint32_t tile_groups(const ahpp_graph* g, uint32_t n_tiles, bool serving);
 int alloc_query_state(ahpp_graph* g);
+// Bytes of a single query's state as limits count them (ahpp_query_dense_noalloc's
+// array, hbm_budget_bytes): its vectors and the sums of rows of more than 2,048
+// entries, whatever the layout of the pull rounds adds to them.
+size_t single_state_bytes(const ahpp_graph* g);
 int run_lambda(ahpp_graph* g);
 int run_query1(ahpp_graph* g, uint32_t q_new, double eps, uint32_t lambda_T_mode,
                cudaStream_t stream, QCtl* h_ctl);

@@ -75,16 +75,15 @@ size_t carve(const ahpp_graph* g, char* base, Q1State* s) {
   return off;
 }
 
-// Bytes of query state by which graphs are taken or rejected.
-size_t state_bytes(const ahpp_graph* g) {
+}  // namespace
+
+size_t single_state_bytes(const ahpp_graph* g) {
   const size_t nv = std::max<uint64_t>(g->n_v, 1), na = std::max<uint64_t>(g->n_a, 1);
   const size_t ns = std::max<size_t>((size_t)g->dg.s1_v.n_split + g->dg.s1_a.n_split + g->n_long_u, 1);
   return 4 * align256(4 * g->n_u) + align256(4 * nv) + 2 * align256(4 * na) + 2 * align256(4 * ns) +
          align256(sizeof(QCtl)) + align256(3 * sizeof(RAcc)) + align256(sizeof(GridBarrier)) +
          align256(2 * sizeof(unsigned int));
 }
-
-}  // namespace
 
 // Parameters of a single query (shared with the allocating entry points).
 Q1Params noalloc_params(const ahpp_graph* g, uint32_t q_new, double eps);
@@ -102,7 +101,7 @@ extern "C" int ahpp_query_dense_noalloc(ahpp_graph* g, uint32_t q, double eps, f
     return AHPP_EINVAL;
   }
   Q1State s;
-  const size_t need = state_bytes(g);
+  const size_t need = single_state_bytes(g);
   if (need > kNoAllocBytes || carve(g, nullptr, &s) > kNoAllocBytes + kLayoutBytes) {
     set_error("ahpp_query_dense_noalloc: the graph needs " + std::to_string(need) +
               " bytes of query state; the static scratch holds " + std::to_string(kNoAllocBytes) +

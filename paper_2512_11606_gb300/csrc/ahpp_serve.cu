@@ -324,13 +324,16 @@ int ahpp_server_start(ahpp_graph* g, const ahpp_server_opts* opts, ahpp_server**
   const DevGraph& G = g->dg;
   const size_t n_split = std::max(G.tl.split_u_max, 1u);        // any chunk choice fits
   const size_t n_table = (size_t)G.n_v + 2 * (size_t)G.tl.acc_max + 1;
-  const size_t tile_bytes = (size_t)G.n_u * kTile * 12 + n_table * kTile * 4 + n_split * (kTile + 1) * 4 +
+  // a tile as the budget counts it: per-node state, one t_A, top-k
+  const size_t tile_bytes = (size_t)G.n_u * kTile * 12 + ((size_t)std::max(G.n_v, 1u) + std::max(G.n_a, 1u)) * kTile * 4 +
                             (size_t)kRadixPasses * kTile * kRadixBins * 4 + (size_t)kTile * s->kmax * 8 + 4096;
   uint32_t tiles;
   if (o.max_slots) {
     tiles = (o.max_slots + kTile - 1) / kTile;
   } else if (g->cfg.hbm_budget_bytes) {
-    const uint64_t used = g->graph_bytes + g->q1_bytes + g->tile_bytes * g->bt.n_groups;
+    // tiles that a batch runs at once by the library's own rule are not counted
+    const uint64_t used = g->graph_bytes + single_state_bytes(g) +
+                          tile_bytes * std::min(g->bt.n_groups, std::max(1u, g->batch_groups));
     if (g->cfg.hbm_budget_bytes <= used + tile_bytes) {
       delete s;
       set_error("ahpp_server_start: hbm_budget_bytes leaves no room for one tile of slots");

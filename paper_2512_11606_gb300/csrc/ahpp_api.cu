@@ -309,21 +309,27 @@ void set_batch_params(const ahpp_graph* g, BatchParams& p) {
   p.switch_log = (float)-std::log(p.lambda);
 }
 
+// The shape of a launch of n queries: buffers and ranges for the tiles that run at
+// once (made if there are none yet), with no memory for so many those there are.
+int plan_batch(ahpp_graph* g, uint32_t n, uint32_t kmax, uint32_t* groups, uint32_t* per_group, BatchParams& p) {
+  int rc = batch_plan(g);
+  if (rc) return rc;
+  *groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile, false);
+  rc = ensure_batch(g, *groups, kmax);
+  if (rc == AHPP_ENOMEM && *groups > std::max(1u, g->bt.n_groups)) {
+    *groups = std::max(1u, g->bt.n_groups);
+    rc = ensure_batch(g, *groups, kmax);
+  }
+  return rc ? rc : plan_groups(g, (uint32_t)g->bt_grid, groups, per_group, p);
+}
+
 int run_batch_launch(ahpp_graph* g, uint32_t n, const uint32_t* d_q, const double* d_eps,
                      const uint32_t* d_k, uint32_t kmax, uint32_t* d_nodes, float* d_scores,
                      uint32_t* d_n, ahpp_stats* d_stats, float* d_dense, cudaStream_t stream) {
-  int rc = batch_plan(g);
-  if (rc) return rc;
-  // with no memory for so many tiles at once, as many as there are buffers for
-  uint32_t groups = tile_groups(g, (n + g->batch_tile - 1) / g->batch_tile, false), per_group;
-  rc = ensure_batch(g, groups, kmax);
-  if (rc == AHPP_ENOMEM && groups > std::max(1u, g->bt.n_groups)) {
-    groups = std::max(1u, g->bt.n_groups);
-    rc = ensure_batch(g, groups, kmax);
-  }
-  if (rc) return rc;
   BatchParams p;
-  if ((rc = plan_groups(g, (uint32_t)g->bt_grid, &groups, &per_group, p))) return rc;
+  uint32_t groups, per_group;
+  int rc = plan_batch(g, n, kmax, &groups, &per_group, p);
+  if (rc) return rc;
   p.n = n;
   p.q = d_q;
   p.eps = d_eps;
@@ -790,6 +796,10 @@ namespace {
 // of the n queries already in io->q / io->eps, with the graph's current
 // launch shape; no outputs besides the stats.
 int time_batch(ahpp_graph* g, GraphIo* io, uint32_t n, float* ms) {
+  // what a shape's first launch makes on the host is no part of its time
+  BatchParams made;
+  uint32_t groups, per_group;
+  if (int r = plan_batch(g, n, 0, &groups, &per_group, made)) return r;
   cudaEvent_t a, b;
   AHPP_CUDA(cudaEventCreate(&a));
   AHPP_CUDA(cudaEventCreate(&b));

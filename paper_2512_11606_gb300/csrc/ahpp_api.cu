@@ -502,7 +502,7 @@ int ahpp_load_graph(const ahpp_graph_desc* desc, const ahpp_config* cfg, ahpp_gr
       cudaStreamCreateWithFlags(&g->upload_stream, cudaStreamNonBlocking) != cudaSuccess) {
     rc = cuda_fail(cudaGetLastError(), "ahpp_load_graph: device setup");
   }
-  if (rc == AHPP_OK) rc = build_graph(desc, g);
+  if (rc == AHPP_OK) rc = no_throw([&] { return build_graph(desc, g); });
   if (rc == AHPP_OK) {
     if (c.algo == AHPP_ASRP && !(c.lambda > 0.0)) rc = run_lambda(g);
     else g->lambda = c.lambda > 0.0 ? c.lambda : 1.0;
@@ -700,8 +700,9 @@ int ahpp_query_batch_device(ahpp_graph* g, uint32_t n, const uint32_t* d_q, cons
   std::lock_guard<std::mutex> lock(g->mu);
   AHPP_CUDA(cudaSetDevice(g->device));
   cudaStream_t s = stream ? (cudaStream_t)stream : g->stream;
-  return run_batch_launch(g, n, d_q, d_eps, d_k, kmax, d_out_nodes, d_out_scores, d_out_n, d_stats,
-                          nullptr, s);
+  return no_throw([&] {
+    return run_batch_launch(g, n, d_q, d_eps, d_k, kmax, d_out_nodes, d_out_scores, d_out_n, d_stats, nullptr, s);
+  });
 }
 
 static int batch_host(ahpp_graph* g, uint32_t n, const uint32_t* q, const double* eps,
@@ -778,14 +779,14 @@ int ahpp_query_batch(ahpp_graph* g, uint32_t n, const uint32_t* q, const double*
                      const uint32_t* k, uint32_t* out_nodes, float* out_scores, uint32_t* out_n,
                      ahpp_stats* st) {
   ahpp::NvtxRange nvtx_range_("ahpp_query_batch");
-  return batch_host(g, n, q, eps, k, out_nodes, out_scores, out_n, st, nullptr);
+  return no_throw([&] { return batch_host(g, n, q, eps, k, out_nodes, out_scores, out_n, st, nullptr); });
 }
 
 int ahpp_query_batch_dense(ahpp_graph* g, uint32_t n, const uint32_t* q, const double* eps,
                            float* out_pi, ahpp_stats* st) {
   ahpp::NvtxRange nvtx_range_("ahpp_query_batch_dense");
   if (!out_pi) { set_error("null output"); return AHPP_EINVAL; }
-  return batch_host(g, n, q, eps, nullptr, nullptr, nullptr, nullptr, st, out_pi);
+  return no_throw([&] { return batch_host(g, n, q, eps, nullptr, nullptr, nullptr, nullptr, st, out_pi); });
 }
 
 }  // extern "C"
@@ -865,20 +866,20 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
   AHPP_CUDA(cudaMemcpyAsync(io->q.p, qv.data(), 4ull * n, cudaMemcpyHostToDevice, g->stream));
   AHPP_CUDA(cudaMemcpyAsync(io->eps.p, ev.data(), 8ull * n, cudaMemcpyHostToDevice, g->stream));
   float ms = 0.f;
-  if ((rc = time_batch(g, io, n, &ms)) != AHPP_OK) return rc;
+  if ((rc = no_throw([&] { return time_batch(g, io, n, &ms); })) != AHPP_OK) return rc;
   // try each value of one knob with the others fixed; keep the fastest
   auto tune_batch = [&](const char* knob, auto set, const std::vector<uint32_t>& values) -> int {
     float best = -1.f;
     uint32_t best_v = values[0];
     for (uint32_t v : values) {
-      if (int r = set(v)) return r;
+      if (int r = no_throw([&] { return set(v); })) return r;
       float t = 0.f;
-      if (int r = time_batch(g, io, n, &t)) return r;
+      if (int r = no_throw([&] { return time_batch(g, io, n, &t); })) return r;
       note(knob, v, t / (float)n);
       // a later value has to be faster by more than runs differ
       if (best < 0.f || t < 0.98f * best) { best = t; best_v = v; }
     }
-    return set(best_v);
+    return no_throw([&] { return set(best_v); });
   };
   // the shapes in use, which come back if anything fails (their layouts are kept)
   const uint32_t saved_groups = g->batch_groups, saved_tile = g->batch_tile, saved_div = g->q1_dense_div;
@@ -896,13 +897,13 @@ extern "C" int ahpp_autotune(ahpp_graph* g, uint32_t n_sample, const uint32_t* q
     float best = -1.f;
     uint32_t best_v = values[0];
     for (uint32_t v : values) {
-      if (int r = set(v)) return r;
+      if (int r = no_throw([&] { return set(v); })) return r;
       float t = 0.f;
       if (int r = time_single(g, q1, eps, &t)) return r;
       note(knob, v, t / (float)q1.size());
       if (best < 0.f || t < best) { best = t; best_v = v; }
     }
-    return set(best_v);
+    return no_throw([&] { return set(best_v); });
   };
   if (rc == AHPP_OK && !g->cl.n_blocks)
     rc = tune_single("single_vec_width", [&](uint32_t v) { return use_q1_layout(g, v); }, {32u, 8u, 2u, 1u});

@@ -275,7 +275,7 @@ extern "C" int ahpp_load_graph_file(const char* path, const ahpp_config* cfg, ah
       fail(AHPP_ECUDA, "ahpp_load_graph_file: id maps");
     }
   }
-  if (rc == AHPP_OK) rc = alloc_query_state(g);
+  if (rc == AHPP_OK) rc = no_throw([&] { return alloc_query_state(g); });
   if (rc == AHPP_OK) {
     // lambda: the configured value, else the cached estimate when it was
     // taken with the same T, else a new estimate on the device

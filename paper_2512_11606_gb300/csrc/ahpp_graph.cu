@@ -30,14 +30,11 @@ template <typename F>
 void parallel_for(size_t n, F fn) {
   unsigned nt = worker_count();
   if (n < 65536 || nt == 1) { fn(size_t(0), n); return; }
-  std::vector<std::thread> th;
-  size_t step = (n + nt - 1) / nt;
-  for (unsigned t = 0; t < nt; ++t) {
-    size_t b = t * step, e = std::min(n, b + step);
-    if (b >= e) break;
-    th.emplace_back([=] { fn(b, e); });
-  }
-  for (auto& x : th) x.join();
+  const size_t step = (n + nt - 1) / nt;
+  run_threads(nt, [&](unsigned t) {
+    const size_t b = t * step, e = std::min(n, b + step);
+    if (b < e) fn(b, e);
+  });
 }
 
 // Rows of (row, col, w) triples: bucketed by row, sorted by col, duplicates

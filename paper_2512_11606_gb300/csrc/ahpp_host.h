@@ -17,6 +17,7 @@
 #include "ahpp_batch.cuh"
 #include "ahpp_cluster.cuh"
 #include "ahpp_groups.h"
+#include "ahpp_threads.h"
 
 namespace ahpp {
 
@@ -37,6 +38,19 @@ int cuda_fail(cudaError_t e, const char* where);
     cudaError_t e_ = (call);                              \
     if (e_ != cudaSuccess) return ::ahpp::cuda_fail(e_, #call); \
   } while (0)
+
+// f's status; AHPP_ENOMEM for what it throws (nothing throws across the ABI).
+template <typename F>
+int no_throw(const F& f) {
+  try {
+    return f();
+  } catch (const std::exception& e) {
+    set_error(std::string("host memory or threads: ") + e.what());
+  } catch (...) {
+    set_error("host code failed");
+  }
+  return AHPP_ENOMEM;
+}
 
 // Host copy of one adjacency direction before upload.
 struct HostAdj {
@@ -107,6 +121,11 @@ struct TileBuilt : Layout {
   } cost[2];
   struct Cut { uint32_t warps; const uint4* r[2]; };
   std::vector<Cut> cuts;
+};
+// Device memory that is freed with its scope.
+struct ScratchBufs {
+  std::vector<void*> bufs;
+  ~ScratchBufs() { for (void* p : bufs) cudaFree(p); }
 };
 // The layouts of one kind that a graph has; `cur` is the one in use.
 template <typename L>

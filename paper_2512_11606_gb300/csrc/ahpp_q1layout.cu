@@ -234,10 +234,7 @@ template <typename F>
 void over_threads(uint32_t n, F fn) {
   const unsigned hw = std::thread::hardware_concurrency();
   const uint32_t nt = std::max(1u, std::min({hw ? hw : 1u, 32u, n}));
-  std::vector<std::thread> th;
-  for (uint32_t t = 0; t < nt; ++t)
-    th.emplace_back([=] { for (uint32_t i = t; i < n; i += nt) fn(i); });
-  for (auto& x : th) x.join();
+  run_threads(nt, [&](unsigned t) { for (uint32_t i = t; i < n; i += nt) fn(i); });
 }
 
 // A block of U rows of the attribute hop.
@@ -380,13 +377,10 @@ int build_q1_layout(ahpp_graph* g, Q1Built* b) {
   b->smem = kQ1RingBytes + 4 * std::max(Q.s.own_cap + Q.hub_u, (Q.hub_a + 3) / 4 * 4 + Q.hub_v);
 
   HostRows hv, hu;
-  {
-    std::thread t([&] {
-      hv = make_rows(nV, lw, none, lg_min, v_steps, v_steps, Q.hub_v);   // split rows' sums are read from shared memory
-    });
-    hu = make_rows(nU, lv, la, lg_min, kLaneStepsMax, kLaneStepsMax, nU);
-    t.join();
-  }
+  run_threads(2, [&](unsigned t) {
+    if (t) hu = make_rows(nU, lv, la, lg_min, kLaneStepsMax, kLaneStepsMax, nU);
+    else hv = make_rows(nV, lw, none, lg_min, v_steps, v_steps, Q.hub_v);   // split rows' sums are read from shared memory
+  });
   std::vector<Block> blk(n_vb);
   over_threads(n_vb, [&](uint32_t i) {
     blk[i] = make_block(i, vb[i].x, vb[i].x + vb[i].y, au, au_idx, s_units);
@@ -414,12 +408,12 @@ int build_q1_layout(ahpp_graph* g, Q1Built* b) {
     return p;
   };
   auto put = [&](auto& v) -> void* { return dev(v.size() * sizeof(v[0]), v.data()); };
-  std::vector<void*> tmp;
+  ScratchBufs tmp;
   auto scratch = [&](auto& v) -> void* {
     void* p = nullptr;
     const size_t n = v.size() * sizeof(v[0]);
     if (g->dev_malloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
-    tmp.push_back(p);
+    tmp.bufs.push_back(p);
     if (upload(g, p, v.data(), n) != cudaSuccess) ok = false;
     return p;
   };
@@ -488,7 +482,6 @@ int build_q1_layout(ahpp_graph* g, Q1Built* b) {
   Q.deg_a = da;
   const cudaError_t e = cudaStreamSynchronize(g->stream);
   const cudaError_t le = cudaGetLastError();
-  for (void* p : tmp) cudaFree(p);
   if (e != cudaSuccess || le != cudaSuccess) return cuda_fail(e != cudaSuccess ? e : le, "single-query layout");
   if (!ok) { set_error("single-query layout: device allocation failed"); return AHPP_ENOMEM; }
   return AHPP_OK;

@@ -290,7 +290,7 @@ void server_loop(ahpp_server* s) {
       s->cv_work.wait(lock, [&] { return s->stop || !s->queue.empty() || s->in_flight > 0; });
       if (s->stop) break;
     }
-    const int rc = server_step(s);
+    const int rc = no_throw([&] { return server_step(s); });
     if (rc != AHPP_OK) {
       std::lock_guard<std::mutex> lock(s->mu);
       s->fatal = rc;

@@ -201,12 +201,12 @@ int build_tile_layout(ahpp_graph* g, TileBuilt* b) {
     return p;
   };
   auto put = [&](auto& v) -> void* { return dev(v.size() * sizeof(v[0]), v.data()); };
-  std::vector<void*> tmp;
+  ScratchBufs tmp;
   auto scratch = [&](auto& v) -> void* {
     void* p = nullptr;
     const size_t n = v.size() * sizeof(v[0]);
     if (g->dev_malloc(&p, std::max<size_t>(n, 16)) != cudaSuccess) { cudaGetLastError(); ok = false; return nullptr; }
-    tmp.push_back(p);
+    tmp.bufs.push_back(p);
     if (upload(g, p, v.data(), n) != cudaSuccess) ok = false;
     return p;
   };
@@ -249,7 +249,6 @@ int build_tile_layout(ahpp_graph* g, TileBuilt* b) {
   T.acc_deg = (const uint32_t*)put(acc_deg);
   T.chunks_of = (const uint32_t*)put(chunks_of);
   const cudaError_t e = cudaStreamSynchronize(g->stream), le = cudaGetLastError();
-  for (void* p : tmp) cudaFree(p);
   if (e != cudaSuccess || le != cudaSuccess) return cuda_fail(e != cudaSuccess ? e : le, "batched layout");
   if (!ok) { set_error("batched layout: device allocation failed"); return AHPP_ENOMEM; }
   return AHPP_OK;

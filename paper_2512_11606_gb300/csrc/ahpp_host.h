@@ -52,13 +52,6 @@ int no_throw(const F& f) {
   return AHPP_ENOMEM;
 }
 
-// Host copy of one adjacency direction before upload.
-struct HostAdj {
-  std::vector<uint32_t> off, idx;
-  std::vector<float> w;        // raw weights
-  std::vector<float> c;        // direction coefficient (structure only)
-};
-
 struct HostItems {
   std::vector<uint4> items;
   std::vector<uint32_t> split_nchunks;
@@ -259,8 +252,6 @@ int alloc_query_state(ahpp_graph* g);
 // entries, whatever the layout of the pull rounds adds to them.
 size_t single_state_bytes(const ahpp_graph* g);
 int run_lambda(ahpp_graph* g);
-int run_query1(ahpp_graph* g, uint32_t q_new, double eps, uint32_t lambda_T_mode,
-               cudaStream_t stream, QCtl* h_ctl);
 int topk_single(ahpp_graph* g, const float* d_score, uint32_t k, uint32_t* d_nodes,
                 float* d_scores, uint32_t* d_n, cudaStream_t stream);
 // The batched kernel's grid (computed once per graph).

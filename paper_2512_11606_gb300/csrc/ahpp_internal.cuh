@@ -28,18 +28,17 @@
 
 namespace ahpp {
 
-constexpr int kThreads = 256;          // threads per block of every persistent kernel
-constexpr int kWarps = kThreads / 32;
+constexpr int kThreads = 256;          // threads per block of the top-k kernel
 constexpr uint32_t kItemLong = 0x40000000u;   // item = one whole long row (warp-cooperative)
 constexpr uint32_t kItemSplit = 0x80000000u;  // item = one chunk of a split row (| slot)
-constexpr uint32_t kItemMask = 0x3fffffffu;
 // Entries per chunk of a long row in the batched pull phases: the choices of
 // the configuration and of ahpp_autotune.
 constexpr int kChunkChoices = 3;
 constexpr uint32_t kChunkSizes[kChunkChoices] = {128, 256, 512};
 constexpr int kChunkDefault = 1;
 
-// Work items of a pull sweep over one row space.
+// Work items of a push round's flush over one row space (split_nchunks, the chunks
+// of each split row, is read by nothing but belongs to the graph cache's files).
 //   x = first row; y = number of rows (short group, one row per lane) or a flag;
 //   z, w = local neighbour range [z, w) for long / split rows.
 struct ItemList {
@@ -110,8 +109,8 @@ struct Q1Layout {
 // rows (rows are sorted by degree), or four chunks of long rows:
 //   {first row, or first chunk; rows | chunk << 31; entries of the longest;
 //    first unit}
-// The chunk items come first, the n_static items from there on that the warps
-// share out beforehand, then those that warps take `batch` at a time when they
+// The chunk items come first, then, up to `pool`, those that the warps share out
+// beforehand (tile_ranges), then those that warps take `batch` at a time when they
 // are done; a last item holds the number of units.
 // Its entries lie in units of 512 bytes: 16 entries of each row, two to a
 // lane's 16 bytes as {index, coefficient, index, coefficient}; pair j of row r
@@ -330,11 +329,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 

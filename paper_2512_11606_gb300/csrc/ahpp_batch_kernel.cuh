@@ -108,6 +108,8 @@ struct TileRing {
   uint32_t base;               // the warp's ring
   uint32_t next, end;          // next unit to copy, end of the stream
 
+  // no block ends while copies to its shared memory are in flight
+  __device__ __forceinline__ ~TileRing() { asm volatile("cp.async.wait_all;" ::: "memory"); }
   __device__ __forceinline__ void refill() {
     if (next < end)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + (next % kTRing) * 512u +

@@ -121,6 +121,8 @@ struct Ring {
   uint32_t base;               // the lane's place in the ring
   uint32_t next, end;          // next unit to copy, end of the stream
 
+  // no block ends while copies to its shared memory are in flight
+  __device__ __forceinline__ ~Ring() { asm volatile("cp.async.wait_all;" ::: "memory"); }
   // the next N units (each its own group of copies, empty past the end)
   template <int N>
   __device__ __forceinline__ void refill() {

@@ -29,6 +29,9 @@ int ahpp_row_access_peak(int device, uint64_t table_bytes, int op, double *rows_
  * for its pull rounds. */
 typedef struct {
     uint64_t layout_bytes;               /* device bytes of the layouts, on top of graph_bytes */
+    uint32_t cluster_blocks;             /* blocks of the one cluster that runs a single query (small
+                                            graphs), 0: the whole-GPU kernel does */
+    uint32_t cluster_smem_bytes;         /* shared memory of each of them */
 } ahpp_layout_info;
 int ahpp_get_layout_info(const ahpp_graph *g, ahpp_layout_info *info);
 

@@ -74,7 +74,8 @@ class GraphInfo(ctypes.Structure):
 
 
 class LayoutInfo(ctypes.Structure):
-    _fields_ = [("layout_bytes", ctypes.c_uint64)]
+    _fields_ = [("layout_bytes", ctypes.c_uint64), ("cluster_blocks", ctypes.c_uint32),
+                ("cluster_smem_bytes", ctypes.c_uint32)]
 
 
 class ServerOpts(ctypes.Structure):

@@ -556,6 +556,8 @@ int ahpp_get_graph_info(const ahpp_graph* g, ahpp_graph_info* info) {
 int ahpp_get_layout_info(const ahpp_graph* g, ahpp_layout_info* info) {
   if (!g || !info) { set_error("null argument"); return AHPP_EINVAL; }
   info->layout_bytes = g->layout_bytes;
+  info->cluster_blocks = g->cl.n_blocks;
+  info->cluster_smem_bytes = g->cl.smem_bytes;
   return AHPP_OK;
 }
 

@@ -151,7 +151,7 @@ k_cluster(const __grid_constant__ DevGraph g, const __grid_constant__ ClusterLay
   extern __shared__ __align__(16) unsigned char cl_smem[];
   __shared__ Q1Loop L;
   __shared__ uint32_t s_part[kSums][kClWarps];
-  __shared__ uint32_t s_sums[2][kClMost][kSums];   // every block's sums, in turn: a block may share again
+  __shared__ uint32_t s_sums[2][kClBlocks][kSums];   // every block's sums, in turn: a block may share again
                                                    // before another has read the last ones
   __shared__ int s_fine;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -558,7 +558,7 @@ int build_cluster_layout(ahpp_graph* g) {
   const uint32_t nU = G.n_u, nV = G.n_v, nA = G.n_a;
   // without padding: the vectors, and each block's share of both phases' entries
   const uint64_t entries = 2 * ((uint64_t)G.n_e + G.n_ea);
-  if (4 * ((uint64_t)nU + nV + nA) + entries / kClMost * 6 > kClSmemMax) return AHPP_OK;
+  if (4 * ((uint64_t)nU + nV + nA) + entries / kClBlocks * 6 > kClSmemMax) return AHPP_OK;
 
   auto down = [&](auto& v, const void* p, size_t n) {
     v.resize(n);
@@ -596,53 +596,51 @@ int build_cluster_layout(ahpp_graph* g) {
     if (k < d) return HostEntry{uvi[uv[u] + k], uvw[uv[u] + k]};
     return HostEntry{nV + uai[ua[u] + k - d], uaw[ua[u] + k - d]};
   };
-  for (uint32_t blocks : {kClMost, 8u}) {
-    const HostPhase t = cut_phase(nV + nA, nV, blocks, len_t, entry_t);
-    const HostPhase u = cut_phase(nU, nU, blocks, len_u, entry_u);
-    if (std::max(t.places_max, u.places_max) > 0xffff) return AHPP_OK;
-    auto up16 = [](uint64_t x) { return (x + 15) / 16 * 16; };
-    uint64_t steps = 0;                    // of any block
-    for (uint32_t b = 0; b < blocks; ++b) steps = std::max<uint64_t>(steps, (uint64_t)t.cta_steps[b].y + u.cta_steps[b].y);
-    const uint64_t smem = up16(4ull * nU) + up16(4ull * (nV + nA)) + up16(4ull * std::max(t.places_max, u.places_max)) +
-                          3 * up16(4ull * u.rows_max) + up16(8ull * t.items_max) + up16(8ull * u.items_max) +
-                          up16(8ull * t.rows_max) + up16(8ull * u.rows_max) + steps * kClStepBytes;
-    if (smem > kClSmemMax || !cluster_fits(blocks, (uint32_t)smem)) continue;
+  const uint32_t blocks = kClBlocks;
+  const HostPhase t = cut_phase(nV + nA, nV, blocks, len_t, entry_t);
+  const HostPhase u = cut_phase(nU, nU, blocks, len_u, entry_u);
+  if (std::max(t.places_max, u.places_max) > 0xffff) return AHPP_OK;
+  auto up16 = [](uint64_t x) { return (x + 15) / 16 * 16; };
+  uint64_t steps = 0;                    // of any block
+  for (uint32_t b = 0; b < blocks; ++b) steps = std::max<uint64_t>(steps, (uint64_t)t.cta_steps[b].y + u.cta_steps[b].y);
+  const uint64_t smem = up16(4ull * nU) + up16(4ull * (nV + nA)) + up16(4ull * std::max(t.places_max, u.places_max)) +
+                        3 * up16(4ull * u.rows_max) + up16(8ull * t.items_max) + up16(8ull * u.items_max) +
+                        up16(8ull * t.rows_max) + up16(8ull * u.rows_max) + steps * kClStepBytes;
+  if (smem > kClSmemMax || !cluster_fits(blocks, (uint32_t)smem)) return AHPP_OK;
 
-    const uint64_t before = g->layout_bytes;
-    auto put = [&](const void* p, size_t bytes) -> void* {
-      void* d = g->alloc(std::max<size_t>(bytes, 16));
-      if (!d || upload(g, d, p, bytes) != cudaSuccess) ok = false;
-      g->layout_bytes += std::max<size_t>(bytes, 16);
-      return d;
-    };
-    auto rows = [&](const HostPhase& h, uint32_t step0, ClusterRows& R) {
-      std::vector<uint2> first = h.cta_steps;
-      for (auto& x : first) x.x += step0;
-      R.cta = (const uint4*)put(h.cta.data(), h.cta.size() * sizeof(uint4));
-      R.steps = (const uint2*)put(first.data(), first.size() * sizeof(uint2));
-      R.items = (const uint2*)put(h.items.data(), h.items.size() * sizeof(uint2));
-      R.meta = (const uint2*)put(h.meta.data(), h.meta.size() * sizeof(uint2));
-      R.ranges = (const uint4*)put(h.ranges.data(), h.ranges.size() * sizeof(uint4));
-      R.rows_max = h.rows_max;
-      R.items_max = h.items_max;
-      R.places_max = h.places_max;
-    };
-    ClusterLayout C;
-    rows(t, 0, C.t);
-    rows(u, (uint32_t)(t.steps.size() / kClStepBytes), C.u);
-    std::vector<unsigned char> all(t.steps);
-    all.insert(all.end(), u.steps.begin(), u.steps.end());
-    C.steps = (const uint4*)put(all.data(), all.size());
-    C.n_blocks = blocks;
-    C.smem_bytes = (uint32_t)smem;
-    if (!ok) {
-      g->layout_bytes = before;
-      set_error("cluster layout: device allocation failed");
-      return AHPP_ENOMEM;
-    }
-    g->cl = C;
-    return AHPP_OK;
+  const uint64_t before = g->layout_bytes;
+  auto put = [&](const void* p, size_t bytes) -> void* {
+    void* d = g->alloc(std::max<size_t>(bytes, 16));
+    if (!d || upload(g, d, p, bytes) != cudaSuccess) ok = false;
+    g->layout_bytes += std::max<size_t>(bytes, 16);
+    return d;
+  };
+  auto rows = [&](const HostPhase& h, uint32_t step0, ClusterRows& R) {
+    std::vector<uint2> first = h.cta_steps;
+    for (auto& x : first) x.x += step0;
+    R.cta = (const uint4*)put(h.cta.data(), h.cta.size() * sizeof(uint4));
+    R.steps = (const uint2*)put(first.data(), first.size() * sizeof(uint2));
+    R.items = (const uint2*)put(h.items.data(), h.items.size() * sizeof(uint2));
+    R.meta = (const uint2*)put(h.meta.data(), h.meta.size() * sizeof(uint2));
+    R.ranges = (const uint4*)put(h.ranges.data(), h.ranges.size() * sizeof(uint4));
+    R.rows_max = h.rows_max;
+    R.items_max = h.items_max;
+    R.places_max = h.places_max;
+  };
+  ClusterLayout C;
+  rows(t, 0, C.t);
+  rows(u, (uint32_t)(t.steps.size() / kClStepBytes), C.u);
+  std::vector<unsigned char> all(t.steps);
+  all.insert(all.end(), u.steps.begin(), u.steps.end());
+  C.steps = (const uint4*)put(all.data(), all.size());
+  C.n_blocks = blocks;
+  C.smem_bytes = (uint32_t)smem;
+  if (!ok) {
+    g->layout_bytes = before;
+    set_error("cluster layout: device allocation failed");
+    return AHPP_ENOMEM;
   }
+  g->cl = C;
   return AHPP_OK;
 }
 

@@ -7,7 +7,7 @@ namespace ahpp {
 
 constexpr int kClThreads = 1024;
 constexpr int kClWarps = kClThreads / 32;
-constexpr uint32_t kClMost = 16;          // blocks of a cluster, at most
+constexpr uint32_t kClBlocks = 16;        // blocks of a cluster
 // Warps that walk; the last one of a block runs the round's control meanwhile.
 constexpr int kClWalkers = kClWarps - 1;
 // A step: four entries for each lane of a warp, 16-bit indices and FP32

@@ -327,7 +327,8 @@ def measured_peak():
 # ------------------------------------------------------------ byte model
 
 def round_bytes(info, lanes, bf16=True):
-    """Algorithmic DRAM bytes of one pull round of a tile with `lanes` queries.
+    """Least DRAM bytes of a pull round of a tile with `lanes` queries whose
+    attribute hop is pushed from phase 2 (tile_round_bytes: as k_tiles does it).
 
     Graph (once per round, shared by the lanes): phase 1 streams V->U (index
     + coefficient, 8 B/edge); phase 2 streams U->V (index + weight, 8 B/edge)
@@ -345,24 +346,37 @@ def round_bytes(info, lanes, bf16=True):
     return graph + state
 
 
+def tile_round_bytes(info, lanes):
+    """Algorithmic DRAM bytes of one round of k_tiles with `lanes` queries.
+
+    Graph (once per round, shared by the lanes): both phases pull both hops,
+    an index and an FP32 coefficient per entry, so 16 B per edge and per
+    attribute entry; the degrees of V and U rows.  State (per lane): phase 1
+    reads r_U and writes the table of t_V and t_A, phase 2 reads the table and
+    clears the next t_A, reads and writes r_U, and read-modify-writes the
+    reserve and its Kahan compensation.
+    """
+    nU, nV, nA, nE, nEA = (info[k] for k in ("n_u", "n_v", "n_a", "n_e", "n_ea"))
+    graph = 16 * (nE + nEA) + 4 * (nU + nV)
+    state = lanes * 4 * (nU + 2 * (nV + nA) + nA + 2 * nU + 4 * nU)
+    return graph + state
+
+
 def q1_round_bytes(info, bf16=True):
     """Algorithmic DRAM bytes of one pull round of the single-query kernel.
 
-    Graph (once per round): phase 1 streams V->U (index + coefficient,
-    8 B/edge); phase 2 streams U->V (index + weight, 8 B/edge) and U->A
-    (index + weight, 4 + 2 B/entry in bfloat16); the row offsets; the
-    attribute normalisers.  With the attribute push (single_attr_push) the
-    attribute hop reuses phase 2's U->A stream; without it phase 1 also
-    streams A->U (index + FP32 pull coefficient, 8 B/entry).  State: the
-    residues gathered in phase 1 (each read once), t_V written and read,
-    t_A read, written (or pushed) and cleared, the residues read and written,
-    the reserve and its Kahan compensation read and written.
+    Graph (once per round): the entries of V->U and U->V (index + FP32
+    coefficient or weight, 8 B/edge each), and of the attribute hop by blocks
+    of U rows and of U->A: 4 B/entry each with bfloat16 weights (16-bit index
+    and weight; U->A with more than 65,536 attributes: 8), 8 with FP32 ones; the
+    degrees of V and U rows and the rows' attribute normalisers.  State: the
+    residues gathered in phase 1 (each read once), t_V written and read, t_A
+    added to, read and cleared, the residues read and written, the reserve and
+    its Kahan compensation read and written.
     """
-    wa = 2 if bf16 else 4
     nU, nV, nA, nE, nEA = (info[k] for k in ("n_u", "n_v", "n_a", "n_e", "n_ea"))
-    graph = 2 * 8 * nE + (4 + wa) * nEA + 4 * (2 * (nU + 1) + (nV + 1)) + 4 * (nU + nA)
-    if not info.get("single_attr_push", 0):
-        graph += 8 * nEA + 4 * (nA + 1)
+    hop, pull = (4 if bf16 else 8), (4 if bf16 and nA <= 65536 else 8)
+    graph = 2 * 8 * nE + (hop + pull) * nEA + 4 * (nU + nV) + 4 * nU
     state = 4 * (nU + 2 * nV + 3 * nA + 2 * nU + 4 * nU)
     return graph + state
 
@@ -450,23 +464,35 @@ def ncu_traffic(kernel, graph, units, key="bytes_per_unit"):
     return rec[key] * units
 
 
-def row_roofline(ahpp, info, tile_rounds, launch_s, device):
+def pulled_rows(info):
+    """Row accesses of a tile-round of k_tiles: phase 1 gathers |E| + |E_A|
+    residue rows from the tile's |U| x 128-byte table, phase 2 |E| t_V rows and
+    |E_A| t_A rows."""
+    nU, nV, nA, nE, nEA = (int(info[k]) for k in ("n_u", "n_v", "n_a", "n_e", "n_ea"))
+    row = 4 * int(info["batch_tile"])
+    return [("gather", nU * row, nE, "phase 1: residue rows over V->U"),
+            ("gather", nU * row, nEA, "phase 1: residue rows over A->U"),
+            ("gather", nV * row, nE, "phase 2: t_V rows"),
+            ("gather", nA * row, nEA, "phase 2: t_A rows")]
+
+
+def row_roofline(ahpp, info, tile_rounds, launch_s, device, parts=None):
     """The batched launch against the L2 row-access ceiling of this GPU.
 
-    Per tile-round the kernel gathers |E| residue rows (phase 1, from the
-    tile's |U| x 128-byte residue table), |E| t_V rows and |E_A| t_A rows
-    (phase 2), and reduces |E_A| rows into the next round's t_A (the attribute
-    push).  The ceiling is the time those row accesses take at the rates
+    parts: the row accesses of a tile-round (op, table bytes, rows, what), by
+    default those of a round whose attribute hop is pushed: |E| residue rows, |E|
+    t_V rows and |E_A| t_A rows gathered, |E_A| rows reduced into the next t_A.
+    The ceiling is the time those row accesses take at the rates
     ahpp_row_access_peak measures for tables of the same sizes; frac is that
     time over the measured launch time (the streamed graph and state bytes
     are left out of the ceiling, so frac is an upper estimate of the gap).
     """
     nU, nV, nA, nE, nEA = (int(info[k]) for k in ("n_u", "n_v", "n_a", "n_e", "n_ea"))
     row = 4 * int(info["batch_tile"])
-    parts = [("gather", nU * row, nE, "phase 1: residue rows"),
-             ("gather", nV * row, nE, "phase 2: t_V rows"),
-             ("gather", nA * row, nEA, "phase 2: t_A rows"),
-             ("reduce", nA * row, nEA, "phase 2: attribute push into t_A")]
+    parts = parts or [("gather", nU * row, nE, "phase 1: residue rows"),
+                      ("gather", nV * row, nE, "phase 2: t_V rows"),
+                      ("gather", nA * row, nEA, "phase 2: t_A rows"),
+                      ("reduce", nA * row, nEA, "phase 2: attribute push into t_A")]
     rates, t_min = [], 0.0
     for op, table, n, what in parts:
         r = ahpp.row_access_peak(table, op, device)
@@ -667,7 +693,7 @@ def run_ours(args, rank, world, local_rank):
 
     # roofline of the dominant kernel (the batched persistent launch)
     peak, peak_kind = measured_peak()
-    alg = tile_rounds * round_bytes(info, tile) + topk_bytes(info, B)   # one launch (last step)
+    alg = tile_rounds * tile_round_bytes(info, tile) + topk_bytes(info, B)   # one launch (last step)
     achieved = alg / (sum(launch_ms) / K / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": ncu_traffic("k_tiles", args.graph, tile_rounds),
@@ -680,7 +706,8 @@ def run_ours(args, rank, world, local_rank):
             "tile_rounds_per_launch": tile_rounds}
 
     try:
-        roof["l2_rows"] = row_roofline(ahpp, info, tile_rounds, sum(launch_ms) / K / 1e3, local_rank)
+        roof["l2_rows"] = row_roofline(ahpp, info, tile_rounds, sum(launch_ms) / K / 1e3, local_rank,
+                                       pulled_rows(info))
     except Exception as e:  # the HBM roofline above stands on its own
         roof["l2_rows"] = {"error": str(e)}
     # L2 -> SM bytes (ncu capture, scaled) against the measured rate of random
@@ -688,7 +715,7 @@ def run_ours(args, rank, world, local_rank):
     l2_bytes = ncu_traffic("k_tiles", args.graph, tile_rounds, "l2_to_sm_bytes_per_unit")
     parts = roof["l2_rows"].get("parts") if isinstance(roof.get("l2_rows"), dict) else None
     if l2_bytes and parts:
-        peak_l2 = parts[1]["peak_rows_per_s"] * 4 * int(info["batch_tile"]) / 1e9
+        peak_l2 = parts[2]["peak_rows_per_s"] * 4 * int(info["batch_tile"]) / 1e9
         ach_l2 = l2_bytes / (sum(launch_ms) / K / 1e3) / 1e9
         roof["l2_sm"] = {"bound": "l2 -> sm bandwidth", "unit": "GB/s", "achieved": ach_l2, "peak": peak_l2,
                          "frac": ach_l2 / peak_l2,

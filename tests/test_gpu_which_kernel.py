@@ -21,22 +21,44 @@ def ahpp():
     return mod
 
 
-@pytest.mark.parametrize("i", range(len(KINDS)))
+# graphs whose vectors are 77 and 98 KB of what a block holds
+LARGE = [dict(n_u=14_003, n_v=5_501, n_a=129, deg=3, m=2, seed=9),
+         dict(n_u=18_001, n_v=7_001, n_a=31, deg=1, m=1, seed=10)]
+GRID_ONLY = (5, 7)                     # of KINDS: the vectors and entries are more than 223 KB a block
+
+
+@pytest.mark.parametrize("i", range(len(KINDS) + len(LARGE)))
 def test_small_graphs_run_on_a_cluster(ahpp, i):
-    g = graph(**KINDS[i])
-    fits = i + 1 < len(KINDS)
+    g = graph(**(KINDS + LARGE)[i])
     G = ahpp.Graph.from_arrays(g, lam=1.5, attr_bf16=0)
     info = G.get_layout_info()
     G.close()
-    assert info["cluster_blocks"] == (16 if fits else 0)
+    assert info["cluster_blocks"] == (0 if i in GRID_ONLY else 16)
     # all residues and t values, and this block's 16th of both directions' entries (6 bytes each)
     least = 4 * (g.n_u + g.n_v + g.n_a)
-    assert not fits or least < info["cluster_smem_bytes"] <= 223 * 1024
-    if i in (5, 6):
-        assert info["cluster_smem_bytes"] > 100 * 1024
+    if i not in GRID_ONLY:
+        assert least < info["cluster_smem_bytes"] <= 223 * 1024
     G = ahpp.Graph.from_arrays(g, lam=1.5, attr_bf16=0, single_vec_width=2)
     assert G.get_layout_info()["cluster_blocks"] == 0
     G.close()
+
+
+@pytest.mark.parametrize("kind", LARGE)
+@pytest.mark.parametrize("algo", ["ASRP", "APP"])
+def test_large_vectors_on_a_cluster_match_oracle(ahpp, kind, algo):
+    g = graph(**kind)
+    og = oracle.OracleGraph.from_arrays(g)
+    lam, _ = og.lambda_estimate(ALPHA, BETA)
+    G = ahpp.Graph.from_arrays(g, lam=lam, attr_bf16=0, algo=getattr(ahpp, "AHPP_" + algo))
+    try:
+        assert G.get_layout_info()["cluster_blocks"] == 16
+        for q in (0, g.n_u // 2, g.n_u - 1):
+            pi, st, rc = G.query_dense(q, EPS)
+            ref = og.push(algo.lower(), ALPHA, BETA, q, EPS, lam=lam)
+            assert rc == 0 and abs(st["rounds"] - ref.stats["rounds"]) <= 1
+            assert np.abs(pi.astype(np.float64) - ref.pi).max() <= TOL
+    finally:
+        G.close()
 
 
 @pytest.mark.parametrize("width", [0, 1])

@@ -251,7 +251,10 @@ int ensure_batch(ahpp_graph* g, uint32_t groups, uint32_t kmax) {
   BatchState s = g->bt;
   const DevGraph& G = g->dg;
   const size_t n_split = std::max(G.tl.split_u_max, 1u);        // any chunk choice fits
-  const uint32_t kcap = std::max(kmax, s.kmax_cap);
+  // in powers of two: buffers that launches were given stay, so what a k that
+  // grows from call to call leaves behind is no more than the last ones take
+  uint32_t kcap = std::max(s.kmax_cap, 1u);
+  while (kcap < kmax) kcap *= 2;
   const uint32_t ng = std::max(groups, s.n_groups);
   const size_t before = g->bufs.size();
   uint64_t bytes = 0;

@@ -75,6 +75,7 @@ def test_a_larger_batch_without_memory_for_more_tiles(ahpp):
     try:
         qs = [int(x) for x in synth.draw_queries(g.n_u, 300, seed=81)]
         small, large = Batch(torch, ahpp, qs[:20], 10), Batch(torch, ahpp, qs, 10)
+        torch.cuda.synchronize()
         assert small.start(G, None) == 0
         torch.cuda.synchronize()
         for skip in (0, 5, 9):                 # of a tile's buffers, of the next one's
@@ -149,11 +150,13 @@ def test_memory_of_a_k_that_grows_by_one(ahpp):
     G = ahpp.Graph.from_arrays(g, attr_bf16=0)
     try:
         calls = [Batch(torch, ahpp, [int(x) for x in synth.draw_queries(g.n_u, 320, seed=84)], k) for k in range(1, 257)]
+        for c in calls:
+            c.eps.fill_(1e-2)
+        torch.cuda.synchronize()
         calls[0].start(G, None)
         torch.cuda.synchronize()
         free = torch.cuda.mem_get_info()[0]
         for c in calls:
-            c.eps.fill_(1e-2)
             assert c.start(G, None) == 0
         torch.cuda.synchronize()
         assert free - torch.cuda.mem_get_info()[0] <= 16 << 20

@@ -301,7 +301,12 @@ void shape_of(const ahpp_graph* g, uint32_t vec_width, uint32_t* grid, uint32_t*
   // lanes per short row: one (16,000 nodes: 1.77 ms a query with eight lanes, 1.69
   // with one; 44,000: 2.62, 1.70; 100,000: 2.94, 2.64), unless that leaves the
   // warps a long slice of U rows or two each (200,000 nodes of 40 entries: 5.35 with
-  // one, 4.89 with two; 277,000 of 36: 10.0, 9.28; but 176,000 of 22: 3.86, 4.85)
+  // one, 4.89 with two; 277,000 of 36: 10.0, 9.28).  Past either line one lane is
+  // faster or as fast (ms with one and two lanes; nodes, entries a node: 140,000 of
+  // 34: 3.12, 3.36; 311,000 of 34: 6.59, 6.98; 374,000 of 40: 9.01, 9.10; 176,000 of
+  // 22: 3.86, 4.85; 171,000 of 28: 3.26, 3.85; 288,000 of 28: 5.44, 6.12), between
+  // them it is one or the other within 3 %, graph by graph (171,000 of 34: 4.17,
+  // 4.05; 233,000 of 34: 5.57, 5.68; 288,000 of 34: 6.29, 6.20)
   const uint64_t slices = G.n_u / 32, warps = (uint64_t)nb * kQ1Warps;
   const bool uneven = slices > warps && 10 * slices < 19 * warps;
   *grid = nb;

@@ -65,7 +65,8 @@ void add_chunks(HostTiles& h, uint32_t warps) {
 
 // Relative cost of a slice, fitted to the blocks' measured times on the medium
 // graph: tenths of a gathered row (of t_A, a small table: seven), and the
-// item's own latencies in kItemT or kItemU.
+// item's own latencies in kItemT or kItemU.  They only even out the warps' shares
+// (on other graphs the pool does the rest).
 constexpr uint32_t kRow = 10, kAttr = 7, kItemT = 75, kItemU = 170;
 // Share of the slices' cost that is left in the pool, in percent.
 constexpr uint32_t kPoolShare = 20;

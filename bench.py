@@ -100,9 +100,9 @@ def workload_config(args, extra=None):
         "batch_queries_per_gpu": args.batch,
         "eps": args.eps,
         "k": args.k,
-        "l2": ("inputs larger than L2 (graph ~0.7 GB + per-tile state ~0.45 GB per round)"
+        "l2": ("inputs larger than L2 (graph layout ~0.7 GB + per-tile state ~0.45 GB per round)"
                if args.graph == "medium" else
-               "inputs larger than L2 (graph ~5 GB + per-tile state ~2.3 GB per round)"
+               "inputs larger than L2 (graph layout ~6 GB + per-tile state ~2.3 GB per round)"
                if args.graph == "large" else "tiny graph: L2-resident, reported, not graded"),
         "parallelism": f"replicas{args.gpus}" if args.gpus > 1 else "1 GPU",
     }
@@ -399,23 +399,22 @@ def topk_bytes(info, queries):
 # any of them changes (comments and layout aside) the figure no longer
 # applies and ncu_traffic returns None.
 NCU_TRAFFIC = {
-    # ncu --set full of one 32-query tile on the medium graph (106 tile-rounds):
-    # profiles/k_tiles_medium_tile32.md
+    # a launch of 64 queries, two tiles of 106 rounds: profiles/k_tiles_medium_tile32.md
     "k_tiles": {
         "graph": "medium",
-        "bytes_per_unit": 2.424642e9,        # dram__bytes_read.sum + dram__bytes_write.sum per tile-round
-        "l2_to_sm_bytes_per_unit": 8.972795e9,   # l1tex__m_xbar2l1tex_read_bytes.sum per tile-round
-        "sources": {"ahpp_batch_kernel.cuh": "f341ce418086809a", "ahpp_batch.cu": "f92167d838a2d532",
-                    "ahpp_batch.cuh": "2f7f8c2bb4bfbcdd", "ahpp_internal.cuh": "45194dba8b4be444"},
+        "bytes_per_unit": 2.519511e9,        # dram__bytes_read.sum + dram__bytes_write.sum per tile-round
+        "l2_to_sm_bytes_per_unit": 1.030348e10,   # l1tex__m_xbar2l1tex_read_bytes.sum per tile-round
+        "sources": {"ahpp_batch_kernel.cuh": "bd34f94bdf927170", "ahpp_batch.cu": "5d599f3b1a5f4330",
+                    "ahpp_batch.cuh": "17704647a89ad0c1", "ahpp_internal.cuh": "bc530504ac2f2a5a"},
     },
-    # the same capture's third k_query1 launch, one plain query (105 pull rounds):
+    # the same run's last k_query1 launch, one plain query (105 pull rounds):
     # profiles/k_query1_medium.md
     "k_query1": {
         "graph": "medium",
-        "bytes_per_unit": 5.008213e8,        # per pull round
-        "l2_to_sm_bytes_per_unit": 1.402732e9,
-        "sources": {"ahpp_query1.cu": "90fefeb4b00d7cd3", "ahpp_query1.cuh": "e356ae0e412d9385",
-                    "ahpp_internal.cuh": "45194dba8b4be444"},
+        "bytes_per_unit": 5.926105e8,        # per pull round
+        "l2_to_sm_bytes_per_unit": 1.723138e9,
+        "sources": {"ahpp_query1.cu": "8d0b8e1f1dded398", "ahpp_query1.cuh": "ed6f55b1b38c3694",
+                    "ahpp_rounds.cuh": "9fa43c7bd387b537", "ahpp_internal.cuh": "bc530504ac2f2a5a"},
     },
 }
 
@@ -697,7 +696,7 @@ def run_ours(args, rank, world, local_rank):
     achieved = alg / (sum(launch_ms) / K / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": ncu_traffic("k_tiles", args.graph, tile_rounds),
-            "traffic_note": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one 32-query tile "
+            "traffic_note": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of two 32-query tiles "
                              "per tile-round (profiles/k_tiles_medium_tile32.md), scaled by the launch's "
                              "tile-rounds"),
             "peak_source": peak_kind,

@@ -87,9 +87,10 @@ typedef struct {
     uint64_t hbm_budget_bytes; /* cap on the device memory of the graph's arrays (graph_bytes), a single
                                   query's state and a server's slots; 0 = no cap.  Not counted, so that
                                   they decide neither which graphs load nor how many slots there are:
-                                  the layouts built from the arrays for the pull rounds (about as much
-                                  again: ahpp_get_layout_info), and the further tiles that a batch of
-                                  several runs at once on a small graph (at most about 0.5 GB) */
+                                  the layouts built from the arrays for the pull rounds (1.6 times as
+                                  much again on large graphs, more on small ones:
+                                  ahpp_get_layout_info), and the further tiles that a batch of
+                                  several runs at once on a small graph (at most about 0.6 GB) */
     int device;                /* CUDA device ordinal (default 0) */
     uint32_t max_rounds;       /* round cap per query; 0: automatic */
     uint32_t batch_tile;       /* queries per batched tile: 16 or 32; 0: 32 (ahpp_autotune picks one);
@@ -370,8 +371,9 @@ int ahpp_selftest_arm_wait_timeout(ahpp_graph *g);
 /* Self-test of running out of device memory (nothing is really exhausted): of
  * the device allocations made for g from here on, the first `skip` go through
  * and the next one fails, once, as if memory had run out.  The call that made
- * it must report AHPP_ENOMEM and leave the graph as it was.  AHPP_EINVAL for a
- * NULL g. */
+ * it must report AHPP_ENOMEM and leave the graph as it was, or do without that
+ * memory (batches and servers, where it is for more tiles at once).
+ * AHPP_EINVAL for a NULL g. */
 int ahpp_selftest_arm_alloc_failure(ahpp_graph *g, uint32_t skip);
 
 #ifdef __cplusplus
